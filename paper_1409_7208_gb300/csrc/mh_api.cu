@@ -436,6 +436,8 @@ void mh_free_kmers(mh_kmers* s) {
     ctx_free(s->ctx, s->counts);
     ctx_free(s->ctx, s->spectrum);
     ctx_free(s->ctx, s->spectrum_len);
+    ctx_free(s->ctx, s->super_off);
+    ctx_free(s->ctx, s->super_idx);
     delete s;
 }
 

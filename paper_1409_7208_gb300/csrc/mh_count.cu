@@ -19,6 +19,9 @@
 //   units     each unit sorted and run-length counted on chip by one warp,
 //             the solid filter applied, both strands out (mh_group.cu)
 //   sort      the solid table by the key-value spread sort, ascending
+// From 2^22 windows on (k >= 20), the default plan counts by super-k-mers
+// instead (mh_super.cu); the unit counting takes the smaller sets and the
+// out-of-core buckets.
 // The spread route (a plan's alternative): passes over the top ceil(log2 n)
 // bits, a fix-up of keys sharing them, a run pass (runs_kernel: run heads
 // in a shared-memory bitmask, run lengths from the next head, the solid
@@ -31,6 +34,7 @@
 #include <vector>
 
 #include "mh_sort_kernels.cuh"
+#include "mh_super.cuh"
 
 namespace mh {
 
@@ -521,7 +525,7 @@ __global__ void __launch_bounds__(kRunThreads) runs_kernel(const uint64_t* __res
                                                            const uint64_t* __restrict__ spec,
                                                            const uint32_t* __restrict__ spec_len, uint64_t n_spec,
                                                            bool spec_mixed,
-                                                           const uint64_t* __restrict__ next_head,
+                                                           SuperIndex super, const uint64_t* __restrict__ next_head,
                                                            uint64_t* __restrict__ out_keys,
                                                            uint32_t* __restrict__ out_cnt, uint32_t slot,
                                                            uint32_t* __restrict__ tile_count,
@@ -620,8 +624,11 @@ __global__ void __launch_bounds__(kRunThreads) runs_kernel(const uint64_t* __res
 #pragma unroll
         for (int w = 0; w < NW; w++) x.w[w] = tk[rp(i) * NW + w];
         if constexpr (IN_MIXED) x = unmix_key<NW>(x);
-        const bool palin = key_eq<NW>(key_rc<NW>(x, K1), x);
-        const uint64_t len = spec ? spectrum_count<NW>(spec, spec_len, n_spec, x, spec_mixed, hint) : end - (start + i);
+        const Key<NW> xr = key_rc<NW>(x, K1);
+        const bool palin = key_eq<NW>(xr, x);
+        const uint64_t len = !spec       ? end - (start + i)
+                             : super.idx ? super_find<NW>(super, spec, spec_len, x, xr, mix_key<NW>(x), K1)
+                                         : spectrum_count<NW>(spec, spec_len, n_spec, x, spec_mixed, hint);
         if (run_keys) {
             // every run, in run order at the tile's own offset (mixed key, length)
 #pragma unroll
@@ -757,7 +764,7 @@ template <int NW>
 void expand_runs(mh_ctx* ctx, const uint64_t* sorted, uint64_t n, int k, int d, Buf<uint64_t>& out_keys,
                  Buf<uint32_t>& out_cnt, uint64_t* n_out, uint64_t* n_canon_runs, uint64_t* n_palin_runs,
                  const uint64_t* spectrum, const uint32_t* spectrum_len, uint64_t n_spectrum, bool in_mixed,
-                 bool spec_mixed, RunList* list) {
+                 bool spec_mixed, RunList* list, const SuperIndex* super) {
     if (list && spectrum) fail(MH_EUNSUPPORTED, "run lists are made while counting");
     const int K1 = k + 1;
     const uint64_t tiles = ceil_div(n ? n : 1, kRunTile);
@@ -786,7 +793,7 @@ void expand_runs(mh_ctx* ctx, const uint64_t* sorted, uint64_t n, int k, int d, 
         Buf<uint32_t> rcount(ctx, list ? tiles : 1);
         Buf<uint32_t> rlen(ctx, list ? tiles * (uint64_t)kRunTile : 1);
         MH_LAUNCH_B(ctx, "runs", n * 8 * NW, (unsigned)tiles, kRunThreads, smem, kern, sorted, n, K1, d, spectrum,
-                    spectrum_len, n_spectrum, spec_mixed, next.p, big_k.p, big_c.p, slot, tcount.p, tstats.p,
+                    spectrum_len, n_spectrum, spec_mixed, super ? *super : SuperIndex{}, next.p, big_k.p, big_c.p, slot, tcount.p, tstats.p,
                     list ? list->slot.p : nullptr, list ? rlen.p : nullptr, list ? rcount.p : nullptr,
                     ctx->d_status);
         if (list) {
@@ -837,13 +844,13 @@ void expand_runs(mh_ctx* ctx, const uint64_t* sorted, uint64_t n, int k, int d, 
 
 template void expand_runs<1>(mh_ctx*, const uint64_t*, uint64_t, int, int, Buf<uint64_t>&, Buf<uint32_t>&, uint64_t*,
                              uint64_t*, uint64_t*, const uint64_t*, const uint32_t*, uint64_t, bool, bool,
-                             RunList*);
+                             RunList*, const SuperIndex*);
 template void expand_runs<2>(mh_ctx*, const uint64_t*, uint64_t, int, int, Buf<uint64_t>&, Buf<uint32_t>&, uint64_t*,
                              uint64_t*, uint64_t*, const uint64_t*, const uint32_t*, uint64_t, bool, bool,
-                             RunList*);
+                             RunList*, const SuperIndex*);
 template void expand_runs<4>(mh_ctx*, const uint64_t*, uint64_t, int, int, Buf<uint64_t>&, Buf<uint32_t>&, uint64_t*,
                              uint64_t*, uint64_t*, const uint64_t*, const uint32_t*, uint64_t, bool, bool,
-                             RunList*);
+                             RunList*, const SuperIndex*);
 
 // Buckets of the mixed canonical keys to count one at a time (0 = all at
 // once).  Memory still free: the HBM budget, or without one 85% of the
@@ -943,6 +950,11 @@ void count_kmers(mh_ctx* ctx, const mh_reads* reads, int k, int d, mh_kmers* out
     out->n_kmers = 2 * n;
     out->spectrum_mixed = kMixed;
     const int bb = count_bucket_bits(ctx, n, NW);
+    if (bb == 0 && use_unit_count(ctx) && use_super(n, k + 1)) {
+        woff.reset();
+        super_count<NW>(ctx, reads, k, d, n, out);
+        return;
+    }
     const GroupPlan gp = group_plan(ctx, n, 0, NW);
     if (bb == 0 && use_unit_count(ctx) && gp.passes >= 0) {
         // 8-bit passes over the top bits, then the units sorted and counted

@@ -112,6 +112,13 @@ struct mh_kmers {
     uint32_t* spectrum_len = nullptr;  // n_spectrum
     uint64_t n_spectrum = 0;
     bool spectrum_mixed = false;
+    // a spectrum in super-k-mer bins instead of ascending (mh_super.cuh);
+    // super_idx set marks it
+    uint64_t* super_off = nullptr;
+    uint2* super_idx = nullptr;
+    uint32_t super_bins = 0;
+    int super_m = 0;
+    uint64_t super_main = 0;
     uint64_t n_kmers = 0, n_distinct = 0;
     mh_ctx* ctx = nullptr;
 };
@@ -759,14 +766,16 @@ void group_count(mh_ctx* ctx, Buf<uint64_t>& sorted, Buf<uint64_t>& other, uint6
                  uint64_t* n_runs, uint64_t* n_palin_runs, RunList* list);
 
 
+struct SuperIndex;
 // Sorted canonical keys -> solid (k+1)-mers, both strands, sorted.  Defined
 // in mh_count.cu, used by mercy too (d = 1, counts looked up in the
 // spectrum).  in_mixed: `sorted` holds mix_key images of the canonical keys;
 // spec_mixed: likewise for the spectrum.
+// super: the spectrum is in super-k-mer bins (mh_super.cuh).
 template <int NW>
 void expand_runs(mh_ctx* ctx, const uint64_t* sorted, uint64_t n, int k, int d, Buf<uint64_t>& out_keys,
                  Buf<uint32_t>& out_cnt, uint64_t* n_out, uint64_t* n_canon_runs, uint64_t* n_palin_runs,
                  const uint64_t* spectrum, const uint32_t* spectrum_len, uint64_t n_spectrum, bool in_mixed = false,
-                 bool spec_mixed = false, RunList* list = nullptr);
+                 bool spec_mixed = false, RunList* list = nullptr, const SuperIndex* super = nullptr);
 
 }  // namespace mh

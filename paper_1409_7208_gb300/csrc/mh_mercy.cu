@@ -30,7 +30,7 @@
 //            mixed spectrum: a hash set of the canonical solid keys.
 //   finish   sort + dedup of the candidates, counts looked up in the
 //            counting spectrum, both strands, sorted.
-#include "mh_internal.cuh"
+#include "mh_super.cuh"
 
 namespace mh {
 
@@ -420,19 +420,19 @@ __global__ void __launch_bounds__(256) mercy_probe_kernel(const uint32_t* __rest
 }
 
 // Walk from each hit to the next solid window; emit the gap if it qualifies.
-// MIXED: candidates out as mix_key images; 1-word keys then take solidity
-// from the counting spectrum (run length, doubled for a palindrome, >= d)
-// through its bucket index, wider keys (and unmixed handles) from the hash
-// set `solid`.
-template <int NW, bool MIXED>
+// SOL 1 and 2: candidates out as mix_key images, solidity from the counting
+// spectrum (run length, doubled for a palindrome, >= d) through its bucket
+// index (1) or its super-k-mer bins (2); SOL 0 (unmixed handles): from the
+// hash set `solid`.
+template <int NW, int SOL>
 __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restrict__ packed,
                                                          const ulonglong2* __restrict__ hits, uint64_t n_hits, int k,
                                                          const Slot<NW>* __restrict__ ends, uint64_t ends_mask,
                                                          const Slot<NW>* __restrict__ solid, uint64_t solid_mask,
                                                          const uint64_t* __restrict__ spec,
                                                          const uint32_t* __restrict__ spec_len,
-                                                         const uint64_t* __restrict__ spec_off, int spec_bits, int d,
-                                                         uint64_t* __restrict__ out, uint64_t out_cap,
+                                                         const uint64_t* __restrict__ spec_off, int spec_bits,
+                                                         SuperIndex super, int d, uint64_t* __restrict__ out, uint64_t out_cap,
                                                          unsigned long long* __restrict__ counter) {
     const int K1 = k + 1;
     for (uint64_t h = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; h < n_hits;
@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restr
             Key<NW> r = key_rc<NW>(x, K1);
             const Key<NW> c = key_less<NW>(r, x) ? r : x;
             bool present;
-            if constexpr (MIXED) {
-                const uint32_t len = spec_find<NW>(spec, spec_len, spec_off, spec_bits, mix_key<NW>(c));
+            if constexpr (SOL != 0) {
+                const uint32_t len = SOL == 2 ? super_find<NW>(super, spec, spec_len, x, r, mix_key<NW>(c), K1)
+                                              : spec_find<NW>(spec, spec_len, spec_off, spec_bits, mix_key<NW>(c));
                 present = (uint64_t)len * (key_eq<NW>(r, x) ? 2 : 1) >= (uint64_t)d;
             } else
                 present = table_has<NW>(solid, solid_mask, c);
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restr
             Key<NW> z = load_window<NW>(packed, j, K1);
             Key<NW> rz = key_rc<NW>(z, K1);
             Key<NW> c = key_less<NW>(rz, z) ? rz : z;
-            if constexpr (MIXED) c = mix_key<NW>(c);
+            if constexpr (SOL != 0) c = mix_key<NW>(c);
             store_key<NW>(out, idx, c);
         }
     }
@@ -515,7 +516,12 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     uint64_t scap = 1;
     Buf<uint64_t> spec_off;
     int spec_bits = 1;
-    if (mixed) {
+    const bool super = solid->super_idx != nullptr;
+    SuperIndex sx;
+    if (super) {
+        sx = SuperIndex{solid->super_off, solid->super_idx, solid->super_bins, solid->super_m, solid->super_main,
+                        solid->n_spectrum};
+    } else if (mixed) {
         while (spec_bits < 40 && (2ull << spec_bits) * 4 <= solid->n_spectrum) spec_bits++;
         spec_off = Buf<uint64_t>(ctx, (1ull << spec_bits) + 1);
         spec_off.zero();
@@ -556,9 +562,9 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
         MH_CUDA(cudaMemsetAsync(stats.p + 1, 0, sizeof(uint64_t), ctx->stream));
         if (n_hits)
             MH_LAUNCH(ctx, "mercy_walk", grid_for(ctx, n_hits, 256, 8), 256, 0,
-                      (mixed ? mercy_walk_kernel<NW, true> : mercy_walk_kernel<NW, false>), reads->packed,
+                      (super ? mercy_walk_kernel<NW, 2> : mixed ? mercy_walk_kernel<NW, 1> : mercy_walk_kernel<NW, 0>), reads->packed,
                       hits.p, n_hits, k, table.p, cap - 1, sset.p, scap - 1, solid->spectrum, solid->spectrum_len,
-                      spec_off.p, spec_bits, solid->d,
+                      spec_off.p, spec_bits, sx, solid->d,
                       cand.p, out_cap, (unsigned long long*)(stats.p + 1));
         read_u64(ctx, stats.p + 1, &n_cand, 1);
         if (n_cand <= out_cap) break;
@@ -576,7 +582,7 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     Buf<uint32_t> mc;
     uint64_t M = 0, runs = 0, palins = 0;
     expand_runs<NW>(ctx, sorted.p, n_cand, k, 1, mk, mc, &M, &runs, &palins, solid->spectrum, solid->spectrum_len,
-                    solid->n_spectrum, mixed, solid->spectrum_mixed);
+                    solid->n_spectrum, mixed, solid->spectrum_mixed, nullptr, super ? &sx : nullptr);
     sync_and_check(ctx);
     out->k = k;
     out->nw = NW;

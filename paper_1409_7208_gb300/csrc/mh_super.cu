@@ -1,0 +1,819 @@
+// Counting by super-k-mers: the count of mh_count_kmers (paper, Sec. 2,
+// third paragraph) for sets whose keys would otherwise be moved by radix
+// passes.
+//
+// Neighbouring windows of a read share all but one symbol, so moving a key a
+// window (8 to 32 bytes, several passes) moves each base some K1 times.  Here
+// a window goes to the bin of its minimizer, the smallest hash among its
+// canonical m-symbol words (Roberts et al., 2004, Bioinformatics 20:3363;
+// binning k-mers by them: Li et al., MSPKmerCounter, 2015, and KMC 2, Deorowicz et al., 2015).
+// A window and its reverse complement have the same canonical words, so equal
+// canonical keys meet in one bin; neighbours mostly share their minimizer, so
+// a run of them (a super-k-mer, 2 / (w + 1) a window for w words a window)
+// travels as one 8-byte record: where the run starts in the packed reads and
+// its number of windows.
+//
+//   split    tiles of 2,048 positions of the packed stream: the hashes of the
+//            tile's words, the smallest over each window, the runs; a run's
+//            record and its rank in its bin (one 64-bit atomic on the bin's
+//            counters: records low, windows high)
+//   place    after a scan of the counters, each record to its bin's place
+//   count    a CTA per bin: a warp takes 32 records at a time, a lane a
+//            window; its mixed canonical key goes into a hash table in
+//            shared memory; then the table's entries (the spectrum) and the
+//            kept keys of both strands are written at places reserved by
+//            one atomic each.  The kept keys are sorted afterwards, so the
+//            bins' order does not matter.
+//   rest     bins with more windows than one CTA should take, or whose keys
+//            do not fit the table, are expanded to keys and counted by the
+//            unit counting (mh_group.cu); their spectrum goes last
+//
+// What bounds it: instruction issue (a hash insertion a window) and the
+// waits at a bin's barriers, not memory: a window moves about 2 bytes of
+// records and 4 of outputs instead of 8 to 32 a pass.  3 Gbp, k = 31, 2.38 G
+// windows: split 6.6 ms (67 thread instructions a position), place 8.1, count
+// 25.1, where the extraction, two passes, the units and their compaction took
+// 18.8 + 28 + 22.3 + 5.2; 3 M reads of 100-150 bp at k = 61: 6.1 ms for 15.2.
+#include <algorithm>
+#include <cmath>
+#include <cstdlib>
+#include <vector>
+
+#include "mh_super.cuh"
+
+namespace mh {
+
+namespace {
+
+constexpr int kSplitTile = 2048;                      // positions a CTA
+constexpr int kSplitHalo = 128;                       // positions past it that its windows reach (w - 1 <= 112)
+constexpr int kSplitWords = kSplitTile / 16 + 12;     // packed words a CTA reads
+constexpr int kSplitMaxRecs = kSplitTile;
+constexpr int kHashPad = (kSplitTile + kSplitHalo) / 8 * 9;  // one word of padding after 8: no bank conflicts
+constexpr int kNwinBits = 12;                         // a record: start << 12 | windows (at most 2,048)
+static_assert(kSplitTile < (1 << kNwinBits), "a run fits a record");
+
+enum { T_SPEC = 0, T_SOLID = 1, T_PALIN = 2, T_DEF = 3, T_DEFWIN = 4, T_RECS = 5, T_N = 6 };
+
+}  // namespace
+
+// first[t] = first fragment f in [0, F] with offs[f] >= t * kSplitTile.
+__global__ void super_tiles_kernel(const uint64_t* __restrict__ offs, uint64_t F, uint64_t n_tiles,
+                                   uint64_t* __restrict__ first) {
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n_tiles;
+         t += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t q = t * kSplitTile;
+        uint64_t lo = 0, hi = F;
+        while (lo < hi) {
+            const uint64_t mid = lo + (hi - lo) / 2;
+            if (offs[mid] < q) lo = mid + 1; else hi = mid;
+        }
+        first[t] = lo;
+    }
+}
+
+template <int M>
+__global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __restrict__ packed, uint64_t n_words,
+                                                          const uint64_t* __restrict__ offs, uint64_t F,
+                                                          const uint64_t* __restrict__ first, int k, uint32_t n_bins,
+                                                          uint32_t most, unsigned long long* __restrict__ rec, uint2* __restrict__ place,
+                                                          uint64_t cap, unsigned long long* __restrict__ bins,
+                                                          unsigned long long* __restrict__ totals) {
+    constexpr int T = kSplitTile;
+    constexpr uint32_t mask = M == 16 ? 0xFFFFFFFFu : (1u << (2 * M)) - 1u;
+    __shared__ uint32_t words[kSplitWords];
+    __shared__ uint32_t hash[kHashPad];                // then the runs' minima
+    __shared__ uint32_t bmin[(T + kSplitHalo) / 8];
+    __shared__ uint32_t inv[T / 32], stop[T / 32];     // no window starts here; a run ends before here
+    __shared__ uint16_t hpos[kSplitMaxRecs];
+    __shared__ uint32_t edge[8], scratch[8];
+    __shared__ uint64_t out0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t base = (uint64_t)blockIdx.x * T;
+    const int w = k + 1 - M + 1;                       // words a window
+    for (int i = tid; i < kSplitWords; i += 256) {
+        const uint64_t g = base / 16 + i;
+        words[i] = g < n_words ? packed[g] : 0u;
+    }
+    if (tid < T / 32) inv[tid] = 0;
+    __syncthreads();
+    // no window starts in the k positions before a fragment's start (or the
+    // stream's end, offs[F])
+    for (uint64_t f = first[blockIdx.x] + tid; f <= F; f += 256) {
+        const uint64_t s64 = offs[f] - base;
+        if (s64 > (uint64_t)(T + k)) break;
+        // (past the stream's end there is none either)
+        const int s = (int)s64, lo = s > k ? s - k : 0, hi = (s < T && f < F) ? s : T;
+        for (int q = lo; q < hi;) {
+            const int e = min(hi, (q | 31) + 1);
+            const uint32_t m = (e - q == 32) ? 0xFFFFFFFFu : ((1u << (e - q)) - 1u) << (q & 31);
+            atomicOr(&inv[q >> 5], m);
+            q = e;
+        }
+    }
+    // hashes of 8 positions a thread, and their smallest
+    uint32_t h[8];
+    const int n_blk = 256 + (w + 6) / 8;
+    for (int blk = tid; blk < n_blk; blk += 256) {
+        const int wi = blk >> 1;
+        const uint64_t hi = ((uint64_t)words[wi] << 32) | words[wi + 1];
+        const uint64_t x = (blk & 1) ? (hi << 16) | (words[wi + 2] >> 16) : hi;  // 32 symbols
+        const uint64_t y = rev2_u64(~x);
+        uint32_t v[8], b = 0xFFFFFFFFu;
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const uint32_t f = (uint32_t)(x >> (64 - 2 * M - 2 * j)) & mask, g = (uint32_t)(y >> (2 * j)) & mask;
+            v[j] = super_hash(min(f, g));
+            hash[blk * 9 + j] = v[j];
+            b = min(b, v[j]);
+        }
+        bmin[blk] = b;
+        if (blk == tid) {
+#pragma unroll
+            for (int j = 0; j < 8; j++) h[j] = v[j];
+        }
+    }
+    __syncthreads();
+    // the smallest of each of the thread's 8 windows (w >= 8 positions each):
+    // its own positions from the window's start on, the positions all eight
+    // windows share (whole blocks by their minima), and the ones after
+    uint32_t mh[8];
+    {
+        uint32_t mid = 0xFFFFFFFFu;
+        const int nb = (w - 8) >> 3;
+        for (int q = 1; q <= nb; q++) mid = min(mid, bmin[tid + q]);
+        for (int p = 8 + 8 * nb; p < w; p++) mid = min(mid, hash[tid * 9 + p + (p >> 3)]);
+        mh[7] = h[7];
+#pragma unroll
+        for (int i = 6; i >= 0; i--) mh[i] = min(h[i], mh[i + 1]);
+        mh[0] = min(mh[0], mid);
+#pragma unroll
+        for (int i = 1; i < 8; i++) {
+            const int p = w - 1 + i;
+            mid = min(mid, hash[tid * 9 + p + (p >> 3)]);
+            mh[i] = min(mh[i], mid);
+        }
+    }
+    // heads: windows whose left neighbour is none or has another minimizer
+    if (lane == 31) edge[warp] = mh[7];
+    __syncthreads();
+    const uint32_t vb = ~(uint32_t)reinterpret_cast<const uint8_t*>(inv)[tid] & 0xFFu;
+    const bool pv = tid > 0 && !(reinterpret_cast<const uint8_t*>(inv)[tid - 1] >> 7);
+    uint32_t pm = __shfl_up_sync(0xFFFFFFFFu, mh[7], 1);
+    if (lane == 0 && warp > 0) pm = edge[warp - 1];
+    uint32_t same = (pv && pm == mh[0]) ? 1u : 0u;
+#pragma unroll
+    for (int i = 1; i < 8; i++) same |= (((vb >> (i - 1)) & 1u) && mh[i] == mh[i - 1]) ? 1u << i : 0u;
+    const uint32_t hm = vb & ~same;
+    reinterpret_cast<uint8_t*>(stop)[tid] = (uint8_t)(hm | ~vb);
+    uint32_t total;
+    uint32_t at = block_excl_scan_256(__popc(hm), scratch, &total);
+    if (tid == 0 && total) out0 = atomicAdd(&totals[T_RECS], (unsigned long long)total);
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        if ((hm >> i) & 1u) {
+            hpos[at] = (uint16_t)(tid * 8 + i);
+            hash[at] = mh[i];
+            at++;
+        }
+    __syncthreads();
+    // a thread per run
+    for (uint32_t j = tid; j < total; j += 256) {
+        const uint32_t q = hpos[j];
+        const uint32_t b = __umulhi(super_mix(hash[j]), n_bins);
+        // (a run of more windows than a record may have, in a repeat, gives
+        // several)
+        uint32_t left = next_bit(stop, q + 1, T) - q, at = 0;
+        uint64_t o = out0 + j;
+        while (true) {
+            const uint32_t nw = min(left, most);
+            const uint64_t r = atomicAdd(&bins[b], 1ull | ((unsigned long long)nw << 32));
+            if (o < cap) {
+                __stcs(&rec[o], (unsigned long long)(((base + q + at) << kNwinBits) | nw));
+                __stcs(&place[o], make_uint2(b, (uint32_t)r));
+            }
+            left -= nw;
+            if (!left) break;
+            at += nw;
+            o = atomicAdd(&totals[T_RECS], 1ull);
+        }
+    }
+}
+
+// Each record to its place in its bin (nothing if the records overflowed).
+__global__ void super_place_kernel(const unsigned long long* __restrict__ rec, const uint2* __restrict__ place, uint64_t cap,
+                                   const unsigned long long* __restrict__ totals, const uint64_t* __restrict__ off,
+                                   uint32_t b0, uint32_t b1, uint64_t* __restrict__ out) {
+    const uint64_t n = totals[T_RECS];
+    if (n > cap) return;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        // (each read once: not to displace the bins' open sectors in L2)
+        const uint2 p = __ldcs(&place[i]);
+        if (p.x - b0 < b1 - b0) out[(uint32_t)off[p.x] + (uint64_t)p.y] = __ldcs(&rec[i]);
+    }
+}
+
+// Two table slots, read again each time (other lanes fill them).
+__device__ __forceinline__ ulonglong2 ld_pair(const uint64_t* p) {
+    ulonglong2 v;
+    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];"
+                 : "=l"(v.x), "=l"(v.y)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p))
+                 : "memory");
+    return v;
+}
+
+// The windows of 32 records (a lane each; n windows in all), 32 at a time:
+// body(valid, position of this lane's window) for every step.
+template <class Body>
+__device__ __forceinline__ uint32_t for_windows(uint64_t rec, const Body& body) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t nw = (uint32_t)rec & ((1u << kNwinBits) - 1u);
+    uint32_t incl = nw;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const uint32_t start = incl - nw, tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    const uint64_t adj = (rec >> kNwinBits) - start;
+    uint32_t before = 0;
+    for (uint32_t j0 = 0; j0 < tot; j0 += 32) {
+        // the record of window j0 + lane: the last one that starts at or before it
+        const uint32_t rel = start - j0;
+        const uint32_t m = __reduce_or_sync(0xFFFFFFFFu, (nw && rel < 32u) ? 1u << rel : 0u);
+        const int idx = (int)(before + __popc(m & (0xFFFFFFFFu >> (31 - lane)))) - 1;
+        before += __popc(m);
+        const uint64_t p = __shfl_sync(0xFFFFFFFFu, adj, idx) + j0 + lane;
+        body(j0 + lane < tot, j0 + lane, p);
+    }
+    return tot;
+}
+
+// Shared memory of a bin's CTA: the table (top words, other words, counts),
+// its occupancy bits and the entries before each word of them, and the
+// records of a round (starts among the round's windows, symbols), over
+// which the list of occupied slots goes afterwards.  For one word 56 KB, so
+// that four CTAs share an SM.
+template <int NW>
+struct SuperSmem {
+    static constexpr int kSlots = SuperCfg<NW>::kSlots;
+    static constexpr int kRecs = NW == 1 ? 352 : 512 / NW;  // records a round
+    static constexpr int kRW = SuperCfg<NW>::kRecWords;    // words a record's symbols take
+    static constexpr int kMost = kSlots / 128 * 108;       // entries a table may hold (0.84 of its slots)
+    static constexpr size_t kFp = 0;
+    static constexpr size_t kLow = kFp + sizeof(uint64_t) * kSlots;
+    static constexpr size_t kCnt = kLow + sizeof(uint64_t) * (NW - 1) * kSlots;
+    static constexpr size_t kOcc = kCnt + sizeof(uint32_t) * kSlots;
+    static constexpr size_t kPre = kOcc + sizeof(uint32_t) * (kSlots / 32);
+    static constexpr size_t kSym = kPre + sizeof(uint16_t) * (kSlots / 32);
+    static constexpr size_t kStart = kSym + sizeof(uint32_t) * kRW * kRecs;
+    static constexpr size_t kRecEnd = kStart + sizeof(uint32_t) * kRecs;
+    static constexpr size_t kListEnd = kSym + sizeof(uint16_t) * kMost;
+    static constexpr size_t kBytes = kRecEnd > kListEnd ? kRecEnd : kListEnd;
+    static_assert(kSym % 16 == 0, "aligned");
+};
+
+// A CTA per bin.  The table's first word is a mixed key's top word (the whole
+// key of one word); kEmpty marks a free slot: the mixed image of the
+// all-ones key, which is not canonical, for one word (wider keys whose top
+// word equals it are left to the rest).  Wider keys' other words are
+// stored beside it by the lane that claimed the slot, which then sets the
+// count's top bit; a lane that finds its top word waits for that bit
+// (bounded) and compares the rest.  A key that finds no place within
+// probe_max slots leaves the bin to the rest, as do more than kMost entries.
+template <int NW>
+__global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
+    super_count_kernel(const uint32_t* __restrict__ packed, const uint64_t* __restrict__ rec,
+                       const uint64_t* __restrict__ off, uint32_t b0, uint32_t b1, uint64_t rec_cap, int K1, int d,
+                       uint32_t hot, int probe_max, uint64_t spec_cap, uint64_t* __restrict__ spec_k,
+                       uint32_t* __restrict__ spec_len, uint64_t solid_cap, uint64_t* __restrict__ solid_k,
+                       uint32_t* __restrict__ solid_c, uint64_t* __restrict__ soff, uint2* __restrict__ sidx,
+                       ulonglong2* __restrict__ deferred, unsigned long long* __restrict__ totals) {
+    using C = SuperCfg<NW>;
+    using L = SuperSmem<NW>;
+    constexpr uint64_t kEmpty = 0ull - kMixC1;
+    constexpr uint32_t kReady = 0x80000000u;
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t* fp = reinterpret_cast<uint64_t*>(smem + L::kFp);
+    uint64_t* low = reinterpret_cast<uint64_t*>(smem + L::kLow);
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + L::kCnt);
+    uint32_t* occ = reinterpret_cast<uint32_t*>(smem + L::kOcc);
+    uint16_t* pre = reinterpret_cast<uint16_t*>(smem + L::kPre);
+    uint32_t* sym = reinterpret_cast<uint32_t*>(smem + L::kSym);
+    uint32_t* start = reinterpret_cast<uint32_t*>(smem + L::kStart);
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem + L::kSym);
+    __shared__ uint32_t over, n_ent;
+    __shared__ uint32_t scratch[8], wsol[8];
+    __shared__ uint64_t base[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    if (totals[T_RECS] > rec_cap) return;
+    uint32_t palins = 0;
+
+    auto insert = [&](const Key<NW>& mk) {
+        const uint64_t t = mk.w[NW - 1];
+        if (NW > 1 && t == kEmpty) {
+            over = 1;
+            return;
+        }
+        uint32_t s = super_slot<NW>(mk);
+        for (int probe = 0; probe < probe_max; probe++) {
+            const ulonglong2 v = ld_pair(fp + s);
+            // the first of the pair that holds the key or nothing
+            uint32_t at = (v.x == t || v.x == kEmpty) ? s : s + 1;
+            uint64_t cur = at == s ? v.x : v.y;
+            if (cur == kEmpty) {
+                cur = atomicCAS((unsigned long long*)&fp[at], (unsigned long long)kEmpty, (unsigned long long)t);
+                if (cur == kEmpty) {
+                    if constexpr (NW > 1) {
+#pragma unroll
+                        for (int q = 0; q < NW - 1; q++) low[q * C::kSlots + at] = mk.w[q];
+                        __threadfence_block();
+                    }
+                    atomicAdd(&cnt[at], NW > 1 ? 1u | kReady : 1u);
+                    atomicOr(&occ[at >> 5], 1u << (at & 31));
+                    return;
+                }
+            }
+            if (cur == t) {
+                bool same = true;
+                if constexpr (NW > 1) {
+                    int spins = 0;
+                    while (!(*(volatile uint32_t*)&cnt[at] & kReady))
+                        if (++spins > 4096) {
+                            over = 1;
+                            return;
+                        }
+                    __threadfence_block();
+#pragma unroll
+                    for (int q = 0; q < NW - 1; q++) same &= *(volatile uint64_t*)&low[q * C::kSlots + at] == mk.w[q];
+                }
+                if (same) {
+                    atomicAdd(&cnt[at], 1u);
+                    return;
+                }
+                over = 1;  // two wide keys with the same top word
+                return;
+            }
+            // (a slot another lane has just taken: the pair again)
+            if (at != s && cur == v.y) s = (s + 2) & (C::kSlots - 1);
+        }
+        over = 1;
+    };
+
+    for (uint32_t b = b0 + blockIdx.x; b < b1; b += gridDim.x) {
+        const uint64_t o0 = off[b], o1 = off[b + 1];
+        const uint32_t r0 = (uint32_t)o0, r1 = (uint32_t)o1;
+        const uint32_t W = (uint32_t)(o1 >> 32) - (uint32_t)(o0 >> 32);
+        if (tid == 0) over = W > hot;
+        for (int i = tid; i < C::kSlots / 2; i += 256)
+            reinterpret_cast<ulonglong2*>(fp)[i] = make_ulonglong2(kEmpty, kEmpty);
+        for (int i = tid; i < C::kSlots / 4; i += 256) reinterpret_cast<uint4*>(cnt)[i] = make_uint4(0, 0, 0, 0);
+        if (tid < C::kWords) occ[tid] = 0;
+        // rounds of up to kRecs records: their windows are numbered through,
+        // an eighth of them to each warp, 32 at a time
+        for (uint32_t rb = r0; rb < r1; rb += L::kRecs) {
+            __syncthreads();
+            if (*(volatile uint32_t*)&over) break;
+            const uint32_t nr = min(r1 - rb, (uint32_t)L::kRecs);
+            constexpr int R = (L::kRecs + 255) / 256;  // records a thread
+            uint64_t rr[R];
+            uint32_t sum = 0;
+#pragma unroll
+            for (int q = 0; q < R; q++) {
+                rr[q] = (uint32_t)(R * tid + q) < nr ? rec[rb + R * tid + q] : 0ull;
+                sum += (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
+            }
+            uint32_t tot;
+            uint32_t ex = block_excl_scan_256(sum, scratch, &tot);
+#pragma unroll
+            for (int q = 0; q < R; q++) {
+                const uint32_t nw = (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
+                if (nw) {
+                    // the record's symbols from the packed reads, aligned to
+                    // a word: all of a thread's loads in flight at once
+                    const uint64_t p = rr[q] >> kNwinBits;
+                    const uint32_t* src = packed + (p >> 4);
+                    const uint32_t sh = 2 * (uint32_t)(p & 15), need = ((uint32_t)(p & 15) + nw + K1 - 1 + 15) / 16;
+                    uint32_t v[L::kRW + 1];
+#pragma unroll
+                    for (int i = 0; i <= L::kRW; i++) v[i] = (uint32_t)i < need ? src[i] : 0u;
+                    uint4* dst = reinterpret_cast<uint4*>(sym + (R * tid + q) * L::kRW);
+#pragma unroll
+                    for (int i = 0; i < L::kRW / 4; i++)
+                        dst[i] = make_uint4(__funnelshift_l(v[4 * i + 1], v[4 * i], sh), __funnelshift_l(v[4 * i + 2], v[4 * i + 1], sh),
+                                            __funnelshift_l(v[4 * i + 3], v[4 * i + 2], sh),
+                                            __funnelshift_l(v[4 * i + 4], v[4 * i + 3], sh));
+                    start[R * tid + q] = ex;
+                }
+                ex += nw;
+            }
+            __syncthreads();
+            const uint32_t per = (tot + 255) / 256 * 32;
+            uint32_t j0 = warp * per;
+            const uint32_t je = min(tot, j0 + per);
+            if (j0 >= je) continue;
+            // the last record that starts at or before window j0
+            uint32_t cur = 0;
+#pragma unroll
+            for (int step = 256; step; step >>= 1)
+                if (cur + step < nr && start[cur + step] <= j0) cur += step;
+            for (; j0 < je; j0 += 32) {
+                // the record of window j0 + lane: the records after cur that
+                // start among these windows, as bits
+                const uint32_t nx = cur + 1 + lane, rel = (nx < nr ? start[nx] : 0xFFFFFFFFu) - j0;
+                const uint32_t m = __reduce_or_sync(0xFFFFFFFFu, rel < 32u ? 1u << rel : 0u);
+                const uint32_t idx = cur + __popc(m & (0xFFFFFFFFu >> (31 - lane)));
+                cur += __popc(m);
+                if (j0 + lane < je) {
+                    // the window's 2 NW words (and one more) of its record
+                    const uint32_t at = j0 + lane - start[idx], sh = 2 * (at & 15);
+                    const uint32_t* src = sym + idx * L::kRW + (at >> 4);
+                    Key<NW> x;
+                    uint32_t hi = src[0];
+#pragma unroll
+                    for (int i = 0; i < NW; i++) {
+                        const uint32_t md = src[2 * i + 1], lo = src[2 * i + 2];
+                        x.w[NW - 1 - i] = ((uint64_t)__funnelshift_l(md, hi, sh) << 32) | __funnelshift_l(lo, md, sh);
+                        hi = lo;
+                    }
+                    x = key_shr<NW>(x, 64 * NW - 2 * K1);
+                    const Key<NW> rc = key_rc<NW>(x, K1);
+                    insert(mix_key<NW>(key_less<NW>(rc, x) ? rc : x));
+                }
+            }
+        }
+        __syncthreads();
+        // entries before each word of the occupancy bits (warp 0)
+        if (warp == 0) {
+            constexpr int per = C::kWords / 32;
+            uint32_t v[per], sum = 0;
+#pragma unroll
+            for (int q = 0; q < per; q++) {
+                v[q] = __popc(occ[lane * per + q]);
+                sum += v[q];
+            }
+            uint32_t x = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= o) x += y;
+            }
+            uint32_t e = x - sum;
+#pragma unroll
+            for (int q = 0; q < per; q++) {
+                pre[lane * per + q] = (uint16_t)e;
+                e += v[q];
+            }
+            if (lane == 31) n_ent = x;
+        }
+        __syncthreads();
+        const uint32_t ne = n_ent;
+        if (over || ne > (uint32_t)L::kMost) {
+            // to the rest; its place among the rest's keys
+            if (tid == 0) {
+                soff[b] = kSuperDeferred;
+                const uint64_t q = atomicAdd(&totals[T_DEF], 1ull);
+                deferred[q] = make_ulonglong2(b, atomicAdd(&totals[T_DEFWIN], (unsigned long long)W));
+            }
+            __syncthreads();
+            continue;
+        }
+        // the occupied slots listed in order
+        if (tid < C::kWords) {
+            uint32_t m = occ[tid], at = pre[tid];
+            sidx[(uint64_t)b * C::kWords + tid] = make_uint2(m, at);
+            while (m) {
+                list[at++] = (uint16_t)(tid * 32 + __ffs(m) - 1);
+                m &= m - 1;
+            }
+        }
+        __syncthreads();
+        auto key_at = [&](uint32_t s) {
+            Key<NW> m;
+            m.w[NW - 1] = fp[s];
+            if constexpr (NW > 1) {
+#pragma unroll
+                for (int q = 0; q < NW - 1; q++) m.w[q] = low[q * C::kSlots + s];
+            }
+            return m;
+        };
+        // kept keys: counted, a place reserved, then written with the entries
+        uint32_t no = 0;
+        for (uint32_t e0 = warp * 32; e0 < ne; e0 += 256) {
+            const uint32_t e = e0 + lane;
+            bool pl = false;
+            uint64_t lit = 0;
+            if (e < ne) {
+                const uint32_t s = list[e];
+                lit = cnt[s] & ~kReady;
+                if (!(K1 & 1)) {
+                    const Key<NW> x = unmix_key<NW>(key_at(s));
+                    pl = key_eq<NW>(key_rc<NW>(x, K1), x);
+                    if (pl) lit *= 2;
+                }
+            }
+            const uint32_t sm = __ballot_sync(0xFFFFFFFFu, e < ne && lit >= (uint64_t)d), pm = __ballot_sync(0xFFFFFFFFu, pl);
+            no += 2 * __popc(sm) - __popc(sm & pm);
+            palins += __popc(pm);
+        }
+        if (lane == 0) wsol[warp] = no;
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t c = 0;
+            for (int q = 0; q < 8; q++) c += wsol[q];
+            base[0] = atomicAdd(&totals[T_SPEC], (unsigned long long)ne);
+            base[1] = atomicAdd(&totals[T_SOLID], (unsigned long long)c);
+            soff[b] = base[0];
+        }
+        __syncthreads();
+        uint32_t po = 0, to = 0;
+        for (int q = 0; q < 8; q++) {
+            po += q < warp ? wsol[q] : 0u;
+            to += wsol[q];
+        }
+        // (past a buffer's end nothing is written: the host sees the totals)
+        if (base[0] + ne <= spec_cap && base[1] + to <= solid_cap) {
+            uint64_t so = base[1] + po;
+            for (uint32_t e0 = warp * 32; e0 < ne; e0 += 256) {
+                const uint32_t e = e0 + lane;
+                bool pl = false;
+                uint32_t lit = 0;
+                Key<NW> x{}, r{};
+                if (e < ne) {
+                    const uint32_t s = list[e];
+                    const Key<NW> m = key_at(s);
+                    lit = cnt[s] & ~kReady;
+                    store_key<NW>(spec_k, base[0] + e, m);
+                    spec_len[base[0] + e] = lit;
+                    x = unmix_key<NW>(m);
+                    r = key_rc<NW>(x, K1);
+                    pl = key_eq<NW>(r, x);
+                    if (pl) lit *= 2;
+                }
+                const bool keep = e < ne && lit >= (uint32_t)d;
+                const uint32_t sm = __ballot_sync(0xFFFFFFFFu, keep), pm = __ballot_sync(0xFFFFFFFFu, pl);
+                if (keep) {
+                    const uint64_t at = so + 2 * __popc(sm & lt) - __popc(sm & pm & lt);
+                    store_key<NW>(solid_k, at, x);
+                    solid_c[at] = lit;
+                    if (!pl) {
+                        store_key<NW>(solid_k, at + 1, r);
+                        solid_c[at + 1] = lit;
+                    }
+                }
+                so += 2 * __popc(sm) - __popc(sm & pm);
+            }
+        }
+        __syncthreads();
+    }
+    if (lane == 0 && palins) atomicAdd(&totals[T_PALIN], (unsigned long long)palins);
+}
+
+// The mixed canonical keys of the deferred bins, bin q's from its place on,
+// in no fixed order (a warp reserves its windows' places on the bin's cursor).
+template <int NW>
+__global__ void __launch_bounds__(256) super_expand_kernel(const uint32_t* __restrict__ packed,
+                                                           const uint64_t* __restrict__ rec,
+                                                           const uint64_t* __restrict__ off,
+                                                           const ulonglong2* __restrict__ deferred, uint64_t n_def,
+                                                           int K1, unsigned long long* __restrict__ cursor,
+                                                           uint64_t* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t wy = blockIdx.y * 8 + (threadIdx.x >> 5), ny = gridDim.y * 8;
+    for (uint64_t q = blockIdx.x; q < n_def; q += gridDim.x) {
+        const uint64_t b = deferred[q].x;
+        const uint32_t r0 = (uint32_t)off[b], r1 = (uint32_t)off[b + 1];
+        for (uint64_t rb = r0 + (uint64_t)wy * 32; rb < r1; rb += (uint64_t)ny * 32) {
+            const uint64_t r = rb + lane < r1 ? rec[rb + lane] : 0ull;
+            const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)r & ((1u << kNwinBits) - 1u));
+            uint64_t at = 0;
+            if (lane == 0) at = deferred[q].y + atomicAdd(&cursor[q], (unsigned long long)tot);
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+            for_windows(r, [&](bool valid, uint32_t j, uint64_t p) {
+                if (!valid) return;
+                const Key<NW> x = load_window<NW>(packed, p, K1);
+                const Key<NW> rc = key_rc<NW>(x, K1);
+                store_key<NW>(out, at + j, mix_key<NW>(key_less<NW>(rc, x) ? rc : x));
+            });
+        }
+    }
+}
+
+// ------------------------------------------------------------------- host
+
+static long env_long(const char* name, long dflt) {
+    const char* e = std::getenv(name);
+    return e ? std::strtol(e, nullptr, 10) : dflt;
+}
+
+// From 2^22 windows on; below, the unit route's few launches cost as much as
+// these.  MH_SUPER=0 turns the route off, =1 on at any size (tests).  The
+// counters of a bin hold 32 bits each, so fewer than 2^32 windows.
+bool use_super(uint64_t n, int K1) {
+    static const long v = env_long("MH_SUPER", -1);
+    if (v == 0 || !n || n >= (1ull << 32) || super_m(K1) == 0) return false;
+    return v == 1 || n >= (1ull << 22);
+}
+
+template <int NW>
+void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, mh_kmers* out) {
+    using C = SuperCfg<NW>;
+    const int K1 = k + 1, m = super_m(K1), w = K1 - m + 1;
+    // tests: bins of more windows than MH_SUPER_HOT, or with a key that finds
+    // no place in MH_SUPER_PROBES slots, are left to the rest
+    static const uint32_t hot = (uint32_t)std::max(0l, env_long("MH_SUPER_HOT", 1 << 16));
+    static const int probes = (int)std::max(1l, std::min(256l, env_long("MH_SUPER_PROBES", 128)));
+    const uint64_t F = reads->n_frags, n_words = ceil_div(reads->n_packed, 16) + kPackPad;
+    const uint64_t n_tiles = ceil_div(reads->n_packed, (uint64_t)kSplitTile);
+    const uint32_t n_bins = (uint32_t)std::max<uint64_t>(1, n / C::kTarget);
+    Buf<uint64_t> first(ctx, n_tiles), off(ctx, (uint64_t)n_bins + 1), totals(ctx, 8);
+    Buf<unsigned long long> bins(ctx, n_bins);
+    MH_LAUNCH(ctx, "super_tiles", grid_for(ctx, n_tiles, 256), 256, 0, super_tiles_kernel, reads->frag_offs, F,
+              n_tiles, first.p);
+    // records: 2 / (w + 1) a window for random sequences, one more a fragment
+    // and a tile; if there are more, again with room for what there is
+    uint64_t cap = (uint64_t)(2.5 / (w + 1) * (double)n) + F + n_tiles + 4096;
+    cap = std::min(cap, n);
+    unsigned long long* tot = reinterpret_cast<unsigned long long*>(totals.p);
+    Buf<uint64_t> rec;
+    uint64_t h[8] = {0};
+    Buf<uint64_t> spec, solid, soff(ctx, n_bins);
+    Buf<uint32_t> spec_len, solid_c;
+    Buf<uint2> sidx(ctx, (uint64_t)n_bins * C::kWords);
+    Buf<ulonglong2> deferred(ctx, n_bins);
+    uint64_t spec_cap = 0, solid_cap = 0;
+    const uint64_t per = d >= 2 ? 1 : 2;  // kept keys of both strands a window, at most
+    constexpr size_t smem = SuperSmem<NW>::kBytes;
+    MH_CUDA(cudaFuncSetAttribute(super_count_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    MH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, super_count_kernel<NW>, 256, smem));
+    auto count = [&](uint32_t b0, uint32_t b1) {
+        if (b0 < b1)
+            MH_LAUNCH_B(ctx, "super_count", n / 4, (unsigned)std::min<uint64_t>(b1 - b0, (uint64_t)ctx->num_sms * std::max(1, per_sm)),
+                        256, smem, super_count_kernel<NW>, reads->packed, rec.p, off.p, b0, b1, cap, K1, d, hot,
+                        probes, spec_cap, spec.p, spec_len.p, solid_cap, solid.p, solid_c.p, soff.p, sidx.p,
+                        deferred.p, tot);
+    };
+    auto room = [&](uint64_t a, uint64_t s) {
+        spec_cap = a;
+        solid_cap = s;
+        spec = Buf<uint64_t>(ctx, a * NW);
+        spec_len = Buf<uint32_t>(ctx, a);
+        solid = Buf<uint64_t>(ctx, s * NW);
+        solid_c = Buf<uint32_t>(ctx, s);
+    };
+    // large sets: a sixteenth of the bins first, to size the outputs by
+    const bool sample = n >= (1ull << 25) && n_bins >= 4096;
+    const uint32_t nb1 = sample ? n_bins / 16 : n_bins;
+    for (int attempt = 0;; attempt++) {
+        rec.reset();
+        rec = Buf<uint64_t>(ctx, cap);
+        {
+            Buf<unsigned long long> raw(ctx, cap);
+            Buf<uint2> place(ctx, cap);
+            bins.zero();
+            totals.zero();
+            const auto split = m == 16 ? super_split_kernel<16> : m == 14 ? super_split_kernel<14> : super_split_kernel<12>;
+            MH_LAUNCH_B(ctx, "super_split", reads->n_packed / 4, (unsigned)n_tiles, 256, 0, split, reads->packed, n_words,
+                        reads->frag_offs, F, first.p, k, n_bins, (uint32_t)(32 * C::kRecWords / 2 - K1 + 1), raw.p, place.p, cap, bins.p, tot);
+            exclusive_scan_u64(ctx, reinterpret_cast<const uint64_t*>(bins.p), off.p, n_bins);
+            // in ranges of bins whose open sectors (32 bytes a bin) and
+            // offsets stay in L2 beside the streams (3 Gbp, 850,000 bins:
+            // 10.6 ms in one range, 8.1 in four, 8.5 in eight)
+            const int G = (int)std::max<uint64_t>(1, std::min<uint64_t>(8, ceil_div(n_bins, 220000)));
+            for (int g = 0; g < G; g++)
+                MH_LAUNCH(ctx, "super_place", grid_for(ctx, cap, 256), 256, 0, super_place_kernel, raw.p, place.p, cap, tot,
+                          off.p, (uint32_t)((uint64_t)n_bins * g / G), (uint32_t)((uint64_t)n_bins * (g + 1) / G), rec.p);
+        }
+        uint64_t n1 = n;
+        if (sample) {
+            read_u64(ctx, off.p + nb1, &n1, 1);
+            n1 >>= 32;
+        }
+        room(std::max<uint64_t>(n1, 1), std::max<uint64_t>(n1 * per, 1));
+        count(0, nb1);
+        read_u64(ctx, totals.p, h, T_N);
+        if (h[T_RECS] <= cap) break;
+        if (attempt) fail(MH_EDEVICE, "super-k-mer records overflow twice");
+        cap = h[T_RECS];
+    }
+    if (sample) {
+        // the other bins into buffers sized by the first ones (bins are by
+        // hash: alike but for chance and the heavy ones), then the first
+        // ones' entries in front of them
+        Buf<uint64_t> k1 = std::move(spec), s1 = std::move(solid);
+        Buf<uint32_t> l1 = std::move(spec_len), c1 = std::move(solid_c);
+        const uint64_t a1 = h[T_SPEC], o1 = h[T_SOLID];
+        const double f = (double)n_bins / nb1;
+        uint64_t a = std::min<uint64_t>(n, (uint64_t)(1.04 * f * (double)a1) + (1u << 20));
+        uint64_t s = std::min<uint64_t>(n * per, (uint64_t)(1.04 * f * (double)o1) + (1u << 20));
+        const std::vector<uint64_t> h1(h, h + T_N);
+        for (int attempt = 0;; attempt++) {
+            room(a, s);
+            if (a1) {
+                MH_CUDA(cudaMemcpyAsync(spec.p, k1.p, a1 * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+                MH_CUDA(cudaMemcpyAsync(spec_len.p, l1.p, a1 * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+            }
+            if (o1) {
+                MH_CUDA(cudaMemcpyAsync(solid.p, s1.p, o1 * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+                MH_CUDA(cudaMemcpyAsync(solid_c.p, c1.p, o1 * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+            }
+            count(nb1, n_bins);
+            read_u64(ctx, totals.p, h, T_N);
+            if (h[T_SPEC] <= a && h[T_SOLID] <= s) break;
+            if (attempt) fail(MH_EDEVICE, "super-k-mer outputs overflow twice");
+            a = h[T_SPEC];
+            s = h[T_SOLID];
+            MH_CUDA(cudaMemcpyAsync(totals.p, h1.data(), sizeof(uint64_t) * T_N, cudaMemcpyHostToDevice, ctx->stream));
+            sync_and_check(ctx);
+        }
+    }
+    uint64_t R = h[T_SPEC], S = h[T_SOLID], runs = R, palins = h[T_PALIN];
+    const uint64_t n_main = R;
+    // the deferred bins, by the unit counting
+    RunList rest;
+    Buf<uint64_t> rest_k;
+    Buf<uint32_t> rest_c;
+    uint64_t rest_S = 0;
+    if (h[T_DEF]) {
+        const uint64_t nd = h[T_DEFWIN];
+        Buf<uint64_t> keys(ctx, nd * NW), alt(ctx, nd * NW);
+        Buf<unsigned long long> cursor(ctx, h[T_DEF]);
+        cursor.zero();
+        const unsigned gx = (unsigned)std::min<uint64_t>(h[T_DEF], 4096);
+        const unsigned gy = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(64, (uint64_t)ctx->num_sms * 8 / gx));
+        MH_LAUNCH(ctx, "super_expand", dim3(gx, gy), 256, 0, super_expand_kernel<NW>, reads->packed, rec.p, off.p,
+                  deferred.p, h[T_DEF], K1, cursor.p, keys.p);
+        rec.reset();
+        const GroupPlan gp = group_plan(ctx, nd, 0, NW);
+        if (gp.passes < 0) fail(MH_EDEVICE, "super-k-mer counting: no unit plan for the deferred bins");
+        const bool in_alt = gp.passes ? radix_sort<NW>(ctx, keys.p, alt.p, nullptr, nullptr, nd, 64 * NW - 8 * gp.passes, 64 * NW)
+                                      : false;
+        uint64_t r2 = 0, p2 = 0;
+        group_count<NW>(ctx, in_alt ? alt : keys, in_alt ? keys : alt, nd, k, d, 0, gp, rest_k, rest_c, &rest_S, &r2, &p2,
+                        &rest);
+        runs += r2;
+        palins += p2;
+        R += rest.n;
+        S += rest_S;
+    }
+    rec.reset();
+    first.reset();
+    off.reset();
+    bins.reset();
+    deferred.reset();
+    // the outputs' buffers grow by the rest, or shrink if much too large
+    auto fit = [&](Buf<uint64_t>& kb, Buf<uint32_t>& cb, uint64_t have, uint64_t have_cap, const Buf<uint64_t>& rk,
+                   const Buf<uint32_t>& rcnt, uint64_t more) {
+        const uint64_t need = have + more;
+        if (need > have_cap || have_cap > need + need / 4 + 4096) {
+            Buf<uint64_t> k2(ctx, (need ? need : 1) * NW);
+            Buf<uint32_t> c2(ctx, need ? need : 1);
+            if (have) {
+                MH_CUDA(cudaMemcpyAsync(k2.p, kb.p, have * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+                MH_CUDA(cudaMemcpyAsync(c2.p, cb.p, have * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+            }
+            kb = std::move(k2);
+            cb = std::move(c2);
+        }
+        if (more) {
+            MH_CUDA(cudaMemcpyAsync(kb.p + have * NW, rk.p, more * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+            MH_CUDA(cudaMemcpyAsync(cb.p + have, rcnt.p, more * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+        }
+    };
+    fit(spec, spec_len, n_main, spec_cap, rest.keys, rest.lens, rest.n);
+    fit(solid, solid_c, h[T_SOLID], solid_cap, rest_k, rest_c, rest_S);
+    rest.keys.reset();
+    rest.lens.reset();
+    rest_k.reset();
+    rest_c.reset();
+    {
+        Buf<uint64_t> alt(ctx, (S ? S : 1) * NW);
+        Buf<uint32_t> calt(ctx, S ? S : 1);
+        if (radix_sort_spread_kv<NW>(ctx, solid.p, alt.p, solid_c.p, calt.p, S, 64 * NW - 2 * K1)) {
+            std::swap(solid, alt);
+            std::swap(solid_c, calt);
+        }
+    }
+    sync_and_check(ctx);
+    out->n = S;
+    out->n_distinct = 2 * runs - palins;
+    out->keys = solid.release();
+    out->counts = solid_c.release();
+    out->n_spectrum = R;
+    out->spectrum = spec.release();
+    out->spectrum_len = spec_len.release();
+    out->super_off = soff.release();
+    out->super_idx = sidx.release();
+    out->super_bins = n_bins;
+    out->super_m = m;
+    out->super_main = n_main;
+}
+
+template void super_count<1>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
+template void super_count<2>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
+template void super_count<4>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
+
+}  // namespace mh
