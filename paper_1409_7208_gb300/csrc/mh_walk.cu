@@ -22,7 +22,17 @@
 // load and a ballot gives the first entry >= node.A, so a step costs a few
 // dependent loads.  Walks write into fixed slots of max_len bytes, compacted
 // afterwards.
+//
+// Long walks take links made beforehand instead (use_links): for every edge
+// where its out-edges lie in both tables (a join of suffixes against
+// prefixes, through the same index), and, by doubling, where 4 and 16 steps
+// lead while every node on the way has one out-edge, with their symbols.  A
+// walk is then a thread that loads its edge's link and both jumps at once and
+// takes the longest that holds: one memory latency for up to 16 symbols
+// instead of one for each.  (A node with one out-edge needs no random value,
+// so jumps skip none that counts.)
 #include <algorithm>
+#include <cstdlib>
 
 #include "mh_internal.cuh"
 
@@ -169,6 +179,146 @@ __global__ void walk_kernel(const uint64_t* __restrict__ S, uint64_t nS, const u
     }
 }
 
+// Where an edge leads: the first of its out-edges in the solid table (x) and
+// in the mercy table (y), and their labels (z: bits 0-3 solid, 4-7 mercy).
+// A jump: the edge reached (x, kNoJump if some node on the way has not
+// exactly one out-edge) and the symbols appended (y, the last one lowest).
+constexpr uint32_t kNoJump = 0xFFFFFFFFu;
+
+// First entry of the table at or after q, within q's bucket.
+template <int NW>
+__device__ __forceinline__ uint64_t bucket_lb(const uint64_t* __restrict__ T, const uint64_t* __restrict__ off,
+                                              const Key<NW>& q, int K1, int bits) {
+    const uint64_t b = top_bits<NW>(q, K1, bits);
+    uint64_t lo = off[b], hi = off[b + 1];
+    while (lo < hi) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (key_less<NW>(load_key<NW>(T, mid), q)) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Links and one-step jumps of the edges T[0, n), numbered from `first`
+// (thread per edge: neighbours' suffixes ascend, so neighbouring threads
+// search the same buckets).
+template <int NW>
+__global__ void __launch_bounds__(256) walk_links_kernel(const uint64_t* __restrict__ T, uint64_t n, uint64_t first,
+                                                         const uint64_t* __restrict__ S, uint64_t nS,
+                                                         const uint64_t* __restrict__ offS,
+                                                         const uint64_t* __restrict__ M, uint64_t nM,
+                                                         const uint64_t* __restrict__ offM, int bits, int k,
+                                                         uint4* __restrict__ link, uint2* __restrict__ jump) {
+    const int K1 = k + 1;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        const Key<NW> v = key_low<NW>(load_key<NW>(T, i), 2 * k), q = key_shl<NW>(v, 2);
+        uint4 l = make_uint4(0, 0, 0, 0);
+        auto find = [&](const uint64_t* __restrict__ A, uint64_t nA, const uint64_t* __restrict__ off, uint32_t& at) {
+            uint32_t mask = 0;
+            if (!nA) return mask;
+            uint64_t p = bucket_lb<NW>(A, off, q, K1, bits);
+            at = (uint32_t)p;
+            for (int t = 0; t < 4 && p < nA; t++, p++) {
+                const Key<NW> e = load_key<NW>(A, p);
+                if (!key_eq<NW>(key_shr<NW>(e, 2), v)) break;
+                mask |= 1u << (e.w[0] & 3u);
+            }
+            return mask;
+        };
+        const uint32_t ms = find(S, nS, offS, l.x), mm = find(M, nM, offM, l.y);
+        l.z = ms | (mm << 4);
+        link[first + i] = l;
+        const uint32_t m = ms | mm;
+        uint2 j = make_uint2(kNoJump, 0);
+        if (__popc(m) == 1) j = make_uint2(ms ? l.x : (uint32_t)nS + l.y, __ffs(m) - 1);
+        jump[first + i] = j;
+    }
+}
+
+// Jumps of twice the steps from jumps of `steps` steps.
+__global__ void __launch_bounds__(256) walk_double_kernel(const uint2* __restrict__ in, uint64_t n, int steps,
+                                                          uint2* __restrict__ out) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        uint2 a = in[i];
+        if (a.x != kNoJump) {
+            const uint2 b = in[a.x];
+            a = make_uint2(b.x, (a.y << (2 * steps)) | b.y);
+        }
+        out[i] = a;
+    }
+}
+
+// A thread per walk, symbols packed 16 a word (first symbol highest) into
+// its slot of `stride` words.  Bound by the latency of the three loads of a
+// step (a few threads an SM): 16,384 walks of up to 10,000 symbols over 25 M
+// edges 0.5 ms, 26.6 ms by a search a symbol.
+template <int NW>
+__global__ void __launch_bounds__(64) walk_linked_kernel(const uint64_t* __restrict__ S, uint64_t nS,
+                                                         const uint64_t* __restrict__ M, uint64_t nM,
+                                                         const uint4* __restrict__ link,
+                                                         const uint2* __restrict__ jump4,
+                                                         const uint2* __restrict__ jump16, int k, uint64_t n_walks,
+                                                         uint32_t max_len, uint64_t seed, uint64_t stride,
+                                                         uint32_t* __restrict__ slots, uint64_t* __restrict__ lens) {
+    const int K1 = k + 1;
+    const uint64_t E = nS + nM;
+    const uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (w >= n_walks) return;
+    uint32_t* out = slots + w * stride;
+    uint64_t acc = 0;   // symbols not written yet, the last one lowest
+    int pending = 0;
+    auto append = [&](uint32_t syms, int n) {
+        acc = (acc << (2 * n)) | syms;
+        pending += n;
+        if (pending >= 16) {
+            pending -= 16;
+            *out++ = (uint32_t)(acc >> (2 * pending));
+        }
+    };
+    const uint64_t s = splitmix64_at(seed, w << 24) % E;
+    const Key<NW> x = s < nS ? load_key<NW>(S, s) : load_key<NW>(M, s - nS);
+    for (int i = 0; i < K1; i++) append(key_sym<NW>(x, K1, i), 1);
+    uint32_t cur = (uint32_t)s, len = K1;
+    while (len < max_len) {
+        const uint2 a = jump16[cur], b = jump4[cur];
+        const uint4 l = link[cur];
+        if (a.x != kNoJump && len + 16 <= max_len) {
+            append(a.y, 16);
+            cur = a.x;
+            len += 16;
+        } else if (b.x != kNoJump && len + 4 <= max_len) {
+            append(b.y, 4);
+            cur = b.x;
+            len += 4;
+        } else {
+            const uint32_t ms = l.z & 15u, mm = l.z >> 4, mask = ms | mm;
+            if (!mask) break;
+            uint32_t m = mask;
+            const uint32_t n = __popc(mask);
+            if (n > 1) {
+                // step j appends symbol K1 + j - 1
+                uint32_t r = (uint32_t)(splitmix64_at(seed, (w << 24) + (len - K1 + 1)) % (uint64_t)n);
+                while (r--) m &= m - 1;
+            }
+            const uint32_t c = __ffs(m) - 1, below = (1u << c) - 1u;
+            cur = (ms >> c) & 1u ? l.x + __popc(ms & below) : (uint32_t)nS + l.y + __popc(mm & below);
+            append(c, 1);
+            len++;
+        }
+    }
+    if (pending) *out = (uint32_t)(acc << (2 * (16 - pending)));
+    lens[w] = len;
+}
+
+// contig w: lens[w] symbols of its slot as letters at off[w] (block per contig)
+__global__ void contig_unpack_kernel(const uint32_t* __restrict__ slots, uint64_t stride,
+                                     const uint64_t* __restrict__ off, uint8_t* __restrict__ ascii) {
+    const uint64_t w = blockIdx.x;
+    const uint64_t o = off[w], len = off[w + 1] - o;
+    const uint32_t* s = slots + w * stride;
+    for (uint64_t i = threadIdx.x; i < len; i += blockDim.x)
+        ascii[o + i] = "ACGT"[(s[i >> 4] >> (30 - 2 * (uint32_t)(i & 15))) & 3u];
+}
+
 // contig w: lens[w] bytes from its slot to off[w]
 __global__ void contig_compact_kernel(const uint8_t* __restrict__ slots, uint32_t max_len,
                                       const uint64_t* __restrict__ off, uint8_t* __restrict__ ascii) {
@@ -177,38 +327,103 @@ __global__ void contig_compact_kernel(const uint8_t* __restrict__ slots, uint32_
     for (uint64_t i = threadIdx.x; i < len; i += blockDim.x) ascii[o + i] = slots[w * max_len + i];
 }
 
+// Whether n_walks walks of up to max_len symbols over E edges take links.
+// A step by search costs about 2.7 us of dependent loads whatever E is (26.6
+// ms for 10,000 steps, 16,384 walks at once); links and jumps cost about 54
+// us a million edges (1.3 ms for 25 M edges) and the walks by them 0.5 ms.
+// They even out near E = 49,000 max_len; the line is drawn at 20,000, since
+// doubling over arrays far beyond L2 costs more an edge.
+// MH_WALK_LINKS=0 / 1 decides it for tests.
+static bool use_links(const mh_ctx* ctx, uint64_t E, uint64_t n_walks, uint64_t max_len) {
+    static const int v = [] {
+        const char* e = std::getenv("MH_WALK_LINKS");
+        return e ? std::atoi(e) : -1;
+    }();
+    if (v == 0 || E >= kNoJump) return false;
+    if (v != 1) {
+        const uint64_t rounds = ceil_div(n_walks, (uint64_t)ctx->num_sms * 64);
+        if (E > 20000 * max_len * rounds) return false;
+    }
+    // 40 bytes an edge: within a budget that has room for it
+    return !ctx->budget || ctx->in_use + 40 * E + n_walks * (max_len / 4 + 64) < ctx->budget;
+}
+
 template <int NW>
 void walk_contigs(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, uint64_t n_walks, uint32_t max_len,
                   uint64_t seed, mh_contigs* out) {
     const int k = solid->k;
-    const uint64_t nS = solid->n, nM = mercy ? mercy->n : 0;
-    if (nS + nM == 0) n_walks = 0;
-    Buf<uint8_t> slots(ctx, n_walks * max_len);
+    const uint64_t nS = solid->n, nM = mercy ? mercy->n : 0, E = nS + nM;
+    const uint64_t* mk = mercy ? mercy->keys : nullptr;
+    if (E == 0) n_walks = 0;
+    bool linked = n_walks && use_links(ctx, E, n_walks, max_len);
+    Buf<uint4> link;
+    Buf<uint2> a, b, c;
+    if (linked) {
+        try {
+            link = Buf<uint4>(ctx, E);
+            a = Buf<uint2>(ctx, E);
+            b = Buf<uint2>(ctx, E);
+            c = Buf<uint2>(ctx, E);
+        } catch (const Error& e) {
+            // no room for them: the walks need none
+            if (e.code != MH_ENOMEM) throw;
+            link.reset();
+            a.reset();
+            b.reset();
+            linked = false;
+        }
+    }
+    const uint64_t stride = linked ? ceil_div(max_len, 16) : max_len;  // of a walk's slot, in words or bytes
+    Buf<uint8_t> slots(ctx, n_walks * stride * (linked ? 4 : 1));
     Buf<uint64_t> lens(ctx, n_walks + 1), off(ctx, n_walks + 1);
-    // bucket indexes over the top bits: about 16 entries a bucket
+    // bucket indexes over the top bits: about 16 entries a bucket (a thread
+    // searching for links: 4)
+    const uint64_t per = linked ? 4 : 16;
     int bits = 1;
-    while (bits < 32 && bits < 2 * (k + 1) && (2ull << bits) * 16 <= std::max(nS, nM)) bits++;
-    Buf<uint64_t> offS(ctx, (1ull << bits) + 1), offM(ctx, (1ull << bits) + 1);
-    offS.zero();
-    offM.zero();
+    while (bits < 32 && bits < 2 * (k + 1) && (2ull << bits) * per <= std::max(nS, nM)) bits++;
     if (n_walks) {
+        Buf<uint64_t> offS(ctx, (1ull << bits) + 1), offM(ctx, (1ull << bits) + 1);
         if (nS)
             MH_LAUNCH(ctx, "walk_index", grid_for(ctx, nS, 256), 256, 0, table_index_kernel<NW>, solid->keys, nS,
                       k + 1, bits, offS.p);
         if (nM)
-            MH_LAUNCH(ctx, "walk_index", grid_for(ctx, nM, 256), 256, 0, table_index_kernel<NW>, mercy->keys, nM,
-                      k + 1, bits, offM.p);
-        Buf<uint64_t> next_walk(ctx, 1);
-        next_walk.zero();
-        MH_LAUNCH(ctx, "walk", grid_for(ctx, n_walks * 32, 256, 8), 256, 0, walk_kernel<NW>, solid->keys, nS, offS.p,
-                  mercy ? mercy->keys : nullptr, nM, offM.p, bits, k, n_walks, max_len, seed, slots.p, lens.p,
-                  (unsigned long long*)next_walk.p);
+            MH_LAUNCH(ctx, "walk_index", grid_for(ctx, nM, 256), 256, 0, table_index_kernel<NW>, mk, nM, k + 1, bits,
+                      offM.p);
+        if (linked) {
+            if (nS)
+                MH_LAUNCH(ctx, "walk_links", grid_for(ctx, nS, 256), 256, 0, walk_links_kernel<NW>, solid->keys, nS,
+                          (uint64_t)0, solid->keys, nS, offS.p, mk, nM, offM.p, bits, k, link.p, a.p);
+            if (nM)
+                MH_LAUNCH(ctx, "walk_links", grid_for(ctx, nM, 256), 256, 0, walk_links_kernel<NW>, mk, nM, nS,
+                          solid->keys, nS, offS.p, mk, nM, offM.p, bits, k, link.p, a.p);
+            const int g = grid_for(ctx, E, 256);
+            MH_LAUNCH(ctx, "walk_double", g, 256, 0, walk_double_kernel, a.p, E, 1, b.p);
+            MH_LAUNCH(ctx, "walk_double", g, 256, 0, walk_double_kernel, b.p, E, 2, a.p);
+            MH_LAUNCH(ctx, "walk_double", g, 256, 0, walk_double_kernel, a.p, E, 4, b.p);
+            MH_LAUNCH(ctx, "walk_double", g, 256, 0, walk_double_kernel, b.p, E, 8, c.p);
+            MH_LAUNCH(ctx, "walk", (unsigned)ceil_div(n_walks, 64), 64, 0, walk_linked_kernel<NW>, solid->keys, nS, mk,
+                      nM, link.p, a.p, c.p, k, n_walks, max_len, seed, stride, reinterpret_cast<uint32_t*>(slots.p),
+                      lens.p);
+        } else {
+            Buf<uint64_t> next_walk(ctx, 1);
+            next_walk.zero();
+            MH_LAUNCH(ctx, "walk", grid_for(ctx, n_walks * 32, 256, 8), 256, 0, walk_kernel<NW>, solid->keys, nS,
+                      offS.p, mk, nM, offM.p, bits, k, n_walks, max_len, seed, slots.p, lens.p,
+                      (unsigned long long*)next_walk.p);
+        }
     }
+    link.reset();
+    a.reset();
+    b.reset();
+    c.reset();
     exclusive_scan_u64(ctx, lens.p, off.p, n_walks);
     uint64_t total = 0;
     read_u64(ctx, off.p + n_walks, &total, 1);
     Buf<uint8_t> ascii(ctx, total + 16);
-    if (n_walks)
+    if (n_walks && linked)
+        MH_LAUNCH(ctx, "contig_unpack", (unsigned)n_walks, 256, 0, contig_unpack_kernel,
+                  reinterpret_cast<const uint32_t*>(slots.p), stride, off.p, ascii.p);
+    else if (n_walks)
         MH_LAUNCH(ctx, "contig_compact", (unsigned)n_walks, 256, 0, contig_compact_kernel, slots.p, max_len, off.p,
                   ascii.p);
     sync_and_check(ctx);
