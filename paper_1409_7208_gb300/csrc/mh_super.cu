@@ -15,9 +15,10 @@
 //
 //   split    tiles of 2,048 positions of the packed stream: the hashes of the
 //            tile's words, the smallest over each window, the runs; a run's
-//            record and its rank in its bin (one 64-bit atomic on the bin's
-//            counters: records low, windows high)
-//   place    after a scan of the counters, each record to its bin's place
+//            record goes to its bin's slots at the rank one 64-bit atomic on
+//            the bin's counters gives (records low, windows high)
+//   place    the records past their bin's slots (half as many again as the
+//            mean), from a list, to places after a scan
 //   count    a CTA per bin: a warp takes 32 records at a time, a lane a
 //            window; its mixed canonical key goes into a hash table in
 //            shared memory; then the table's entries (the spectrum) and the
@@ -72,11 +73,13 @@ __global__ void super_tiles_kernel(const uint64_t* __restrict__ offs, uint64_t F
     }
 }
 
-template <int M>
+// HALVES: bins by the smallest hashes of a window's halves (super_half).
+template <int M, bool HALVES>
 __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __restrict__ packed, uint64_t n_words,
                                                           const uint64_t* __restrict__ offs, uint64_t F,
                                                           const uint64_t* __restrict__ first, int k, uint32_t n_bins,
-                                                          uint32_t most, unsigned long long* __restrict__ rec, uint2* __restrict__ place,
+                                                          uint32_t most, uint32_t slots, uint64_t* __restrict__ rec,
+                                                          uint64_t* __restrict__ more, uint2* __restrict__ place,
                                                           uint64_t cap, unsigned long long* __restrict__ bins,
                                                           unsigned long long* __restrict__ totals) {
     constexpr int T = kSplitTile;
@@ -87,10 +90,11 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
     __shared__ uint32_t inv[T / 32], stop[T / 32];     // no window starts here; a run ends before here
     __shared__ uint16_t hpos[kSplitMaxRecs];
     __shared__ uint32_t edge[8], scratch[8];
-    __shared__ uint64_t out0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t base = (uint64_t)blockIdx.x * T;
-    const int w = k + 1 - M + 1;                       // words a window
+    const int words_all = k + 1 - M + 1;               // words a window
+    const int w = HALVES ? words_all / 2 : words_all;  // words a minimum is taken over
+    __shared__ uint32_t hmin[HALVES ? (T / 8 + 8) * 9 : 1];
     for (int i = tid; i < kSplitWords; i += 256) {
         const uint64_t g = base / 16 + i;
         words[i] = g < n_words ? packed[g] : 0u;
@@ -113,7 +117,7 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
     }
     // hashes of 8 positions a thread, and their smallest
     uint32_t h[8];
-    const int n_blk = 256 + (w + 6) / 8;
+    const int n_blk = 256 + (words_all + (HALVES ? 20 : 6)) / 8;
     for (int blk = tid; blk < n_blk; blk += 256) {
         const int wi = blk >> 1;
         const uint64_t hi = ((uint64_t)words[wi] << 32) | words[wi + 1];
@@ -134,25 +138,48 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
         }
     }
     __syncthreads();
-    // the smallest of each of the thread's 8 windows (w >= 8 positions each):
-    // its own positions from the window's start on, the positions all eight
-    // windows share (whole blocks by their minima), and the ones after
+    // the smallest of w positions from each of 8 on (w >= 8): the block's own
+    // positions from there on, the positions all eight share (whole blocks
+    // by their minima), and the ones after
     uint32_t mh[8];
-    {
+    auto minima = [&](int blk, const uint32_t h[8], uint32_t out[8]) {
         uint32_t mid = 0xFFFFFFFFu;
         const int nb = (w - 8) >> 3;
-        for (int q = 1; q <= nb; q++) mid = min(mid, bmin[tid + q]);
-        for (int p = 8 + 8 * nb; p < w; p++) mid = min(mid, hash[tid * 9 + p + (p >> 3)]);
-        mh[7] = h[7];
+        for (int q = 1; q <= nb; q++) mid = min(mid, bmin[blk + q]);
+        for (int p = 8 + 8 * nb; p < w; p++) mid = min(mid, hash[blk * 9 + p + (p >> 3)]);
+        out[7] = h[7];
 #pragma unroll
-        for (int i = 6; i >= 0; i--) mh[i] = min(h[i], mh[i + 1]);
-        mh[0] = min(mh[0], mid);
+        for (int i = 6; i >= 0; i--) out[i] = min(h[i], out[i + 1]);
+        out[0] = min(out[0], mid);
 #pragma unroll
         for (int i = 1; i < 8; i++) {
             const int p = w - 1 + i;
-            mid = min(mid, hash[tid * 9 + p + (p >> 3)]);
-            mh[i] = min(mh[i], mid);
+            mid = min(mid, hash[blk * 9 + p + (p >> 3)]);
+            out[i] = min(out[i], mid);
         }
+    };
+    if constexpr (HALVES) {
+        const int shift = words_all - w;  // from the first half to the last
+        for (int blk = tid; blk < 256 + (shift + 7) / 8; blk += 256) {
+            uint32_t v[8], o[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) v[j] = hash[blk * 9 + j];
+            minima(blk, v, o);
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                o[j] = super_mix(o[j]);
+                hmin[blk * 9 + j] = o[j];
+                if (blk == tid) mh[j] = o[j];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const int p = shift + i;
+            mh[i] += hmin[tid * 9 + p + (p >> 3)];
+        }
+    } else {
+        minima(tid, h, mh);
     }
     // heads: windows whose left neighbour is none or has another minimizer
     if (lane == 31) edge[warp] = mh[7];
@@ -168,7 +195,6 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
     reinterpret_cast<uint8_t*>(stop)[tid] = (uint8_t)(hm | ~vb);
     uint32_t total;
     uint32_t at = block_excl_scan_256(__popc(hm), scratch, &total);
-    if (tid == 0 && total) out0 = atomicAdd(&totals[T_RECS], (unsigned long long)total);
 #pragma unroll
     for (int i = 0; i < 8; i++)
         if ((hm >> i) & 1u) {
@@ -184,34 +210,59 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
         // (a run of more windows than a record may have, in a repeat, gives
         // several)
         uint32_t left = next_bit(stop, q + 1, T) - q, at = 0;
-        uint64_t o = out0 + j;
-        while (true) {
+        while (left) {
             const uint32_t nw = min(left, most);
-            const uint64_t r = atomicAdd(&bins[b], 1ull | ((unsigned long long)nw << 32));
-            if (o < cap) {
-                __stcs(&rec[o], (unsigned long long)(((base + q + at) << kNwinBits) | nw));
-                __stcs(&place[o], make_uint2(b, (uint32_t)r));
+            const uint32_t r = (uint32_t)atomicAdd(&bins[b], 1ull | ((unsigned long long)nw << 32));
+            const uint64_t v = ((base + q + at) << kNwinBits) | nw;
+            if (r < slots) {
+                rec[(uint64_t)b * slots + r] = v;
+            } else {
+                const uint64_t o = atomicAdd(&totals[T_RECS], 1ull);
+                if (o < cap) {
+                    more[o] = v;
+                    place[o] = make_uint2(b, r - slots);
+                }
             }
             left -= nw;
-            if (!left) break;
             at += nw;
-            o = atomicAdd(&totals[T_RECS], 1ull);
         }
     }
 }
 
-// Each record to its place in its bin (nothing if the records overflowed).
-__global__ void super_place_kernel(const unsigned long long* __restrict__ rec, const uint2* __restrict__ place, uint64_t cap,
+// over[b] = records of bin b past its slots.
+__global__ void super_over_kernel(const unsigned long long* __restrict__ bins, uint32_t n_bins, uint32_t slots,
+                                  uint32_t* __restrict__ over) {
+    for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < n_bins; b += gridDim.x * blockDim.x) {
+        const uint32_t r = (uint32_t)bins[b];
+        over[b] = r > slots ? r - slots : 0u;
+    }
+}
+
+// Each listed record to its place past its bin's slots (nothing if the list
+// overflowed).
+__global__ void super_place_kernel(const uint64_t* __restrict__ more, const uint2* __restrict__ place, uint64_t cap,
                                    const unsigned long long* __restrict__ totals, const uint64_t* __restrict__ off,
-                                   uint32_t b0, uint32_t b1, uint64_t* __restrict__ out) {
+                                   uint64_t* __restrict__ out) {
     const uint64_t n = totals[T_RECS];
     if (n > cap) return;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        // (each read once: not to displace the bins' open sectors in L2)
-        const uint2 p = __ldcs(&place[i]);
-        if (p.x - b0 < b1 - b0) out[(uint32_t)off[p.x] + (uint64_t)p.y] = __ldcs(&rec[i]);
+        const uint2 p = place[i];
+        out[off[p.x] + p.y] = more[i];
     }
 }
+
+// The records of the bins: bin b's first `slots` at rec[b * slots], the others
+// at more[off[b]]; bins[b] counts them (low half) and their windows (high).
+struct SuperRecs {
+    const uint64_t* rec;
+    const uint64_t* more;
+    const uint64_t* off;
+    const unsigned long long* bins;
+    uint32_t slots;
+    __device__ __forceinline__ uint64_t at(uint64_t b, uint64_t o, uint32_t i) const {
+        return i < slots ? rec[b * slots + i] : more[o + i - slots];
+    }
+};
 
 // Two table slots, read again each time (other lanes fill them).
 __device__ __forceinline__ ulonglong2 ld_pair(const uint64_t* p) {
@@ -284,8 +335,8 @@ struct SuperSmem {
 // probe_max slots leaves the bin to the rest, as do more than kMost entries.
 template <int NW>
 __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
-    super_count_kernel(const uint32_t* __restrict__ packed, const uint64_t* __restrict__ rec,
-                       const uint64_t* __restrict__ off, uint32_t b0, uint32_t b1, uint64_t rec_cap, int K1, int d,
+    super_count_kernel(const uint32_t* __restrict__ packed, SuperRecs recs, uint32_t b0, uint32_t b1,
+                       uint64_t rec_cap, int K1, int d,
                        uint32_t hot, int probe_max, uint64_t spec_cap, uint64_t* __restrict__ spec_k,
                        uint32_t* __restrict__ spec_len, uint64_t solid_cap, uint64_t* __restrict__ solid_k,
                        uint32_t* __restrict__ solid_c, uint64_t* __restrict__ soff, uint2* __restrict__ sidx,
@@ -363,9 +414,8 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     };
 
     for (uint32_t b = b0 + blockIdx.x; b < b1; b += gridDim.x) {
-        const uint64_t o0 = off[b], o1 = off[b + 1];
-        const uint32_t r0 = (uint32_t)o0, r1 = (uint32_t)o1;
-        const uint32_t W = (uint32_t)(o1 >> 32) - (uint32_t)(o0 >> 32);
+        const uint64_t have = recs.bins[b], o0 = recs.off[b];
+        const uint32_t n_rec = (uint32_t)have, W = (uint32_t)(have >> 32);
         if (tid == 0) over = W > hot;
         for (int i = tid; i < C::kSlots / 2; i += 256)
             reinterpret_cast<ulonglong2*>(fp)[i] = make_ulonglong2(kEmpty, kEmpty);
@@ -373,16 +423,16 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
         if (tid < C::kWords) occ[tid] = 0;
         // rounds of up to kRecs records: their windows are numbered through,
         // an eighth of them to each warp, 32 at a time
-        for (uint32_t rb = r0; rb < r1; rb += L::kRecs) {
+        for (uint32_t rb = 0; rb < n_rec; rb += L::kRecs) {
             __syncthreads();
             if (*(volatile uint32_t*)&over) break;
-            const uint32_t nr = min(r1 - rb, (uint32_t)L::kRecs);
+            const uint32_t nr = min(n_rec - rb, (uint32_t)L::kRecs);
             constexpr int R = (L::kRecs + 255) / 256;  // records a thread
             uint64_t rr[R];
             uint32_t sum = 0;
 #pragma unroll
             for (int q = 0; q < R; q++) {
-                rr[q] = (uint32_t)(R * tid + q) < nr ? rec[rb + R * tid + q] : 0ull;
+                rr[q] = (uint32_t)(R * tid + q) < nr ? recs.at(b, o0, rb + R * tid + q) : 0ull;
                 sum += (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
             }
             uint32_t tot;
@@ -575,18 +625,17 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
 // in no fixed order (a warp reserves its windows' places on the bin's cursor).
 template <int NW>
 __global__ void __launch_bounds__(256) super_expand_kernel(const uint32_t* __restrict__ packed,
-                                                           const uint64_t* __restrict__ rec,
-                                                           const uint64_t* __restrict__ off,
+                                                           SuperRecs recs,
                                                            const ulonglong2* __restrict__ deferred, uint64_t n_def,
                                                            int K1, unsigned long long* __restrict__ cursor,
                                                            uint64_t* __restrict__ out) {
     const int lane = threadIdx.x & 31;
     const uint32_t wy = blockIdx.y * 8 + (threadIdx.x >> 5), ny = gridDim.y * 8;
     for (uint64_t q = blockIdx.x; q < n_def; q += gridDim.x) {
-        const uint64_t b = deferred[q].x;
-        const uint32_t r0 = (uint32_t)off[b], r1 = (uint32_t)off[b + 1];
-        for (uint64_t rb = r0 + (uint64_t)wy * 32; rb < r1; rb += (uint64_t)ny * 32) {
-            const uint64_t r = rb + lane < r1 ? rec[rb + lane] : 0ull;
+        const uint64_t b = deferred[q].x, o0 = recs.off[b];
+        const uint32_t n_rec = (uint32_t)recs.bins[b];
+        for (uint64_t rb = (uint64_t)wy * 32; rb < n_rec; rb += (uint64_t)ny * 32) {
+            const uint64_t r = rb + lane < n_rec ? recs.at(b, o0, (uint32_t)rb + lane) : 0ull;
             const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)r & ((1u << kNwinBits) - 1u));
             uint64_t at = 0;
             if (lane == 0) at = deferred[q].y + atomicAdd(&cursor[q], (unsigned long long)tot);
@@ -632,12 +681,18 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     Buf<unsigned long long> bins(ctx, n_bins);
     MH_LAUNCH(ctx, "super_tiles", grid_for(ctx, n_tiles, 256), 256, 0, super_tiles_kernel, reads->frag_offs, F,
               n_tiles, first.p);
-    // records: 2 / (w + 1) a window for random sequences, one more a fragment
-    // and a tile; if there are more, again with room for what there is
-    uint64_t cap = (uint64_t)(2.5 / (w + 1) * (double)n) + F + n_tiles + 4096;
-    cap = std::min(cap, n);
+    // records: 2 / (w + 1) a window for random sequences (about 8 / w by
+    // halves), one more a fragment and a tile; each bin has slots for half as
+    // many again as its share, and the list of those past them room for a
+    // quarter of all (again with room for what there is, if there are more)
+    const double run = super_half(K1) ? w / 8.0 : (w + 1) / 2.0;
+    const uint64_t expect = std::min(n, (uint64_t)((double)n / run) + F + n_tiles + 1);
+    const uint32_t slots = (uint32_t)((double)expect / n_bins * 1.5) + 16;
+    uint64_t cap = expect / 4 + 4096;
+    Buf<uint64_t> rec(ctx, (uint64_t)n_bins * slots);
     unsigned long long* tot = reinterpret_cast<unsigned long long*>(totals.p);
-    Buf<uint64_t> rec;
+    Buf<uint64_t> more;
+    SuperRecs recs{rec.p, nullptr, off.p, bins.p, slots};
     uint64_t h[8] = {0};
     Buf<uint64_t> spec, solid, soff(ctx, n_bins);
     Buf<uint32_t> spec_len, solid_c;
@@ -652,7 +707,7 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     auto count = [&](uint32_t b0, uint32_t b1) {
         if (b0 < b1)
             MH_LAUNCH_B(ctx, "super_count", n / 4, (unsigned)std::min<uint64_t>(b1 - b0, (uint64_t)ctx->num_sms * std::max(1, per_sm)),
-                        256, smem, super_count_kernel<NW>, reads->packed, rec.p, off.p, b0, b1, cap, K1, d, hot,
+                        256, smem, super_count_kernel<NW>, reads->packed, recs, b0, b1, cap, K1, d, hot,
                         probes, spec_cap, spec.p, spec_len.p, solid_cap, solid.p, solid_c.p, soff.p, sidx.p,
                         deferred.p, tot);
     };
@@ -667,37 +722,40 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     // large sets: a sixteenth of the bins first, to size the outputs by
     const bool sample = n >= (1ull << 25) && n_bins >= 4096;
     const uint32_t nb1 = sample ? n_bins / 16 : n_bins;
+    bool all = false;
     for (int attempt = 0;; attempt++) {
-        rec.reset();
-        rec = Buf<uint64_t>(ctx, cap);
+        more.reset();
+        more = Buf<uint64_t>(ctx, cap);
+        recs.more = more.p;
         {
-            Buf<unsigned long long> raw(ctx, cap);
+            Buf<uint64_t> raw(ctx, cap);
             Buf<uint2> place(ctx, cap);
+            Buf<uint32_t> over(ctx, n_bins);
             bins.zero();
             totals.zero();
-            const auto split = m == 16 ? super_split_kernel<16> : m == 14 ? super_split_kernel<14> : super_split_kernel<12>;
+            const auto split = super_half(K1) ? super_split_kernel<16, true>
+                               : m == 16      ? super_split_kernel<16, false>
+                               : m == 14      ? super_split_kernel<14, false>
+                                              : super_split_kernel<12, false>;
             MH_LAUNCH_B(ctx, "super_split", reads->n_packed / 4, (unsigned)n_tiles, 256, 0, split, reads->packed, n_words,
-                        reads->frag_offs, F, first.p, k, n_bins, (uint32_t)(32 * C::kRecWords / 2 - K1 + 1), raw.p, place.p, cap, bins.p, tot);
-            exclusive_scan_u64(ctx, reinterpret_cast<const uint64_t*>(bins.p), off.p, n_bins);
-            // in ranges of bins whose open sectors (32 bytes a bin) and
-            // offsets stay in L2 beside the streams (3 Gbp, 850,000 bins:
-            // 10.6 ms in one range, 8.1 in four, 8.5 in eight)
-            const int G = (int)std::max<uint64_t>(1, std::min<uint64_t>(8, ceil_div(n_bins, 220000)));
-            for (int g = 0; g < G; g++)
-                MH_LAUNCH(ctx, "super_place", grid_for(ctx, cap, 256), 256, 0, super_place_kernel, raw.p, place.p, cap, tot,
-                          off.p, (uint32_t)((uint64_t)n_bins * g / G), (uint32_t)((uint64_t)n_bins * (g + 1) / G), rec.p);
+                        reads->frag_offs, F, first.p, k, n_bins, (uint32_t)(32 * C::kRecWords / 2 - K1 + 1), slots, rec.p,
+                        raw.p, place.p, cap, bins.p, tot);
+            MH_LAUNCH(ctx, "super_over", grid_for(ctx, n_bins, 256), 256, 0, super_over_kernel, bins.p, n_bins, slots,
+                      over.p);
+            exclusive_scan_u32(ctx, over.p, off.p, n_bins);
+            MH_LAUNCH(ctx, "super_place", grid_for(ctx, cap, 256), 256, 0, super_place_kernel, raw.p, place.p, cap, tot,
+                      off.p, more.p);
         }
-        uint64_t n1 = n;
-        if (sample) {
-            read_u64(ctx, off.p + nb1, &n1, 1);
-            n1 >>= 32;
-        }
+        // (room for a sample with twice its share of the windows; with all of
+        // them if it has more)
+        const uint64_t n1 = sample && !all ? n / 8 : n;
         room(std::max<uint64_t>(n1, 1), std::max<uint64_t>(n1 * per, 1));
         count(0, nb1);
         read_u64(ctx, totals.p, h, T_N);
-        if (h[T_RECS] <= cap) break;
-        if (attempt) fail(MH_EDEVICE, "super-k-mer records overflow twice");
-        cap = h[T_RECS];
+        if (h[T_RECS] <= cap && h[T_SPEC] <= spec_cap && h[T_SOLID] <= solid_cap) break;
+        if (attempt >= 2) fail(MH_EDEVICE, "super-k-mer records overflow again");
+        all = h[T_RECS] <= cap;
+        cap = std::max(cap, h[T_RECS]);
     }
     if (sample) {
         // the other bins into buffers sized by the first ones (bins are by
@@ -744,9 +802,10 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         cursor.zero();
         const unsigned gx = (unsigned)std::min<uint64_t>(h[T_DEF], 4096);
         const unsigned gy = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(64, (uint64_t)ctx->num_sms * 8 / gx));
-        MH_LAUNCH(ctx, "super_expand", dim3(gx, gy), 256, 0, super_expand_kernel<NW>, reads->packed, rec.p, off.p,
+        MH_LAUNCH(ctx, "super_expand", dim3(gx, gy), 256, 0, super_expand_kernel<NW>, reads->packed, recs,
                   deferred.p, h[T_DEF], K1, cursor.p, keys.p);
         rec.reset();
+        more.reset();
         const GroupPlan gp = group_plan(ctx, nd, 0, NW);
         if (gp.passes < 0) fail(MH_EDEVICE, "super-k-mer counting: no unit plan for the deferred bins");
         const bool in_alt = gp.passes ? radix_sort<NW>(ctx, keys.p, alt.p, nullptr, nullptr, nd, 64 * NW - 8 * gp.passes, 64 * NW)
@@ -760,6 +819,7 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         S += rest_S;
     }
     rec.reset();
+    more.reset();
     first.reset();
     off.reset();
     bins.reset();

@@ -12,6 +12,17 @@ namespace mh {
 // windows over more bins and shorter ones give longer super-k-mers.
 __host__ __device__ inline int super_m(int K1) { return K1 >= 32 ? 16 : K1 >= 26 ? 14 : K1 >= 21 ? 12 : 0; }
 
+// Windows of many words: a bin by one minimizer would get whole runs of about
+// w / 2 windows at a time, times the coverage, more than a bin's table holds
+// where a genome is abundant.  From 48 words on, the window's bin is by the
+// smallest hash of its first and of its last half words together (swapped in
+// the reverse complement, so combined by a sum): runs of about w / 8 windows.
+// 0: by one minimizer, else the words of a half.
+__host__ __device__ inline int super_half(int K1) {
+    const int w = K1 - super_m(K1) + 1;
+    return w >= 48 ? w / 2 : 0;
+}
+
 // Order of the canonical minimizer-length words: an affine map of 32-bit
 // words (one multiply-add), so that runs of one symbol are not the smallest.
 __host__ __device__ __forceinline__ uint32_t super_hash(uint32_t c) { return c * 0x9E3779B1u + 0x7F4A7C15u; }
@@ -58,14 +69,15 @@ struct SuperIndex {
     uint64_t n_main = 0, n = 0;
 };
 
-// Smallest hash over the canonical minimizer-length words of a window x of
-// K1 symbols with reverse complement r.
+// What decides the bin of a window x of K1 symbols with reverse complement
+// r: the smallest hash over its canonical minimizer-length words, or (halves)
+// the sum of its halves' mixed smallest hashes.
 template <int NW>
 __device__ __forceinline__ uint32_t super_min(Key<NW> x, Key<NW> r, int K1, int m) {
     const uint32_t mask = m == 16 ? 0xFFFFFFFFu : (1u << (2 * m)) - 1u;
     // word j from the end: x's symbols [K1 - m - j, K1 - j), r's [j, j + m)
-    uint32_t best = 0xFFFFFFFFu;
-    const int w = K1 - m + 1;
+    uint32_t best = 0xFFFFFFFFu, last = 0xFFFFFFFFu;
+    const int w = K1 - m + 1, half = super_half(K1);
     const int top = 2 * (K1 - m);
     if constexpr (NW == 1) {
         for (int j = 0; j < w; j++) {
@@ -78,10 +90,11 @@ __device__ __forceinline__ uint32_t super_min(Key<NW> x, Key<NW> r, int K1, int 
             const uint32_t f = (uint32_t)key_shr<NW>(x, 2 * j).w[0] & mask;
             const uint32_t g = (uint32_t)key_shr<NW>(r, top - 2 * j).w[0] & mask;
             const uint32_t h = super_hash(f < g ? f : g);
-            best = h < best ? h : best;
+            if (!half || j < half) best = h < best ? h : best;
+            if (half && j >= w - half) last = h < last ? h : last;
         }
     }
-    return best;
+    return half ? super_mix(best) + super_mix(last) : best;
 }
 
 // Run length of a window (x, its reverse complement r) in the spectrum, 0 if
