@@ -12,16 +12,10 @@
 //   analyse   per entry: minus flag (an earlier entry of the same group
 //             e[1..k-1] has the same label; groups are contiguous and hold at
 //             most 16 entries), node head/last flags
-//   nodes     B = reversed source nodes (ck >> 2 at heads), ascending
-//   targets   A = reversed targets (label, e[k-1], ..., e[1]) of unflagged
-//             entries; already ascending within each label, so one stable
-//             radix pass on their top 8 bits sorts them
-//   joins     zero indegree = B \ A, zero outdegree = A \ B, both from one
-//             merge-path merge of A and B (an element of both has its copies
-//             adjacent in the merge); B and A are tile compactions with a
-//             decoupled look-back
+//   degrees   zero outdegree: a join of the targets against the nodes, both in
+//             colex order; zero indegree: their reverse complements
 //   padding   dummy entries (node $ v[0..k-2], label v[k-1]) sorted by
-//             (v[k-2..0], v[k-1]); $ entries in the order of A \ B
+//             (v[k-2..0], v[k-1]); $ entries in the order of their nodes
 //   merge     final position of every entry: its rank in its own list plus
 //             the number of entries of the other lists below it, by binary
 //             search and a scan of insertion counts over E
@@ -140,88 +134,210 @@ __global__ void analyse_kernel(const uint64_t* __restrict__ ck, uint64_t E, uint
     }
 }
 
-// Tile compaction: 256 threads x 8 consecutive entries per tile, a block
-// scan of the per-thread counts and a decoupled look-back for the tile's
-// output offset (one read of the input, no flag or position arrays).
-constexpr int kCmpItems = 8;
-constexpr int kCmpTile = 256 * kCmpItems;
-
-// Heads (new nodes) -> B = reversed source nodes; unflagged entries -> A =
-// reversed targets (label, e[k-1], ..., e[1]).  Two output streams.
+// Zero-outdegree nodes.  In colex order the targets of the edges with label c
+// are c followed by their groups (e[k-1], ..., e[1]), ascending; so a tile of
+// whole groups of the order meets, for each label, one contiguous range of
+// the order's nodes.  The tile's groups and the labels each holds stay in
+// shared memory, the four ranges are streamed past them, and a node c.g
+// clears label c of group g: what is left are targets that no edge leaves.
+// Reads every key twice and writes next to nothing; bound by the searches in
+// shared memory.  3.5e8 edges of one word: 4.9 ms, where writing the sorted
+// nodes and targets, one radix pass and the merge of their differences took
+// 12.6.
 template <int NW>
-__global__ void __launch_bounds__(256) nodes_targets_kernel(const uint64_t* __restrict__ ck,
-                                                            const uint8_t* __restrict__ fl, uint64_t E, int k,
-                                                            uint64_t* __restrict__ B, uint64_t* __restrict__ A,
-                                                            uint64_t* __restrict__ status_b,
-                                                            uint64_t* __restrict__ status_a,
-                                                            uint32_t* __restrict__ tile_counter,
-                                                            uint32_t* __restrict__ err) {
+struct ZeroTile {
+    static constexpr int kItems = 8 / NW;             // entries a thread
+    static constexpr int kCap = 256 * kItems;
+    static constexpr int kTile = kCap - 16;           // a group holds at most 16 entries
+};
+
+// st[t] = the first group start at or after t * kTile (t = 0..n_tiles; E at
+// the end); tb[4 t + c] = the first entry whose node is c.g or above, g the
+// group at st[t] (the end of c's block for t = n_tiles or no such group).
+template <int NW>
+__global__ void zero_bounds_kernel(const uint64_t* __restrict__ ck, uint64_t E, int k, uint64_t n_tiles,
+                                   uint64_t* __restrict__ st, uint64_t* __restrict__ tb) {
+    for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < (n_tiles + 1) * 4;
+         q += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t t = q >> 2;
+        const uint32_t c = (uint32_t)(q & 3);
+        uint64_t s = t < n_tiles ? t * ZeroTile<NW>::kTile : E;
+        if (s > 0)
+            while (s < E && key_eq<NW>(key_shr<NW>(load_key<NW>(ck, s), 4), key_shr<NW>(load_key<NW>(ck, s - 1), 4))) s++;
+        if (c == 0) st[t] = s;
+        Key<NW> x = key_zero<NW>();
+        uint64_t b = E;
+        if (!(s >= E && c == 3)) {
+            x.w[0] = s >= E ? c + 1 : c;
+            x = key_shl<NW>(x, 2 * k);
+            if (t > 0 && s < E) {
+                const Key<NW> g = key_shl<NW>(key_shr<NW>(load_key<NW>(ck, s), 4), 2);
+#pragma unroll
+                for (int w = 0; w < NW; w++) x.w[w] |= g.w[w];
+            }
+            uint64_t lo = 0;
+            while (lo < b) {
+                const uint64_t mid = (lo + b) >> 1;
+                if (key_less<NW>(load_key<NW>(ck, mid), x)) lo = mid + 1; else b = mid;
+            }
+        }
+        tb[q] = b;
+    }
+}
+
+// Tile t's targets without out-edges, as reversed nodes: cnt[c * n_tiles + t]
+// of them with label c, ascending, from found[at[t]] on, label after label.
+template <int NW>
+__global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restrict__ ck, int k, uint64_t n_tiles,
+                                                       const uint64_t* __restrict__ st,
+                                                       const uint64_t* __restrict__ tb, uint64_t* __restrict__ found,
+                                                       uint64_t* __restrict__ at, uint32_t* __restrict__ cnt,
+                                                       unsigned long long* __restrict__ n_found) {
+    using Z = ZeroTile<NW>;
+    constexpr int I = Z::kItems;
+    __shared__ __align__(16) uint64_t gk[Z::kCap * NW];  // the groups
+    __shared__ uint32_t gm[Z::kCap];        // labels left
     __shared__ uint32_t scratch[8];
-    __shared__ uint64_t offs[2];
-    __shared__ uint32_t s_tile;
-    if (threadIdx.x == 0) s_tile = atomicAdd(tile_counter, 1u);
-    __syncthreads();
-    const uint64_t tile = s_tile;
-    const uint64_t i0 = tile * kCmpTile + (uint64_t)threadIdx.x * kCmpItems;
-    uint32_t hm = 0, pm = 0;
-    // the 8 flags in one load, and the keys loaded before the look-back waits
-    static_assert(kCmpItems == 8, "one 8-byte flag load per thread");
-    uint8_t f8[kCmpItems];
-    if (i0 + kCmpItems <= E) {
-        const uint2 v = *reinterpret_cast<const uint2*>(fl + i0);
+    __shared__ uint64_t wsum[8], base;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t t = blockIdx.x, s0 = st[t];
+    const uint32_t n = (uint32_t)(st[t + 1] - s0);  // at most kTile + 15
+    // groups, numbered in order
+    Key<NW> x[I];
+    uint32_t heads = 0;
+    const uint32_t i0 = tid * I;
+    for (int j = 0; j < I; j++) gm[i0 + j] = 0;
+    {
+        Key<NW> prev = key_zero<NW>();
+        if (i0 > 0 && i0 < n) prev = load_key<NW>(ck, s0 + i0 - 1);
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            f8[j] = (uint8_t)(v.x >> (8 * j));
-            f8[4 + j] = (uint8_t)(v.y >> (8 * j));
-        }
-    } else {
+        for (int j = 0; j < I; j++)
+            if (i0 + j < n) x[j] = load_key<NW>(ck, s0 + i0 + j);
 #pragma unroll
-        for (int j = 0; j < kCmpItems; j++) f8[j] = i0 + j < E ? fl[i0 + j] : 0;
-    }
-    Key<NW> xs[kCmpItems];
-#pragma unroll
-    for (int j = 0; j < kCmpItems; j++) {
-        if (i0 + j < E) {
-            hm |= ((f8[j] >> 1) & 1u) << j;
-            pm |= ((f8[j] & 1u) ^ 1u) << j;
-            if ((f8[j] & 3u) != 1u) xs[j] = load_key<NW>(ck, i0 + j);
+        for (int j = 0; j < I; j++) {
+            if (i0 + j >= n) continue;
+            if (i0 + j == 0 || !key_eq<NW>(key_shr<NW>(x[j], 4), key_shr<NW>(j ? x[j > 0 ? j - 1 : 0] : prev, 4)))
+                heads |= 1u << j;
         }
     }
-    uint32_t tot_b, tot_a;
-    const uint32_t eb = block_excl_scan_256(__popc(hm), scratch, &tot_b);
-    const uint32_t ea = block_excl_scan_256(__popc(pm), scratch, &tot_a);
-    const int warp = threadIdx.x >> 5;
-    if (warp == 0) {
-        const uint64_t o = warp_lookback_u64(status_b, tile, tot_b, err);
-        if ((threadIdx.x & 31) == 0) offs[0] = o;
-    } else if (warp == 1) {
-        const uint64_t o = warp_lookback_u64(status_a, tile, tot_a, err);
-        if ((threadIdx.x & 31) == 0) offs[1] = o;
+    uint32_t ng;
+    uint32_t g = block_excl_scan_256(__popc(heads), scratch, &ng);
+#pragma unroll
+    for (int j = 0; j < I; j++) {
+        if (i0 + j >= n) continue;
+        if ((heads >> j) & 1u) store_key<NW>(gk, g++, key_shr<NW>(x[j], 4));
+        atomicOr(&gm[g - 1], 1u << (uint32_t)(x[j].w[0] & 3u));
     }
     __syncthreads();
-    uint64_t pb = offs[0] + eb, pa = offs[1] + ea;
+    // the nodes with first symbol c: two warps a label, I entries a thread,
+    // the first one's group by bisection, the others' from there on
+    {
+        const uint32_t c = (uint32_t)warp >> 1;
+        const uint64_t b0 = tb[4 * t + c], b1 = tb[4 * (t + 1) + c];
+        for (uint64_t q = b0 + (uint64_t)(tid & 63) * I; q < b1; q += 64 * I) {
+            Key<NW> y[I];
 #pragma unroll
-    for (int j = 0; j < kCmpItems; j++) {
-        if (!(((hm | pm) >> j) & 1u)) continue;
-        const Key<NW> x = xs[j];
-        if ((hm >> j) & 1u) store_key<NW>(B, pb++, key_shr<NW>(x, 2));
-        if ((pm >> j) & 1u) {
-            Key<NW> t = key_shr<NW>(x, 4);
-            Key<NW> lab = key_zero<NW>();
-            lab.w[0] = x.w[0] & 3u;
-            lab = key_shl<NW>(lab, 2 * (k - 1));
+            for (int j = 0; j < I; j++)
+                if (q + j < b1) y[j] = key_low<NW>(key_shr<NW>(load_key<NW>(ck, q + j), 2), 2 * (k - 1));
+            uint32_t p = 0;
+            {
+                uint32_t hi = ng;
+                while (p < hi) {
+                    const uint32_t mid = (p + hi) >> 1;
+                    if (key_less<NW>(load_key<NW>(gk, mid), y[0])) p = mid + 1; else hi = mid;
+                }
+            }
 #pragma unroll
-            for (int w = 0; w < NW; w++) t.w[w] |= lab.w[w];
-            store_key<NW>(A, pa++, t);
+            for (int j = 0; j < I; j++) {
+                if (q + j >= b1 || (j && key_eq<NW>(y[j], y[j > 0 ? j - 1 : 0]))) continue;
+                while (p < ng && key_less<NW>(load_key<NW>(gk, p), y[j])) p++;
+                if (p < ng && key_eq<NW>(load_key<NW>(gk, p), y[j])) atomicAnd(&gm[p], ~(1u << c));
+            }
+        }
+    }
+    __syncthreads();
+    // what is left, label by label (the four counts in one 64-bit scan)
+    uint64_t mine = 0;
+    uint32_t m[I];
+#pragma unroll
+    for (int j = 0; j < I; j++) {
+        m[j] = i0 + j < ng ? gm[i0 + j] : 0u;
+#pragma unroll
+        for (int c = 0; c < 4; c++) mine += (uint64_t)((m[j] >> c) & 1u) << (16 * c);
+    }
+    uint64_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint64_t pre = incl - mine, tot = 0;
+    for (int q = 0; q < 8; q++) {
+        pre += q < warp ? wsum[q] : 0ull;
+        tot += wsum[q];
+    }
+    uint32_t tc[4], to[4], all = 0;
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        tc[c] = (uint32_t)(tot >> (16 * c)) & 0xFFFFu;
+        to[c] = all;
+        all += tc[c];
+    }
+    if (tid == 0) {
+        base = all ? atomicAdd(n_found, (unsigned long long)all) : 0ull;
+        at[t] = base;
+#pragma unroll
+        for (int c = 0; c < 4; c++) cnt[c * n_tiles + t] = tc[c];
+    }
+    if (!all) return;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        uint64_t o = base + to[c] + ((uint32_t)(pre >> (16 * c)) & 0xFFFFu);
+#pragma unroll
+        for (int j = 0; j < I; j++)
+            if ((m[j] >> c) & 1u) {
+                Key<NW> v = key_zero<NW>();
+                v.w[0] = (uint64_t)c;
+                v = key_shl<NW>(v, 2 * (k - 1));
+                const Key<NW> gg = load_key<NW>(gk, i0 + j);
+#pragma unroll
+                for (int w = 0; w < NW; w++) v.w[w] |= gg.w[w];
+                store_key<NW>(found, o++, v);
+            }
+    }
+}
+
+// The tiles' finds in order: those of (label c, tile t) to off[c * n_tiles + t]
+// (thread per tile: a few finds each).
+template <int NW>
+__global__ void zero_gather_kernel(const uint64_t* __restrict__ found, const uint64_t* __restrict__ at,
+                                   const uint32_t* __restrict__ cnt, const uint64_t* __restrict__ off,
+                                   uint64_t n_tiles, uint64_t* __restrict__ out) {
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n_tiles;
+         t += (uint64_t)gridDim.x * blockDim.x) {
+        uint64_t a = at[t];
+        for (int c = 0; c < 4; c++) {
+            const uint32_t m = cnt[c * n_tiles + t];
+            const uint64_t o = off[c * n_tiles + t];
+            for (uint32_t j = 0; j < m; j++) store_key<NW>(out, o + j, load_key<NW>(found, a + j));
+            a += m;
         }
     }
 }
 
-// zero-indegree reversed node v_rev -> dummy key (v[k-2], ..., v[0], v[k-1])
+// The zero-indegree nodes are the reverse complements v of the zero-outdegree
+// nodes u (the edges are closed under reverse complement): reversed node u ->
+// dummy key (v[k-2], ..., v[0], v[k-1]).
 template <int NW>
-__global__ void dummy_keys_kernel(const uint64_t* __restrict__ zin, uint64_t t, int k, uint64_t* __restrict__ dk) {
+__global__ void dummy_keys_kernel(const uint64_t* __restrict__ zout, uint64_t t, int k, uint64_t* __restrict__ dk) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < t; i += (uint64_t)gridDim.x * blockDim.x) {
-        Key<NW> v = load_key<NW>(zin, i);
+        // v reversed = the complement of u
+        Key<NW> v = key_rev<NW>(load_key<NW>(zout, i), k);
+#pragma unroll
+        for (int w = 0; w < NW; w++) v.w[w] = ~v.w[w];
         Key<NW> low = key_low<NW>(v, 2 * (k - 1));
         Key<NW> top = key_shr<NW>(v, 2 * (k - 1));
         store_key<NW>(dk, i, key_or_low<NW>(key_shl<NW>(low, 2), top.w[0] & 3u));
@@ -373,40 +489,38 @@ void build_sdbg(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, mh_sd
     }
     ck2.reset();
     cv2.reset();
-    // per-entry flags, node list B, target list A
+    // per-entry flags
     Buf<uint8_t> fl(ctx, E ? E : 1);
     if (E) MH_LAUNCH(ctx, "analyse", grid_for(ctx, E, 256), 256, 0, analyse_kernel<NW>, ck.p, E, fl.p);
-    Buf<uint64_t> B(ctx, (E ? E : 1) * NW), A(ctx, (E ? E : 1) * NW);
-    uint64_t nB = 0, nA = 0;
+    // zero outdegree, ascending (as many nodes have zero indegree)
+    Buf<uint64_t> zout;
+    uint64_t u = 0;
     if (E) {
-        const uint64_t tiles = ceil_div(E, kCmpTile);
-        Buf<uint64_t> st(ctx, 2 * tiles);
-        Buf<uint32_t> counter(ctx, 1);
-        st.zero();
-        counter.zero();
-        MH_LAUNCH(ctx, "nodes_targets", (unsigned)tiles, 256, 0, nodes_targets_kernel<NW>, ck.p, fl.p, E, k, B.p, A.p,
-                  st.p, st.p + tiles, counter.p, ctx->d_status);
-        uint64_t last[2];
-        read_u64(ctx, st.p + tiles - 1, &last[0], 1);
-        read_u64(ctx, st.p + 2 * tiles - 1, &last[1], 1);
-        nB = last[0] & kLbCountMask;
-        nA = last[1] & kLbCountMask;
+        const uint64_t tiles = ceil_div(E, (uint64_t)ZeroTile<NW>::kTile);
+        Buf<uint64_t> st(ctx, tiles + 1), tb(ctx, 4 * (tiles + 1)), found(ctx, E * NW), at(ctx, tiles + 1),
+            off(ctx, 4 * tiles + 1);
+        Buf<uint32_t> cnt(ctx, 4 * tiles);
+        Buf<unsigned long long> n_found(ctx, 1);
+        n_found.zero();
+        MH_LAUNCH(ctx, "zero_bounds", grid_for(ctx, 4 * (tiles + 1), 256), 256, 0, zero_bounds_kernel<NW>, ck.p, E, k,
+                  tiles, st.p, tb.p);
+        MH_LAUNCH_B(ctx, "zero_out", 2 * E * 8 * NW, (unsigned)tiles, 256, 0, zero_out_kernel<NW>, ck.p, k, tiles, st.p,
+                    tb.p, found.p, at.p, cnt.p, n_found.p);
+        exclusive_scan_u32(ctx, cnt.p, off.p, 4 * tiles);
+        read_u64(ctx, off.p + 4 * tiles, &u, 1);
+        zout = Buf<uint64_t>(ctx, (u ? u : 1) * NW);
+        if (u)
+            MH_LAUNCH(ctx, "zero_gather", grid_for(ctx, tiles, 256), 256, 0, zero_gather_kernel<NW>, found.p, at.p,
+                      cnt.p, off.p, tiles, zout.p);
+    } else {
+        zout = Buf<uint64_t>(ctx, NW);
     }
-    Buf<uint64_t> A2(ctx, (nA ? nA : 1) * NW);
-    if (radix_sort<NW>(ctx, A.p, A2.p, nullptr, nullptr, nA, std::max(0, 2 * k - 8), 2 * k)) std::swap(A, A2);
-    A2.reset();
-    // zero indegree: B \ A; zero outdegree: A \ B
-    Buf<uint64_t> zin(ctx, (nB ? nB : 1) * NW), zout(ctx, (nA ? nA : 1) * NW);
-    uint64_t t = 0, u = 0;
-    set_differences<NW>(ctx, B.p, nB, A.p, nA, zin.p, &t, zout.p, &u);
-    B.reset();
-    A.reset();
+    const uint64_t t = u;
     // dummy entries in colex order
     Buf<uint64_t> dk(ctx, (t ? t : 1) * NW), dk2(ctx, (t ? t : 1) * NW);
-    if (t) MH_LAUNCH(ctx, "dummy_keys", grid_for(ctx, t, 256), 256, 0, dummy_keys_kernel<NW>, zin.p, t, k, dk.p);
+    if (t) MH_LAUNCH(ctx, "dummy_keys", grid_for(ctx, t, 256), 256, 0, dummy_keys_kernel<NW>, zout.p, t, k, dk.p);
     if (radix_sort<NW>(ctx, dk.p, dk2.p, nullptr, nullptr, t, 0, 2 * k)) std::swap(dk, dk2);
     dk2.reset();
-    zin.reset();
     // merge positions
     const uint64_t m = E + t + u;
     Buf<uint32_t> ins(ctx, E + 1);

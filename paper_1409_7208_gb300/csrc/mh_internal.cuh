@@ -539,64 +539,6 @@ __device__ __forceinline__ bool any_bit(const uint32_t* b, uint32_t i, uint32_t 
     return next_bit(b, i, j) < j;
 }
 
-// ------------------------------------------------ tile compaction helpers
-// 64-bit per-tile status words for decoupled look-back: flag in the top two
-// bits (aggregate / inclusive), count in the low 62.
-constexpr uint64_t kLbAgg = 1ull << 62;
-constexpr uint64_t kLbInc = 2ull << 62;
-constexpr uint64_t kLbCountMask = (1ull << 62) - 1;
-
-__device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t* p) {
-    uint64_t v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed_u64(uint64_t* p, uint64_t v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// Called by one whole warp of the tile: publishes the tile's total, looks
-// back over earlier tiles (lane l reads tile j - l, the window is used up to
-// the nearest inclusive entry; every wait is bounded) and returns the sum of
-// all earlier tiles' totals.  Tiles must be numbered in launch-claim order
-// (a dynamic tile id) so that every earlier tile is running or done.
-__device__ __forceinline__ uint64_t warp_lookback_u64(uint64_t* status, uint64_t tile, uint64_t total,
-                                                      uint32_t* err) {
-    const int lane = threadIdx.x & 31;
-    uint64_t* st = status + tile;
-    if (lane == 0) st_relaxed_u64(st, (tile == 0 ? kLbInc : kLbAgg) | total);
-    uint64_t excl = 0;
-    bool ok = true;
-    for (int64_t j = (int64_t)tile - 1; j >= 0 && ok; j -= 32) {
-        const int64_t idx = j - lane;
-        uint64_t v = idx >= 0 ? ld_relaxed_u64(status + idx) : kLbInc;
-        int spins = 0;
-        uint32_t inc;
-        while (true) {
-            inc = __ballot_sync(0xFFFFFFFFu, (v & ~kLbCountMask) == kLbInc);
-            const uint32_t need = inc ? ((inc & (0u - inc)) << 1) - 1u : 0xFFFFFFFFu;
-            const uint32_t waiting = __ballot_sync(0xFFFFFFFFu, (v & ~kLbCountMask) == 0) & need;
-            if (!waiting) break;
-            if (++spins > (1 << 23)) {
-                ok = false;
-                break;
-            }
-            if (spins > 64) __nanosleep(128);
-            if (idx >= 0 && (v & ~kLbCountMask) == 0) v = ld_relaxed_u64(status + idx);
-        }
-        const uint32_t need = inc ? ((inc & (0u - inc)) << 1) - 1u : 0xFFFFFFFFu;
-        uint64_t c = ((need >> lane) & 1u) ? (v & kLbCountMask) : 0;
-        for (int off = 16; off; off >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, off);
-        excl += c;
-        if (inc) break;
-    }
-    if (lane == 0) {
-        if (!ok) atomicOr(err, 1u);  // ST_SPIN_TIMEOUT
-        if (tile > 0) st_relaxed_u64(st, kLbInc | (excl + total));
-    }
-    return excl;
-}
-
 // Exclusive prefix of a per-thread count over a block of 256 threads (8
 // warps); `scratch` holds 8 words of shared memory.  Also returns the total.
 __device__ __forceinline__ uint32_t block_excl_scan_256(uint32_t v, uint32_t* scratch, uint32_t* total) {
@@ -707,11 +649,6 @@ void exclusive_scan_u32(mh_ctx* ctx, const uint32_t* in, uint64_t* out, uint64_t
 template <int NW>
 bool merge_runs(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* vals, uint32_t* valt,
                 const std::vector<uint64_t>& bounds);
-
-// X \ Y and Y \ X of two sorted arrays without repeats, each in order.
-template <int NW>
-void set_differences(mh_ctx* ctx, const uint64_t* X, uint64_t nx, const uint64_t* Y, uint64_t ny, uint64_t* outX,
-                     uint64_t* n_outX, uint64_t* outY, uint64_t* n_outY);
 
 // One read set through pack, count and (by flags) mercy and build on
 // context w (mh_batch.cu); a failed set keeps no outputs.
