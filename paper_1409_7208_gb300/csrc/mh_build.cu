@@ -9,17 +9,15 @@
 //             table backwards from its end, each block of equal first symbol
 //             f[0] gives ck ascending; so the ck of solid and mercy edges are
 //             8 sorted runs, merged by a tree of merge-path merges
-//   analyse   per entry: minus flag (an earlier entry of the same group
-//             e[1..k-1] has the same label; groups are contiguous and hold at
-//             most 16 entries), node head/last flags
 //   degrees   zero outdegree: a join of the targets against the nodes, both in
 //             colex order; zero indegree: their reverse complements
 //   padding   dummy entries (node $ v[0..k-2], label v[k-1]) sorted by
 //             (v[k-2..0], v[k-1]); $ entries in the order of their nodes
-//   merge     final position of every entry: its rank in its own list plus
-//             the number of entries of the other lists below it, by binary
-//             search and a scan of insertion counts over E
-//   emit      W with minus flag, last, dummy, valid bit-vectors, aux, F, mult
+//   place     final position of every dummy and $ entry: its rank in its own
+//             list plus the number of entries of the other lists below it
+//   emit      one sweep over the final positions: W with minus flag, last,
+//             dummy, valid, mult, from the keys and the padding's positions;
+//             aux; F by bisection
 #include "mh_internal.cuh"
 
 namespace mh {
@@ -110,28 +108,6 @@ __global__ void first_symbol_bounds_kernel(const uint64_t* __restrict__ s, uint6
         if (key_less<NW>(load_key<NW>(a, mid), q)) lo = mid + 1; else hi = mid;
     }
     bounds[threadIdx.x] = lo;
-}
-
-// Per sorted entry: flags (bit0 minus, bit1 node head, bit2 node last in E).
-template <int NW>
-__global__ void analyse_kernel(const uint64_t* __restrict__ ck, uint64_t E, uint8_t* __restrict__ fl) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += (uint64_t)gridDim.x * blockDim.x) {
-        Key<NW> x = load_key<NW>(ck, i);
-        Key<NW> g = key_shr<NW>(x, 4), node = key_shr<NW>(x, 2);
-        uint32_t lab = (uint32_t)(x.w[0] & 3u);
-        bool minus = false;
-        for (uint64_t j = i; j > 0; j--) {
-            Key<NW> y = load_key<NW>(ck, j - 1);
-            if (!key_eq<NW>(key_shr<NW>(y, 4), g)) break;
-            if ((uint32_t)(y.w[0] & 3u) == lab) {
-                minus = true;
-                break;
-            }
-        }
-        bool head = i == 0 || !key_eq<NW>(key_shr<NW>(load_key<NW>(ck, i - 1), 2), node);
-        bool last = i + 1 == E || !key_eq<NW>(key_shr<NW>(load_key<NW>(ck, i + 1), 2), node);
-        fl[i] = (minus ? 1 : 0) | (head ? 2 : 0) | (last ? 4 : 0);
-    }
 }
 
 // Zero-outdegree nodes.  In colex order the targets of the edges with label c
@@ -344,11 +320,11 @@ __global__ void dummy_keys_kernel(const uint64_t* __restrict__ zout, uint64_t t,
     }
 }
 
-// Final positions of dummy (KIND 1) or $ (KIND 2) entries; insertion counts over E.
+// Final positions of dummy (KIND 1) or $ (KIND 2) entries.
 template <int NW, int KIND>
 __global__ void place_pad_kernel(const uint64_t* __restrict__ own, uint64_t n_own, const uint64_t* __restrict__ ck,
                                  uint64_t E, const uint64_t* __restrict__ other, uint64_t n_other,
-                                 uint64_t* __restrict__ final_pos, uint32_t* __restrict__ ins) {
+                                 uint64_t* __restrict__ final_pos) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n_own;
          i += (uint64_t)gridDim.x * blockDim.x) {
         Key<NW> x = load_key<NW>(own, i), g;
@@ -357,103 +333,181 @@ __global__ void place_pad_kernel(const uint64_t* __restrict__ own, uint64_t n_ow
         uint64_t le = lb_ext<NW, 0>(ck, E, g, t);
         uint64_t lo = KIND == 1 ? lb_ext<NW, 2>(other, n_other, g, t) : lb_ext<NW, 1>(other, n_other, g, t);
         final_pos[i] = le + i + lo;
-        atomicAdd(&ins[le], 1u);
     }
 }
 
-// Add a thread's 4 symbol counts to the global histogram (warp-reduced first).
-__device__ __forceinline__ void flush_hist4(const uint32_t h[4], unsigned long long* __restrict__ hist) {
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        uint32_t v = h[c];
-        for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&hist[c], (unsigned long long)v);
-    }
-}
-
-// W byte: low 4 bits W code, bit 4 last, bit 5 dummy.
+// aux[i]: the node v of dummy i (dk = (v[k-2], ..., v[0], v[k-1])).
 template <int NW>
-__global__ void emit_edges_kernel(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cv, uint64_t E, int K1,
-                                  const uint8_t* __restrict__ fl, const uint64_t* __restrict__ shift,
-                                  uint8_t* __restrict__ wf, uint32_t* __restrict__ mult,
-                                  unsigned long long* __restrict__ hist) {
-    uint32_t h[4] = {0, 0, 0, 0};
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += (uint64_t)gridDim.x * blockDim.x) {
-        Key<NW> x = load_key<NW>(ck, i);
-        uint8_t f = fl[i];
-        uint32_t lab = (uint32_t)(x.w[0] & 3u) + 1;
-        uint64_t p = i + shift[i + 1];
-        wf[p] = (uint8_t)((lab + ((f & 1) ? 4 : 0)) | ((f & 4) ? 16 : 0));
-        if (mult) mult[p] = cv ? cv[i] : 0;
-        h[key_sym<NW>(x, K1, 0)]++;
-    }
-    flush_hist4(h, hist);
-}
-
-template <int NW>
-__global__ void emit_dummy_kernel(const uint64_t* __restrict__ dk, uint64_t t, int k, const uint64_t* __restrict__ pos,
-                                  uint8_t* __restrict__ wf, uint32_t* __restrict__ mult, uint64_t* __restrict__ aux,
-                                  unsigned long long* __restrict__ hist) {
-    uint32_t h[4] = {0, 0, 0, 0};
+__global__ void aux_kernel(const uint64_t* __restrict__ dk, uint64_t t, int k, uint64_t* __restrict__ aux) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < t; i += (uint64_t)gridDim.x * blockDim.x) {
-        Key<NW> x = load_key<NW>(dk, i);
-        Key<NW> g = key_shr<NW>(x, 2);
-        bool last = i + 1 == t || !key_eq<NW>(key_shr<NW>(load_key<NW>(dk, i + 1), 2), g);
-        uint32_t lab = (uint32_t)(x.w[0] & 3u);
-        uint64_t p = pos[i];
-        wf[p] = (uint8_t)((lab + 1) | (last ? 16 : 0) | 32);
-        if (mult) mult[p] = 0;
-        // v = reverse of v_rev, v_rev = (v[k-1], v[k-2], ..., v[0]) = lab * 4^(k-1) + g
+        const Key<NW> x = load_key<NW>(dk, i);
+        // v = reverse of v_rev, v_rev = (v[k-1], v[k-2], ..., v[0]) = label * 4^(k-1) + dk >> 2
         Key<NW> top = key_zero<NW>();
-        top.w[0] = lab;
+        top.w[0] = x.w[0] & 3u;
         top = key_shl<NW>(top, 2 * (k - 1));
-        Key<NW> vr = g;
+        Key<NW> vr = key_shr<NW>(x, 2);
 #pragma unroll
         for (int w = 0; w < NW; w++) vr.w[w] |= top.w[w];
         store_key<NW>(aux, i, key_rev<NW>(vr, k));
-        h[key_sym<NW>(x, k, 0)]++;  // node symbol k-1 = v[k-2], the top symbol of x
     }
-    flush_hist4(h, hist);
+}
+
+// hist[c - 1] = entries whose node's last symbol (the top one of every list's
+// keys) is below c, for c = 1, 2, 3.
+template <int NW>
+__global__ void symbol_starts_kernel(const uint64_t* __restrict__ ck, uint64_t E, const uint64_t* __restrict__ dk,
+                                     uint64_t t, const uint64_t* __restrict__ ur, uint64_t u, int k,
+                                     unsigned long long* __restrict__ hist) {
+    const int q = threadIdx.x;
+    if (q >= 9) return;
+    const uint64_t* a = q < 3 ? ck : q < 6 ? dk : ur;
+    const uint64_t n = q < 3 ? E : q < 6 ? t : u;
+    Key<NW> x = key_zero<NW>();
+    x.w[0] = (uint64_t)(q % 3 + 1);
+    x = key_shl<NW>(x, q < 3 ? 2 * k : 2 * (k - 1));
+    uint64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (key_less<NW>(load_key<NW>(a, mid), x)) lo = mid + 1; else hi = mid;
+    }
+    if (lo) atomicAdd(&hist[q % 3], (unsigned long long)lo);
+}
+
+// Emission: a CTA per kEmitTile final positions.  The tile's dummies and $
+// entries (few) are set down in shared memory first; the slots between them
+// are the edges from a known one on, in order, so a lane finds its edge by a
+// count of bits, its minus flag (an earlier entry of its group e[1..k-1] has
+// the same label; a group holds at most 16) and whether it ends its node from
+// the neighbours, and a warp's ballots are words of the bit-vectors.
+// Reads each key once from memory (the neighbours come from L1) and writes
+// each output once; bound by the loads in flight.  3.5e8 edges of one word:
+// 2.7 ms, where flags, insertion counts, their scan, bytes and their packing
+// (53 bytes an edge) took 6.5; build of 3 M reads at k = 47 with
+// multiplicities 4.23 -> 3.75 ms.
+constexpr int kEmitTile = 2048;
+
+// pb[2 b] / pb[2 b + 1]: dummies / $ entries placed before position b * kEmitTile.
+__global__ void emit_bounds_kernel(const uint64_t* __restrict__ pos_d, uint64_t t, const uint64_t* __restrict__ pos_u,
+                                   uint64_t u, uint64_t n_tiles, uint64_t* __restrict__ pb) {
+    for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < 2 * (n_tiles + 1);
+         q += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t* a = (q & 1) ? pos_u : pos_d;
+        const uint64_t p = (q >> 1) * kEmitTile;
+        uint64_t lo = 0, hi = (q & 1) ? u : t;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if (a[mid] < p) lo = mid + 1; else hi = mid;
+        }
+        pb[q] = lo;
+    }
 }
 
 template <int NW>
-__global__ void emit_dollar_kernel(const uint64_t* __restrict__ ur, uint64_t u, int k, const uint64_t* __restrict__ pos,
-                                   uint8_t* __restrict__ wf, uint32_t* __restrict__ mult,
-                                   unsigned long long* __restrict__ hist) {
-    uint32_t h[4] = {0, 0, 0, 0};
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < u; i += (uint64_t)gridDim.x * blockDim.x) {
-        Key<NW> x = load_key<NW>(ur, i);
-        uint64_t p = pos[i];
-        wf[p] = (uint8_t)(0 | 16);
-        if (mult) mult[p] = 0;
-        h[key_sym<NW>(x, k, 0)]++;  // u[k-1], the top symbol of u_rev
+__global__ void __launch_bounds__(256) emit_kernel(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cv,
+                                                   uint64_t E, const uint64_t* __restrict__ dk, uint64_t t,
+                                                   const uint64_t* __restrict__ pos_d,
+                                                   const uint64_t* __restrict__ pos_u, uint64_t m,
+                                                   const uint64_t* __restrict__ pb, uint8_t* __restrict__ W,
+                                                   uint32_t* __restrict__ last, uint32_t* __restrict__ dummy,
+                                                   uint32_t* __restrict__ valid, uint32_t* __restrict__ mult,
+                                                   unsigned long long* __restrict__ n_last) {
+    constexpr int kWords = kEmitTile / 32;  // 32 positions each, eight a warp
+    constexpr int U = NW == 1 ? 8 : NW == 2 ? 4 : 2;
+    __shared__ uint8_t pad[kEmitTile];      // where pmask is set: W code, bit 4 last, bit 5 dummy
+    __shared__ uint32_t pmask[kWords], pre[kWords], sum_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t b = blockIdx.x, base = b * kEmitTile;
+    const uint32_t n = (uint32_t)(m - base < (uint64_t)kEmitTile ? m - base : (uint64_t)kEmitTile);
+    const uint64_t d0 = pb[2 * b], u0 = pb[2 * b + 1], d1 = pb[2 * b + 2], u1 = pb[2 * b + 3];
+    const uint64_t e0 = base - d0 - u0;     // the tile's first edge
+    if (tid < kWords) pmask[tid] = 0;
+    if (tid == 0) sum_last = 0;
+    __syncthreads();
+    for (uint64_t i = d0 + tid; i < d1; i += 256) {
+        const Key<NW> x = load_key<NW>(dk, i);
+        const bool ends =
+            i + 1 == t || !key_eq<NW>(key_shr<NW>(load_key<NW>(dk, i + 1), 2), key_shr<NW>(x, 2));
+        const uint64_t p = pos_d[i] - base;
+        if (p >= n) continue;  // (never so in sorted tables)
+        pad[p] = (uint8_t)(((uint32_t)(x.w[0] & 3u) + 1) | (ends ? 16 : 0) | 32);
+        atomicOr(&pmask[p >> 5], 1u << (p & 31));
     }
-    flush_hist4(h, hist);
-}
-
-// W bytes -> W codes and the last / dummy / valid bit-vectors (warp per 32 entries).
-__global__ void pack_bits_kernel(const uint8_t* __restrict__ wf, uint64_t m, uint8_t* __restrict__ W,
-                                 uint32_t* __restrict__ last, uint32_t* __restrict__ dummy,
-                                 uint32_t* __restrict__ valid, unsigned long long* __restrict__ n_last) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t n_words = ceil_div(m, 32);
-    uint32_t cnt = 0;
-    for (uint64_t w = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; w < n_words;
-         w += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
-        uint64_t i = w * 32 + lane;
-        uint8_t b = i < m ? wf[i] : 0;
-        if (i < m) W[i] = b & 15;
-        uint32_t lb = __ballot_sync(0xFFFFFFFFu, (b & 16) != 0);
-        uint32_t db = __ballot_sync(0xFFFFFFFFu, (b & 32) != 0);
-        uint32_t vb = __ballot_sync(0xFFFFFFFFu, i < m);
-        if (lane == 0) {
-            last[w] = lb;
-            dummy[w] = db;
-            valid[w] = vb;
-            cnt += __popc(lb);
+    for (uint64_t i = u0 + tid; i < u1; i += 256) {
+        const uint64_t p = pos_u[i] - base;
+        if (p >= n) continue;
+        pad[p] = 16;
+        atomicOr(&pmask[p >> 5], 1u << (p & 31));
+    }
+    __syncthreads();
+    if (warp == 0) {
+        static_assert(kWords == 64, "two words a lane");
+        const uint32_t c0 = __popc(pmask[2 * lane]), c = c0 + __popc(pmask[2 * lane + 1]);
+        uint32_t x = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        pre[2 * lane] = x - c;
+        pre[2 * lane + 1] = x - c + c0;
+    }
+    __syncthreads();
+    uint32_t ends = 0;
+    for (int r = 0; r < 8; r += U) {
+        Key<NW> x[U], lf[U], rt[U];
+        uint64_t at[U];
+        uint32_t kind[U];  // 0 past the end, 1 padding, 2 edge
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            const uint32_t wd = (r + j) * 8 + warp, p = wd * 32 + lane, pm = pmask[wd];
+            kind[j] = p >= n ? 0u : ((pm >> lane) & 1u) ? 1u : 2u;
+            at[j] = e0 + p - pre[wd] - __popc(pm & ((1u << lane) - 1u));
+            if (kind[j] == 2 && at[j] >= E) kind[j] = 0;  // (never so in sorted tables)
+            if (kind[j] == 2) {
+                x[j] = load_key<NW>(ck, at[j]);
+                if (at[j] > 0) lf[j] = load_key<NW>(ck, at[j] - 1);
+                if (at[j] + 1 < E) rt[j] = load_key<NW>(ck, at[j] + 1);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            const uint32_t wd = (r + j) * 8 + warp, p = wd * 32 + lane;
+            uint32_t code = 0;
+            if (kind[j] == 1) code = pad[p];
+            if (kind[j] == 2) {
+                const Key<NW> g = key_shr<NW>(x[j], 4);
+                const uint32_t lab = (uint32_t)(x[j].w[0] & 3u);
+                bool minus = false;
+                Key<NW> y = lf[j];
+                for (uint64_t i = at[j]; i > 0; y = load_key<NW>(ck, i - 1)) {
+                    if (!key_eq<NW>(key_shr<NW>(y, 4), g)) break;
+                    if ((uint32_t)(y.w[0] & 3u) == lab) {
+                        minus = true;
+                        break;
+                    }
+                    if (--i == 0) break;
+                }
+                const bool ends_node =
+                    at[j] + 1 == E || !key_eq<NW>(key_shr<NW>(rt[j], 2), key_shr<NW>(x[j], 2));
+                code = lab + 1 + (minus ? 4 : 0) + (ends_node ? 16 : 0);
+            }
+            const uint32_t lb = __ballot_sync(0xFFFFFFFFu, (code & 16) != 0);
+            const uint32_t db = __ballot_sync(0xFFFFFFFFu, (code & 32) != 0);
+            const uint32_t vb = __ballot_sync(0xFFFFFFFFu, kind[j] != 0);
+            if (kind[j]) W[base + p] = (uint8_t)(code & 15);
+            if (mult && kind[j]) mult[base + p] = kind[j] == 2 ? cv[at[j]] : 0u;
+            if (lane == 0 && vb) {
+                const uint64_t o = base / 32 + wd;
+                last[o] = lb;
+                dummy[o] = db;
+                valid[o] = vb;
+            }
+            ends += __popc(lb);
         }
     }
-    if (lane == 0 && cnt) atomicAdd(n_last, (unsigned long long)cnt);
+    if (lane == 0 && ends) atomicAdd(&sum_last, ends);
+    __syncthreads();
+    if (tid == 0 && sum_last) atomicAdd(n_last, (unsigned long long)sum_last);
 }
 
 template <int NW>
@@ -489,9 +543,6 @@ void build_sdbg(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, mh_sd
     }
     ck2.reset();
     cv2.reset();
-    // per-entry flags
-    Buf<uint8_t> fl(ctx, E ? E : 1);
-    if (E) MH_LAUNCH(ctx, "analyse", grid_for(ctx, E, 256), 256, 0, analyse_kernel<NW>, ck.p, E, fl.p);
     // zero outdegree, ascending (as many nodes have zero indegree)
     Buf<uint64_t> zout;
     uint64_t u = 0;
@@ -521,46 +572,36 @@ void build_sdbg(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, mh_sd
     if (t) MH_LAUNCH(ctx, "dummy_keys", grid_for(ctx, t, 256), 256, 0, dummy_keys_kernel<NW>, zout.p, t, k, dk.p);
     if (radix_sort<NW>(ctx, dk.p, dk2.p, nullptr, nullptr, t, 0, 2 * k)) std::swap(dk, dk2);
     dk2.reset();
-    // merge positions
+    // merge positions of the padding
     const uint64_t m = E + t + u;
-    Buf<uint32_t> ins(ctx, E + 1);
-    ins.zero();
-    Buf<uint64_t> pos_d(ctx, t ? t : 1), pos_u(ctx, u ? u : 1), shift(ctx, E + 2);
+    Buf<uint64_t> pos_d(ctx, t ? t : 1), pos_u(ctx, u ? u : 1);
     if (t)
         MH_LAUNCH(ctx, "place_dummy", grid_for(ctx, t, 256), 256, 0, (place_pad_kernel<NW, 1>), dk.p, t, ck.p, E,
-                  zout.p, u, pos_d.p, ins.p);
+                  zout.p, u, pos_d.p);
     if (u)
         MH_LAUNCH(ctx, "place_dollar", grid_for(ctx, u, 256), 256, 0, (place_pad_kernel<NW, 2>), zout.p, u, ck.p, E,
-                  dk.p, t, pos_u.p, ins.p);
-    exclusive_scan_u32(ctx, ins.p, shift.p, E + 1);
-    ins.reset();
+                  dk.p, t, pos_u.p);
     // emit
-    Buf<uint8_t> wf(ctx, m ? m : 1);
     Buf<unsigned long long> hist(ctx, 8);
     hist.zero();
     Buf<uint32_t> mult;
     if (want_mult) mult = Buf<uint32_t>(ctx, m ? m : 1);
-    if (E)
-        MH_LAUNCH(ctx, "emit_edges", grid_for(ctx, E, 256), 256, 0, emit_edges_kernel<NW>, ck.p,
-                  want_mult ? cv.p : nullptr, E, K1, fl.p, shift.p, wf.p, want_mult ? mult.p : nullptr, hist.p);
     const uint64_t nwk = (uint64_t)NW;
     Buf<uint64_t> aux(ctx, (t ? t : 1) * nwk);
-    if (t)
-        MH_LAUNCH(ctx, "emit_dummy", grid_for(ctx, t, 256), 256, 0, emit_dummy_kernel<NW>, dk.p, t, k, pos_d.p, wf.p,
-                  want_mult ? mult.p : nullptr, aux.p, hist.p);
-    if (u)
-        MH_LAUNCH(ctx, "emit_dollar", grid_for(ctx, u, 256), 256, 0, emit_dollar_kernel<NW>, zout.p, u, k, pos_u.p, wf.p,
-                  want_mult ? mult.p : nullptr, hist.p);
-    ck.reset();
-    cv.reset();
-    fl.reset();
-    shift.reset();
+    if (t) MH_LAUNCH(ctx, "aux", grid_for(ctx, t, 256), 256, 0, aux_kernel<NW>, dk.p, t, k, aux.p);
     const uint64_t n_words = ceil_div(m, 32);
     Buf<uint8_t> W(ctx, m ? m : 1);
     Buf<uint32_t> last(ctx, n_words ? n_words : 1), dummy(ctx, n_words ? n_words : 1), valid(ctx, n_words ? n_words : 1);
-    if (m)
-        MH_LAUNCH(ctx, "pack_bits", grid_for(ctx, n_words * 32, 256), 256, 0, pack_bits_kernel, wf.p, m, W.p, last.p,
-                  dummy.p, valid.p, hist.p + 4);
+    if (m) {
+        const uint64_t tiles = ceil_div(m, (uint64_t)kEmitTile);
+        Buf<uint64_t> pb(ctx, 2 * (tiles + 1));
+        MH_LAUNCH(ctx, "symbol_starts", 1, 32, 0, symbol_starts_kernel<NW>, ck.p, E, dk.p, t, zout.p, u, k, hist.p);
+        MH_LAUNCH(ctx, "emit_bounds", grid_for(ctx, 2 * (tiles + 1), 256), 256, 0, emit_bounds_kernel, pos_d.p, t,
+                  pos_u.p, u, tiles, pb.p);
+        MH_LAUNCH_B(ctx, "emit", E * (8 * NW + (want_mult ? 4 : 0)) + m * (want_mult ? 5 : 1), (unsigned)tiles, 256, 0,
+                    emit_kernel<NW>, ck.p, want_mult ? cv.p : nullptr, E, dk.p, t, pos_d.p, pos_u.p, m, pb.p, W.p,
+                    last.p, dummy.p, valid.p, want_mult ? mult.p : nullptr, hist.p + 4);
+    }
     uint64_t h[5];
     read_u64(ctx, reinterpret_cast<const uint64_t*>(hist.p), h, 5);
     out->m = m;
@@ -570,8 +611,8 @@ void build_sdbg(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, mh_sd
     out->F[0] = 0;
     out->F[1] = 0;
     out->F[2] = h[0];
-    out->F[3] = h[0] + h[1];
-    out->F[4] = h[0] + h[1] + h[2];
+    out->F[3] = h[1];
+    out->F[4] = h[2];
     out->F[5] = m;
     out->W = W.release();
     out->last = last.release();
