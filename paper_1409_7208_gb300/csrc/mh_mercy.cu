@@ -13,15 +13,12 @@
 //   ends     the edges with out0 or in0 (the graph's dead ends, a small
 //            fraction of S) go into a small open-addressing hash table with
 //            their two flags, which stays in L2.
-//   probe    fragments in groups of 32 a warp (a lane per short fragment,
-//            its window rolled on; a long fragment by the whole warp, a
-//            window a lane): a test of three bits
-//            of one word in a blocked Bloom filter of the edges without
-//            outdegree (about 8 bits per dead end), and for the few
-//            positives a probe of the small table;
-//            every window p without outdegree is recorded as a hit (its
-//            position and the end of its fragment).
-//   walk     thread per hit: step forward to the next solid window q; if
+//   probe    every window against a blocked Bloom filter of the edges without
+//            outdegree, four windows a lookup by the symbols they share, and
+//            the few positives against the small table; every window p
+//            without outdegree is recorded as a hit (its position and the end
+//            of its fragment).
+//   walk     a few lanes per hit: step forward to the next solid window q; if
 //            q > p+1 and q has no indegree, the windows p+1..q-1 are emitted
 //            (canonical keys).  Solidity: a search of the counting spectrum
 //            (distinct canonical keys, ascending as mix_key images, so their
@@ -190,11 +187,22 @@ __global__ void degree_flags_kernel(const uint8_t* __restrict__ fout, uint8_t* _
 }
 
 // Prefilter of the edges without outdegree: a blocked Bloom filter, three
-// bits of one 32-bit word per key, so a query is one load; about 5% false
-// positives at 8 bits per key.  Its hash is one multiply per key word (the
-// filter is probed for every read window; the table keeps key_hash): the
-// word comes from the product's top 32 bits, the bit positions from three
-// 5-bit fields of its middle bits.
+// bits of one 32-bit word per key, so a query is one load.  Its hash is one
+// multiply per key word (the table keeps key_hash): the word comes from the
+// product's top 32 bits, the bit positions from three 5-bit fields of its
+// middle bits.
+//
+// Four neighbouring windows of a read share K1 - 3 symbols, their core, and
+// an edge is the j-th of such a group with its symbols [3 - j, K1 - j) as the
+// core, j = 0..3.  So the filter holds every edge's four cores beside the
+// edge itself: a group is looked up once, and only the groups it lets
+// through (some 5% and the true ones) a window each.  At least 24 bits per dead
+// end, of which about half have no outdegree: 4.8 to 19 bits a key.
+constexpr int kProbeGroup = 4;
+template <int NW>
+__device__ __forceinline__ Key<NW> probe_core(const Key<NW>& x, int j, int K1) {
+    return key_low<NW>(key_shr<NW>(x, 2 * j), 2 * (K1 - kProbeGroup + 1));
+}
 template <int NW>
 __device__ __forceinline__ uint64_t filter_hash(const Key<NW>& x) {
     uint64_t h = x.w[0] * 0x9E3779B97F4A7C15ull;
@@ -208,30 +216,62 @@ __device__ __forceinline__ uint32_t filter_bits(uint64_t h) {
 }
 
 // Dead-end edges (oriented) with their flags into the small table; edges
-// without outdegree also into the prefilter bitmap.
+// without outdegree also into the prefilter.  A CTA lists the flagged entries
+// of a tile first (a few in a hundred), so that its lanes wait for their
+// insertions' round trips to memory together: 3.5e8 edges 3.5 -> 0.3 ms.
+constexpr int kEndsTile = 4096;
 template <int NW>
-__global__ void __launch_bounds__(256) ends_insert_kernel(const uint64_t* __restrict__ S, uint64_t n,
+__global__ void __launch_bounds__(256) ends_insert_kernel(const uint64_t* __restrict__ S, uint64_t n, int K1,
                                                           const uint8_t* __restrict__ flags,
                                                           Slot<NW>* __restrict__ table, uint64_t cap_mask,
                                                           uint32_t* __restrict__ filter, uint64_t filter_mask,
                                                           uint32_t* __restrict__ err) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        uint8_t f = flags[i];
-        if (!f) continue;
-        Key<NW> x = load_key<NW>(S, i);
-        uint64_t h = key_hash<NW>(x);
-        if (f & 1u) {
-            const uint64_t fh = filter_hash<NW>(x);
+    __shared__ uint16_t list[kEndsTile];  // entry << 2 | flags (14 bits)
+    __shared__ uint32_t scratch[8];
+    const uint64_t base = blockIdx.x * (uint64_t)kEndsTile;
+    const uint32_t i0 = threadIdx.x * 16;
+    uint32_t f[4] = {0, 0, 0, 0};
+    if (base + i0 + 16 <= n) {
+        const uint4 v = *reinterpret_cast<const uint4*>(flags + base + i0);
+        f[0] = v.x;
+        f[1] = v.y;
+        f[2] = v.z;
+        f[3] = v.w;
+    } else {
+        for (uint32_t j = 0; j < 16; j++)
+            if (base + i0 + j < n) f[j >> 2] |= (uint32_t)flags[base + i0 + j] << (8 * (j & 3));
+    }
+    uint32_t mine = 0, total;
+#pragma unroll
+    for (int j = 0; j < 16; j++) mine += ((f[j >> 2] >> (8 * (j & 3))) & 3u) != 0;
+    uint32_t at = block_excl_scan_256(mine, scratch, &total);
+#pragma unroll
+    for (int j = 0; j < 16; j++) {
+        const uint32_t g = (f[j >> 2] >> (8 * (j & 3))) & 3u;
+        if (g) list[at++] = (uint16_t)((i0 + j) << 2 | g);
+    }
+    __syncthreads();
+    for (uint32_t e = threadIdx.x; e < total; e += 256) {
+        const uint32_t fl = list[e] & 3u;
+        const Key<NW> x = load_key<NW>(S, base + (list[e] >> 2));
+        if (fl & 1u) {
+            uint64_t fh = filter_hash<NW>(x);
             atomicOr(&filter[filter_word(fh, filter_mask)], filter_bits(fh));
+#pragma unroll
+            for (int j = 0; j < kProbeGroup; j++) {
+                fh = filter_hash<NW>(probe_core<NW>(x, j, K1));
+                atomicOr(&filter[filter_word(fh, filter_mask)], filter_bits(fh));
+            }
         }
-        uint32_t tag = slot_tag(h);
+        const uint64_t h = key_hash<NW>(x);
+        const uint32_t tag = slot_tag(h);
         uint64_t s = h & cap_mask;
         bool placed = false;
         for (uint64_t probe = 0; probe <= cap_mask; probe++) {
             if (atomicCAS(&table[s].tag, 0u, tag) == 0u) {
 #pragma unroll
                 for (int w = 0; w < NW; w++) table[s].k[w] = x.w[w];
-                table[s].flags = f;
+                table[s].flags = fl;
                 placed = true;
                 break;
             }
@@ -341,90 +381,122 @@ __device__ __forceinline__ bool table_has(const Slot<NW>* __restrict__ table, ui
     return false;
 }
 
-// Fragments of at most this many windows are probed by one lane.
-constexpr int kProbeLaneWindows = 48;
-
 // Probe every window; record windows without outdegree as (position, end).
-// Fragments in groups of 32 a warp: a short fragment is probed by one lane,
-// which assembles its first window and rolls it on by one symbol a window
-// (the lanes step together to the group's longest short fragment, so that
-// the hits of a step are counted by one atomic); longer fragments are then
-// probed by the whole warp, a window a lane.
+// A warp takes up to 32 fragments and numbers their groups of four windows through,
+// a group a lane and step: its core is the end of its first window.  The
+// groups the filter lets through queue in shared memory until eight of them
+// give every lane one window to look up.  Bound by the random filter reads (a
+// line of L1 a lane): four windows a lookup took 2.38e9 windows from 9.3 to
+// 3.7 ms, 3 M reads at k = 31 from 1.27 to 0.56.
 template <int NW>
 __global__ void __launch_bounds__(256) mercy_probe_kernel(const uint32_t* __restrict__ packed,
                                                           const uint64_t* __restrict__ frag_offs, uint64_t n_frags,
-                                                          int k, const Slot<NW>* __restrict__ ends, uint64_t cap_mask,
-                                                          const uint32_t* __restrict__ filter, uint64_t filter_mask,
-                                                          ulonglong2* __restrict__ hits, uint64_t hit_cap,
-                                                          unsigned long long* __restrict__ n_hits) {
-    const int lane = threadIdx.x & 31;
+                                                          int take_frags, int k, const Slot<NW>* __restrict__ ends,
+                                                          uint64_t cap_mask, const uint32_t* __restrict__ filter,
+                                                          uint64_t filter_mask, ulonglong2* __restrict__ hits,
+                                                          uint64_t hit_cap, unsigned long long* __restrict__ n_hits) {
+    constexpr int G = kProbeGroup, B = 32 / G;
+    __shared__ ulonglong2 frags[8][32];      // first group's position less G x its number; end of the windows
+    __shared__ ulonglong2 queue[8][32 + B];  // groups let through: position, end of the windows
+    __shared__ uint64_t starts[8][32];       // number of the fragment's first group
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
     const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const int K1 = k + 1;
-    auto probe = [&](const Key<NW>& x) {
+    auto in_filter = [&](const Key<NW>& x) {
         const uint64_t h = filter_hash<NW>(x);
         const uint32_t fm = filter_bits(h);
-        return (__ldg(&filter[filter_word(h, filter_mask)]) & fm) == fm && (ends_find<NW>(ends, cap_mask, x) & 1u);
+        return (__ldg(&filter[filter_word(h, filter_mask)]) & fm) == fm;
     };
-    // the hits of one step of the warp, placed by one atomic
-    auto record = [&](bool hit, uint64_t p, uint64_t end) {
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
-        if (!m) return;
-        uint64_t first = 0;
-        if (lane == __ffs(m) - 1) first = atomicAdd(n_hits, (unsigned long long)__popc(m));
-        first = __shfl_sync(0xFFFFFFFFu, first, __ffs(m) - 1);
-        if (hit) {
-            const uint64_t idx = first + __popc(m & ((1u << lane) - 1));
-            if (idx < hit_cap) hits[idx] = make_ulonglong2(p, end);
+    // the last B groups (or fewer) of the queue's n: a window a lane, their
+    // hits placed by one atomic
+    auto probe = [&](uint32_t n) {
+        const uint32_t take = n < (uint32_t)B ? n : (uint32_t)B, e = lane / G;
+        bool hit = false;
+        uint64_t p = 0, end = 0;
+        if (e < take) {
+            const ulonglong2 q = queue[wid][n - take + e];
+            p = q.x + lane % G;
+            end = q.y;
+            if (p < end) {
+                const Key<NW> x = load_window<NW>(packed, p, K1);
+                hit = in_filter(x) && (ends_find<NW>(ends, cap_mask, x) & 1u);
+            }
         }
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
+        if (m) {
+            uint64_t first = 0;
+            if (lane == 0) first = atomicAdd(n_hits, (unsigned long long)__popc(m));
+            first = __shfl_sync(0xFFFFFFFFu, first, 0);
+            const uint64_t idx = first + __popc(m & lt);
+            if (hit && idx < hit_cap) hits[idx] = make_ulonglong2(p, end);
+        }
+        __syncwarp();
+        return n - take;
     };
-    for (uint64_t g = warp; g * 32 < n_frags; g += n_warps) {
-        const uint64_t f = g * 32 + lane;
+    uint32_t queued = 0;
+    for (uint64_t g = warp; g * take_frags < n_frags; g += n_warps) {
+        const uint64_t f = g * take_frags + lane;
         uint64_t b = 0, nwin = 0;
-        if (f < n_frags) {
+        if (lane < take_frags && f < n_frags) {
             b = frag_offs[f];
             const uint64_t L = frag_offs[f + 1] - b;
             nwin = L > (uint64_t)k ? L - k : 0;
         }
-        const bool alone = nwin <= (uint64_t)kProbeLaneWindows;
-        const uint64_t mine = alone ? nwin : 0;
-        uint64_t most = mine;
-        for (int off = 16; off; off >>= 1) {
-            const uint64_t o = __shfl_xor_sync(0xFFFFFFFFu, most, off);
-            most = o > most ? o : most;
+        const uint64_t mine = (nwin + G - 1) / G;
+        uint64_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += y;
         }
-        Key<NW> x{};
-        if (mine) x = load_window<NW>(packed, b, K1);
-        for (uint64_t i = 0; i < most; i++) {
-            bool hit = false;
-            if (i < mine) {
-                if (i) roll_forward<NW>(x, packed_sym(packed, b + i + K1 - 1), K1);
-                hit = probe(x);
+        const uint64_t tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        // the fragments that have windows, side by side
+        const uint32_t some = __ballot_sync(0xFFFFFFFFu, mine != 0);
+        if (mine) {
+            const int r = __popc(some & lt);
+            starts[wid][r] = incl - mine;
+            frags[wid][r] = make_ulonglong2(b - G * (incl - mine), b + nwin);
+        }
+        __syncwarp();
+        const uint64_t start = lane < __popc(some) ? starts[wid][lane] : ~0ull;
+        uint32_t before = 0;
+        for (uint64_t j0 = 0; j0 < tot; j0 += 32) {
+            // the fragment of group j0 + lane: the last one that starts at or before it
+            const uint64_t rel = start - j0;
+            const uint32_t m = __reduce_or_sync(0xFFFFFFFFu, rel < 32u ? 1u << (uint32_t)rel : 0u);
+            const uint32_t idx = before + __popc(m & (0xFFFFFFFFu >> (31 - lane))) - 1;
+            before += __popc(m);
+            bool pass = false;
+            ulonglong2 q = make_ulonglong2(0, 0);
+            if (j0 + lane < tot) {
+                q = frags[wid][idx];
+                q.x += G * (j0 + lane);
+                pass = in_filter(probe_core<NW>(load_window<NW>(packed, q.x, K1), 0, K1));
             }
-            record(hit, b + i, b + mine);
+            const uint32_t pm = __ballot_sync(0xFFFFFFFFu, pass);
+            if (pass) queue[wid][queued + __popc(pm & lt)] = q;
+            __syncwarp();
+            queued += __popc(pm);
+            while (queued >= (uint32_t)B) queued = probe(queued);
         }
-        uint32_t big = __ballot_sync(0xFFFFFFFFu, !alone);
-        while (big) {
-            const int src = __ffs(big) - 1;
-            big &= big - 1;
-            const uint64_t fb = __shfl_sync(0xFFFFFFFFu, b, src);
-            const uint64_t fn = __shfl_sync(0xFFFFFFFFu, nwin, src);
-            for (uint64_t base = 0; base < fn; base += 32) {
-                const uint64_t p = base + lane;
-                bool hit = false;
-                if (p < fn) hit = probe(load_window<NW>(packed, fb + p, K1));
-                record(hit, fb + p, fb + fn);
-            }
-        }
+        __syncwarp();
     }
+    if (queued) probe(queued);
 }
 
 // Walk from each hit to the next solid window; emit the gap if it qualifies.
+// G lanes a hit look G windows up at a time: a lookup is a chain of
+// dependent reads, and an error makes K1 windows in a row unsolid.  3 Gbp at
+// k = 31 3.9 ms with a lane a hit; 2.79, 2.55, 2.49 and 2.63 with 4, 8, 16 and
+// 32; one job's 450 k reads 0.48, and 0.17, 0.12, 0.09 and 0.08.
 // SOL 1 and 2: candidates out as mix_key images, solidity from the counting
 // spectrum (run length, doubled for a palindrome, >= d) through its bucket
 // index (1) or its super-k-mer bins (2); SOL 0 (unmixed handles): from the
 // hash set `solid`.
-template <int NW, int SOL>
+constexpr int kWalkLanes = 16;
+template <int NW, int SOL, int G>
 __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restrict__ packed,
                                                          const ulonglong2* __restrict__ hits, uint64_t n_hits, int k,
                                                          const Slot<NW>* __restrict__ ends, uint64_t ends_mask,
@@ -434,33 +506,43 @@ __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restr
                                                          const uint64_t* __restrict__ spec_off, int spec_bits,
                                                          SuperIndex super, int d, uint64_t* __restrict__ out, uint64_t out_cap,
                                                          unsigned long long* __restrict__ counter) {
-    const int K1 = k + 1;
-    for (uint64_t h = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; h < n_hits;
-         h += (uint64_t)gridDim.x * blockDim.x) {
+    const int K1 = k + 1, lane = threadIdx.x & 31, gl = lane % G;
+    const uint32_t group = (G == 32 ? 0xFFFFFFFFu : ((1u << (G & 31)) - 1u)) << (lane - gl);
+    for (uint64_t h = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / G; h < n_hits;
+         h += (uint64_t)gridDim.x * blockDim.x / G) {
         const ulonglong2 hp = hits[h];
         const uint64_t p = hp.x, end = hp.y;
-        uint64_t q = p + 1;
-        Key<NW> y;
-        for (; q < end; q++) {
-            Key<NW> x = load_window<NW>(packed, q, K1);
-            Key<NW> r = key_rc<NW>(x, K1);
-            const Key<NW> c = key_less<NW>(r, x) ? r : x;
-            bool present;
-            if constexpr (SOL != 0) {
-                const uint32_t len = SOL == 2 ? super_find<NW>(super, spec, spec_len, x, r, mix_key<NW>(c), K1)
-                                              : spec_find<NW>(spec, spec_len, spec_off, spec_bits, mix_key<NW>(c));
-                present = (uint64_t)len * (key_eq<NW>(r, x) ? 2 : 1) >= (uint64_t)d;
-            } else
-                present = table_has<NW>(solid, solid_mask, c);
-            if (present) {
-                y = x;
+        uint64_t q = end;
+        bool closes = false;  // window q has no indegree
+        for (uint64_t q0 = p + 1; q0 < end; q0 += G) {
+            const uint64_t mine = q0 + gl;
+            bool present = false;
+            Key<NW> x;
+            if (mine < end) {
+                x = load_window<NW>(packed, mine, K1);
+                const Key<NW> r = key_rc<NW>(x, K1);
+                const Key<NW> c = key_less<NW>(r, x) ? r : x;
+                if constexpr (SOL != 0) {
+                    const uint32_t len = SOL == 2 ? super_find<NW>(super, spec, spec_len, x, r, mix_key<NW>(c), K1)
+                                                  : spec_find<NW>(spec, spec_len, spec_off, spec_bits, mix_key<NW>(c));
+                    present = (uint64_t)len * (key_eq<NW>(r, x) ? 2 : 1) >= (uint64_t)d;
+                } else
+                    present = table_has<NW>(solid, solid_mask, c);
+            }
+            const uint32_t m = __ballot_sync(group, present);
+            if (m) {
+                const int src = __ffs(m) - 1;
+                q = q0 + (src - (lane - gl));
+                const bool none = lane == src && (ends_find<NW>(ends, ends_mask, x) & 2u);
+                closes = __ballot_sync(group, none) != 0;
                 break;
             }
         }
-        if (q >= end || q == p + 1) continue;
-        if (!(ends_find<NW>(ends, ends_mask, y) & 2u)) continue;
-        uint64_t idx = atomicAdd(counter, (unsigned long long)(q - p - 1));
-        for (uint64_t j = p + 1; j < q; j++, idx++) {
+        if (!closes || q == p + 1) continue;
+        uint64_t idx = 0;
+        if (gl == 0) idx = atomicAdd(counter, (unsigned long long)(q - p - 1));
+        idx = __shfl_sync(group, idx, lane - gl) + gl;
+        for (uint64_t j = p + 1 + gl; j < q; j += G, idx += G) {
             if (idx >= out_cap) continue;
             Key<NW> z = load_window<NW>(packed, j, K1);
             Key<NW> rz = key_rc<NW>(z, K1);
@@ -500,13 +582,13 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     const uint64_t cap = next_pow2(std::max<uint64_t>(2 * n_ends, 64));
     Buf<Slot<NW>> table(ctx, cap);
     table.zero();
-    // prefilter: about 8 bits per dead end (at least 2^20 bits)
-    const uint64_t fbits = next_pow2(std::max<uint64_t>(8 * n_ends, 1u << 20));
+    // prefilter: at least 24 bits per dead end and 2^20 in all
+    const uint64_t fbits = next_pow2(std::max<uint64_t>(24 * n_ends, 1u << 20));
     Buf<uint32_t> filter(ctx, fbits / 32);
     filter.zero();
     if (n_ends)
-        MH_LAUNCH(ctx, "mercy_ends_insert", grid_for(ctx, S, 256), 256, 0, ends_insert_kernel<NW>, solid->keys, S,
-                  flags.p, table.p, cap - 1, filter.p, fbits / 32 - 1, ctx->d_status);
+        MH_LAUNCH(ctx, "mercy_ends_insert", (unsigned)ceil_div(S, (uint64_t)kEndsTile), 256, 0, ends_insert_kernel<NW>,
+                  solid->keys, S, k + 1, flags.p, table.p, cap - 1, filter.p, fbits / 32 - 1, ctx->d_status);
     flags.reset();
     // solidity: the counting handle's ascending mixed spectrum with a bucket
     // index (4 to 8 keys a bucket); without one, a hash set of the canonical
@@ -538,14 +620,18 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     }
     // windows without outdegree
     uint64_t hit_cap = std::max<uint64_t>(1u << 20, reads->n_packed / 256);
+    // (few fragments: fewer a warp, so that there are warps for every SM)
+    const int take_frags =
+        (int)std::max<uint64_t>(4, std::min<uint64_t>(32, reads->n_frags / ((uint64_t)ctx->num_sms * 64)));
     Buf<ulonglong2> hits;
     uint64_t n_hits = 0;
     for (int attempt = 0; attempt < 2; attempt++) {
         hits = Buf<ulonglong2>(ctx, hit_cap);
         MH_CUDA(cudaMemsetAsync(stats.p + 1, 0, sizeof(uint64_t), ctx->stream));
         if (reads->n_frags && n_ends)
-            MH_LAUNCH_B(ctx, "mercy_probe", reads->n_packed / 4, grid_for(ctx, reads->n_frags * 32, 256, 8), 256, 0,
-                        mercy_probe_kernel<NW>, reads->packed, reads->frag_offs, reads->n_frags, k, table.p, cap - 1,
+            MH_LAUNCH_B(ctx, "mercy_probe", reads->n_packed / 4,
+                        grid_for(ctx, ceil_div(reads->n_frags, (uint64_t)take_frags) * 32, 256, 8), 256, 0,
+                        mercy_probe_kernel<NW>, reads->packed, reads->frag_offs, reads->n_frags, take_frags, k, table.p, cap - 1,
                         filter.p, fbits / 32 - 1, hits.p, hit_cap, (unsigned long long*)(stats.p + 1));
         read_u64(ctx, stats.p + 1, &n_hits, 1);
         if (n_hits <= hit_cap) break;
@@ -555,14 +641,16 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     // candidates in the spectrum's order (mix_key images), so that their
     // sorted spectrum lookups ascend
     uint64_t out_cap = std::max<uint64_t>(1u << 20, 16 * n_hits);
+    const auto walk = super   ? mercy_walk_kernel<NW, 2, kWalkLanes>
+                      : mixed ? mercy_walk_kernel<NW, 1, kWalkLanes>
+                              : mercy_walk_kernel<NW, 0, kWalkLanes>;
     Buf<uint64_t> cand;
     uint64_t n_cand = 0;
     for (int attempt = 0; attempt < 2; attempt++) {
         cand = Buf<uint64_t>(ctx, out_cap * NW);
         MH_CUDA(cudaMemsetAsync(stats.p + 1, 0, sizeof(uint64_t), ctx->stream));
         if (n_hits)
-            MH_LAUNCH(ctx, "mercy_walk", grid_for(ctx, n_hits, 256, 8), 256, 0,
-                      (super ? mercy_walk_kernel<NW, 2> : mixed ? mercy_walk_kernel<NW, 1> : mercy_walk_kernel<NW, 0>), reads->packed,
+            MH_LAUNCH(ctx, "mercy_walk", grid_for(ctx, n_hits * kWalkLanes, 256, 8), 256, 0, walk, reads->packed,
                       hits.p, n_hits, k, table.p, cap - 1, sset.p, scap - 1, solid->spectrum, solid->spectrum_len,
                       spec_off.p, spec_bits, sx, solid->d,
                       cand.p, out_cap, (unsigned long long*)(stats.p + 1));
