@@ -117,7 +117,7 @@ __global__ void first_symbol_bounds_kernel(const uint64_t* __restrict__ s, uint6
 // shared memory, the four ranges are streamed past them, and a node c.g
 // clears label c of group g: what is left are targets that no edge leaves.
 // Reads every key twice and writes next to nothing; bound by the searches in
-// shared memory.  3.5e8 edges of one word: 4.9 ms, where writing the sorted
+// shared memory.  3.5e8 edges of one word: 4.4 ms, where writing the sorted
 // nodes and targets, one radix pass and the merge of their differences took
 // 12.6.
 template <int NW>
@@ -171,8 +171,12 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
                                                        unsigned long long* __restrict__ n_found) {
     using Z = ZeroTile<NW>;
     constexpr int I = Z::kItems;
-    __shared__ __align__(16) uint64_t gk[Z::kCap * NW];  // the groups
-    __shared__ uint32_t gm[Z::kCap];        // labels left
+    // (one place of padding after kItems: a thread's entries, and so the
+    // groups its neighbours search and walk, lie about kItems apart)
+    constexpr int kPadded = Z::kCap / I * (I + 1);
+    __shared__ __align__(16) uint64_t gk[kPadded * NW];  // the groups
+    __shared__ uint32_t gm[kPadded];                     // labels left
+    auto at_pad = [](uint32_t i) { return i + i / I; };
     __shared__ uint32_t scratch[8];
     __shared__ uint64_t wsum[8], base;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -182,7 +186,7 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
     Key<NW> x[I];
     uint32_t heads = 0;
     const uint32_t i0 = tid * I;
-    for (int j = 0; j < I; j++) gm[i0 + j] = 0;
+    for (int j = 0; j < I; j++) gm[at_pad(i0 + j)] = 0;
     {
         Key<NW> prev = key_zero<NW>();
         if (i0 > 0 && i0 < n) prev = load_key<NW>(ck, s0 + i0 - 1);
@@ -201,8 +205,8 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
 #pragma unroll
     for (int j = 0; j < I; j++) {
         if (i0 + j >= n) continue;
-        if ((heads >> j) & 1u) store_key<NW>(gk, g++, key_shr<NW>(x[j], 4));
-        atomicOr(&gm[g - 1], 1u << (uint32_t)(x[j].w[0] & 3u));
+        if ((heads >> j) & 1u) store_key<NW>(gk, at_pad(g++), key_shr<NW>(x[j], 4));
+        atomicOr(&gm[at_pad(g - 1)], 1u << (uint32_t)(x[j].w[0] & 3u));
     }
     __syncthreads();
     // the nodes with first symbol c: two warps a label, I entries a thread,
@@ -220,14 +224,14 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
                 uint32_t hi = ng;
                 while (p < hi) {
                     const uint32_t mid = (p + hi) >> 1;
-                    if (key_less<NW>(load_key<NW>(gk, mid), y[0])) p = mid + 1; else hi = mid;
+                    if (key_less<NW>(load_key<NW>(gk, at_pad(mid)), y[0])) p = mid + 1; else hi = mid;
                 }
             }
 #pragma unroll
             for (int j = 0; j < I; j++) {
                 if (q + j >= b1 || (j && key_eq<NW>(y[j], y[j > 0 ? j - 1 : 0]))) continue;
-                while (p < ng && key_less<NW>(load_key<NW>(gk, p), y[j])) p++;
-                if (p < ng && key_eq<NW>(load_key<NW>(gk, p), y[j])) atomicAnd(&gm[p], ~(1u << c));
+                while (p < ng && key_less<NW>(load_key<NW>(gk, at_pad(p)), y[j])) p++;
+                if (p < ng && key_eq<NW>(load_key<NW>(gk, at_pad(p)), y[j])) atomicAnd(&gm[at_pad(p)], ~(1u << c));
             }
         }
     }
@@ -237,7 +241,7 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
     uint32_t m[I];
 #pragma unroll
     for (int j = 0; j < I; j++) {
-        m[j] = i0 + j < ng ? gm[i0 + j] : 0u;
+        m[j] = i0 + j < ng ? gm[at_pad(i0 + j)] : 0u;
 #pragma unroll
         for (int c = 0; c < 4; c++) mine += (uint64_t)((m[j] >> c) & 1u) << (16 * c);
     }
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
                 Key<NW> v = key_zero<NW>();
                 v.w[0] = (uint64_t)c;
                 v = key_shl<NW>(v, 2 * (k - 1));
-                const Key<NW> gg = load_key<NW>(gk, i0 + j);
+                const Key<NW> gg = load_key<NW>(gk, at_pad(i0 + j));
 #pragma unroll
                 for (int w = 0; w < NW; w++) v.w[w] |= gg.w[w];
                 store_key<NW>(found, o++, v);
@@ -380,10 +384,11 @@ __global__ void symbol_starts_kernel(const uint64_t* __restrict__ ck, uint64_t E
 // the same label; a group holds at most 16) and whether it ends its node from
 // the neighbours, and a warp's ballots are words of the bit-vectors.
 // Reads each key once from memory (the neighbours come from L1) and writes
-// each output once; bound by the loads in flight.  3.5e8 edges of one word:
-// 2.7 ms, where flags, insertion counts, their scan, bytes and their packing
-// (53 bytes an edge) took 6.5; build of 3 M reads at k = 47 with
-// multiplicities 4.23 -> 3.75 ms.
+// each output once; bound by the loads in flight (four keys a thread at five
+// CTAs an SM: eight at two took 2.7 ms for 3.5e8 edges).  3.5e8 edges of one
+// word: 1.8 ms, where flags, insertion counts, their scan, bytes and their
+// packing (53 bytes an edge) took 6.5; build of 3 M reads at k = 47 with
+// multiplicities: 0.34 ms.
 constexpr int kEmitTile = 2048;
 
 // pb[2 b] / pb[2 b + 1]: dummies / $ entries placed before position b * kEmitTile.
@@ -403,7 +408,7 @@ __global__ void emit_bounds_kernel(const uint64_t* __restrict__ pos_d, uint64_t 
 }
 
 template <int NW>
-__global__ void __launch_bounds__(256) emit_kernel(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cv,
+__global__ void __launch_bounds__(256, NW == 4 ? 3 : 5) emit_kernel(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cv,
                                                    uint64_t E, const uint64_t* __restrict__ dk, uint64_t t,
                                                    const uint64_t* __restrict__ pos_d,
                                                    const uint64_t* __restrict__ pos_u, uint64_t m,
@@ -412,7 +417,7 @@ __global__ void __launch_bounds__(256) emit_kernel(const uint64_t* __restrict__ 
                                                    uint32_t* __restrict__ valid, uint32_t* __restrict__ mult,
                                                    unsigned long long* __restrict__ n_last) {
     constexpr int kWords = kEmitTile / 32;  // 32 positions each, eight a warp
-    constexpr int U = NW == 1 ? 8 : NW == 2 ? 4 : 2;
+    constexpr int U = NW == 1 ? 4 : 2;
     __shared__ uint8_t pad[kEmitTile];      // where pmask is set: W code, bit 4 last, bit 5 dummy
     __shared__ uint32_t pmask[kWords], pre[kWords], sum_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
