@@ -650,6 +650,11 @@ template <int NW>
 bool merge_runs(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* vals, uint32_t* valt,
                 const std::vector<uint64_t>& bounds);
 
+// The edges of both tables (mercy may be null) as colex keys, ascending, with
+// their counts where cv is set (mh_colex.cu).
+template <int NW>
+void colex_merge(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, int k, uint64_t* ck, uint32_t* cv);
+
 // One read set through pack, count and (by flags) mercy and build on
 // context w (mh_batch.cu); a failed set keeps no outputs.
 int run_set_job(mh_ctx* w, const mh_read_set& s, int k, int d, int flags, mh_set_result& r);
