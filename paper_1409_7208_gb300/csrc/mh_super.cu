@@ -19,22 +19,26 @@
 //            the bin's counters gives (records low, windows high)
 //   place    the records past their bin's slots (half as many again as the
 //            mean), from a list, to places after a scan
-//   count    a CTA per bin: a warp takes 32 records at a time, a lane a
-//            window; its mixed canonical key goes into a hash table in
-//            shared memory; then the table's entries (the spectrum) and the
-//            kept keys of both strands are written at places reserved by
-//            one atomic each.  The kept keys are sorted afterwards, so the
+//   count    a CTA per bin: equal records merged, then 32 windows at a time
+//            a warp; a window's mixed canonical key goes into a hash table
+//            in shared memory; then each warp writes its eighth of the table
+//            (the spectrum, and the kept keys of both strands) at places
+//            reserved by one atomic each, and clears it for the next bin.  The kept keys are sorted afterwards, so the
 //            bins' order does not matter.
 //   rest     bins with more windows than one CTA should take, or whose keys
 //            do not fit the table, are expanded to keys and counted by the
 //            unit counting (mh_group.cu); their spectrum goes last
 //
-// What bounds it: instruction issue (a hash insertion a window) and the
-// waits at a bin's barriers, not memory: a window moves about 2 bytes of
-// records and 4 of outputs instead of 8 to 32 a pass.  3 Gbp, k = 31, 2.38 G
-// windows: split 6.6 ms (67 thread instructions a position), place 8.1, count
-// 25.1, where the extraction, two passes, the units and their compaction took
-// 18.8 + 28 + 22.3 + 5.2; 3 M reads of 100-150 bp at k = 61: 6.1 ms for 15.2.
+// What bounds it: the waits between a bin's barriers and instruction issue (a
+// hash insertion a window), not memory: a window moves about 2 bytes of
+// records and 4 of outputs instead of 8 to 32 a pass.  Equal records are
+// counted once with their number (keys of one word: their records are short
+// against a read, so most recur whole), which at 3 Gbp and k = 31 takes the
+// count from 24.6 to 21.4 ms; for wider keys most runs end with their read,
+// and it would cost more than it saves.  3 Gbp, k = 31, 2.38 G windows: split
+// 7.4 ms (67 thread instructions a position), count 21.4, where the
+// extraction, two passes, the units and their compaction took 18.8 + 28 + 22.3
+// + 5.2; 3 M reads of 100-150 bp at k = 61: 5.6 ms for 15.2.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -301,28 +305,31 @@ __device__ __forceinline__ uint32_t for_windows(uint64_t rec, const Body& body) 
     return tot;
 }
 
-// Shared memory of a bin's CTA: the table (top words, other words, counts),
-// its occupancy bits and the entries before each word of them, and the
-// records of a round (starts among the round's windows, symbols), over
+// Shared memory of a bin's CTA: the table (top words, other words, counts)
+// and the records of a round (starts among the round's windows, symbols), over
 // which the list of occupied slots goes afterwards.  For one word 56 KB, so
 // that four CTAs share an SM.
 template <int NW>
 struct SuperSmem {
     static constexpr int kSlots = SuperCfg<NW>::kSlots;
-    static constexpr int kRecs = NW == 1 ? 352 : 512 / NW;  // records a round
+    static constexpr int kRecs = NW == 1 ? 448 : 512 / NW;  // records a round
     static constexpr int kRW = SuperCfg<NW>::kRecWords;    // words a record's symbols take
     static constexpr int kMost = kSlots / 128 * 108;       // entries a table may hold (0.84 of its slots)
+    static constexpr int kRegion = kSlots / 8;             // a warp's share of the slots
+    static constexpr bool kAlike = NW == 1;                // equal records are counted once, with their number
+    static constexpr int kOwners = 1024;
     static constexpr size_t kFp = 0;
     static constexpr size_t kLow = kFp + sizeof(uint64_t) * kSlots;
     static constexpr size_t kCnt = kLow + sizeof(uint64_t) * (NW - 1) * kSlots;
-    static constexpr size_t kOcc = kCnt + sizeof(uint32_t) * kSlots;
-    static constexpr size_t kPre = kOcc + sizeof(uint32_t) * (kSlots / 32);
-    static constexpr size_t kSym = kPre + sizeof(uint16_t) * (kSlots / 32);
+    static constexpr size_t kSym = kCnt + (NW == 1 ? sizeof(uint16_t) : sizeof(uint32_t)) * kSlots;
     static constexpr size_t kStart = kSym + sizeof(uint32_t) * kRW * kRecs;
-    static constexpr size_t kRecEnd = kStart + sizeof(uint32_t) * kRecs;
-    static constexpr size_t kListEnd = kSym + sizeof(uint16_t) * kMost;
+    static constexpr size_t kMul = kStart + sizeof(uint32_t) * kRecs;
+    static constexpr size_t kOwn = kMul + (kAlike ? sizeof(uint32_t) * kRecs : 0);
+    static constexpr size_t kRecEnd = kOwn + (kAlike ? sizeof(uint32_t) * kOwners : 0);
+    static constexpr size_t kListEnd = kSym + sizeof(uint16_t) * kSlots;
     static constexpr size_t kBytes = kRecEnd > kListEnd ? kRecEnd : kListEnd;
-    static_assert(kSym % 16 == 0, "aligned");
+    static_assert(!kAlike || (kRecs <= kOwners / 2 && kRecs * (16 * kRW) < (1 << 16)), "records and windows of a round");
+    static_assert(kSym % 16 == 0 && kOwn % 16 == 0, "aligned");
 };
 
 // A CTA per bin.  The table's first word is a mixed key's top word (the whole
@@ -349,20 +356,48 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     uint64_t* fp = reinterpret_cast<uint64_t*>(smem + L::kFp);
     uint64_t* low = reinterpret_cast<uint64_t*>(smem + L::kLow);
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + L::kCnt);
-    uint32_t* occ = reinterpret_cast<uint32_t*>(smem + L::kOcc);
-    uint16_t* pre = reinterpret_cast<uint16_t*>(smem + L::kPre);
     uint32_t* sym = reinterpret_cast<uint32_t*>(smem + L::kSym);
     uint32_t* start = reinterpret_cast<uint32_t*>(smem + L::kStart);
-    uint16_t* list = reinterpret_cast<uint16_t*>(smem + L::kSym);
-    __shared__ uint32_t over, n_ent;
-    __shared__ uint32_t scratch[8], wsol[8];
+    __shared__ uint32_t over;
+    __shared__ uint32_t scratch[8], wsol[8], went[8];
     __shared__ uint64_t base[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem + L::kSym) + warp * L::kRegion;  // the warp's occupied slots
     if (totals[T_RECS] > rec_cap) return;
     uint32_t palins = 0;
 
-    auto insert = [&](const Key<NW>& mk) {
+    // exclusive prefix over the CTA (scratch is free again after the next barrier)
+    auto scan = [&](uint32_t v, uint32_t* total) {
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) scratch[warp] = x;
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; w++) {
+            before += w < warp ? scratch[w] : 0u;
+            all += scratch[w];
+        }
+        *total = all;
+        return before + x - v;
+    };
+    uint32_t* mul = reinterpret_cast<uint32_t*>(smem + L::kMul);
+    uint32_t* owner = reinterpret_cast<uint32_t*>(smem + L::kOwn);
+    // counts: 16 bits for one word (a bin has fewer windows than that)
+    auto add = [&](uint32_t at, uint32_t c) {
+        if constexpr (NW == 1) atomicAdd(&cnt[at >> 1], c << (16 * (at & 1)));
+        else atomicAdd(&cnt[at], c);
+    };
+    auto count_at = [&](uint32_t at) -> uint32_t {
+        if constexpr (NW == 1) return reinterpret_cast<const uint16_t*>(cnt)[at];
+        else return cnt[at] & ~kReady;
+    };
+    auto insert = [&](const Key<NW>& mk, uint32_t c) {
         const uint64_t t = mk.w[NW - 1];
         if (NW > 1 && t == kEmpty) {
             over = 1;
@@ -376,15 +411,16 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
             uint64_t cur = at == s ? v.x : v.y;
             if (cur == kEmpty) {
                 cur = atomicCAS((unsigned long long*)&fp[at], (unsigned long long)kEmpty, (unsigned long long)t);
-                if (cur == kEmpty) {
-                    if constexpr (NW > 1) {
+                if constexpr (NW > 1) {
+                    if (cur == kEmpty) {
 #pragma unroll
                         for (int q = 0; q < NW - 1; q++) low[q * C::kSlots + at] = mk.w[q];
                         __threadfence_block();
+                        add(at, c | kReady);
+                        return;
                     }
-                    atomicAdd(&cnt[at], NW > 1 ? 1u | kReady : 1u);
-                    atomicOr(&occ[at >> 5], 1u << (at & 31));
-                    return;
+                } else if (cur == kEmpty) {
+                    cur = t;
                 }
             }
             if (cur == t) {
@@ -401,7 +437,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                     for (int q = 0; q < NW - 1; q++) same &= *(volatile uint64_t*)&low[q * C::kSlots + at] == mk.w[q];
                 }
                 if (same) {
-                    atomicAdd(&cnt[at], 1u);
+                    add(at, c);
                     return;
                 }
                 over = 1;  // two wide keys with the same top word
@@ -413,73 +449,175 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
         over = 1;
     };
 
+    // the next bin's counters and first round of records, fetched while the
+    // bin before it is written out (those past a bin's slots later)
+    constexpr int R = (L::kRecs + 255) / 256;  // records a thread
+    uint64_t next_have = 0, next_off = 0, next_rr[R];
+    auto fetch = [&](uint32_t b) {
+        if (b >= b1) return;
+        next_have = recs.bins[b];
+        next_off = recs.off[b];
+#pragma unroll
+        for (int q = 0; q < R; q++) {
+            const uint32_t i = R * tid + q;
+            if (i < recs.slots) next_rr[q] = recs.rec[(uint64_t)b * recs.slots + i];
+        }
+    };
+    auto next_hot = [&]() -> uint32_t { return (uint32_t)(next_have >> 32) > (NW == 1 ? min(hot, 0xFFFFu) : hot); };
+    fetch(b0 + blockIdx.x);
+    if (tid == 0) over = next_hot();
+    for (int i = tid; i < C::kSlots / 2; i += 256)
+        reinterpret_cast<ulonglong2*>(fp)[i] = make_ulonglong2(kEmpty, kEmpty);
+    for (int i = tid; i < C::kSlots / (NW == 1 ? 8 : 4); i += 256)
+        reinterpret_cast<uint4*>(cnt)[i] = make_uint4(0, 0, 0, 0);
     for (uint32_t b = b0 + blockIdx.x; b < b1; b += gridDim.x) {
-        const uint64_t have = recs.bins[b], o0 = recs.off[b];
+        const uint64_t have = next_have, o0 = next_off;
         const uint32_t n_rec = (uint32_t)have, W = (uint32_t)(have >> 32);
-        if (tid == 0) over = W > hot;
-        for (int i = tid; i < C::kSlots / 2; i += 256)
-            reinterpret_cast<ulonglong2*>(fp)[i] = make_ulonglong2(kEmpty, kEmpty);
-        for (int i = tid; i < C::kSlots / 4; i += 256) reinterpret_cast<uint4*>(cnt)[i] = make_uint4(0, 0, 0, 0);
-        if (tid < C::kWords) occ[tid] = 0;
         // rounds of up to kRecs records: their windows are numbered through,
         // an eighth of them to each warp, 32 at a time
         for (uint32_t rb = 0; rb < n_rec; rb += L::kRecs) {
             __syncthreads();
             if (*(volatile uint32_t*)&over) break;
             const uint32_t nr = min(n_rec - rb, (uint32_t)L::kRecs);
-            constexpr int R = (L::kRecs + 255) / 256;  // records a thread
             uint64_t rr[R];
             uint32_t sum = 0;
 #pragma unroll
             for (int q = 0; q < R; q++) {
-                rr[q] = (uint32_t)(R * tid + q) < nr ? recs.at(b, o0, rb + R * tid + q) : 0ull;
+                const uint32_t i = R * tid + q;
+                rr[q] = i >= nr ? 0ull : rb == 0 && i < recs.slots ? next_rr[q] : recs.at(b, o0, rb + i);
                 sum += (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
             }
-            uint32_t tot;
-            uint32_t ex = block_excl_scan_256(sum, scratch, &tot);
+            // a record's symbols from the packed reads, aligned to a word:
+            // all of a thread's loads in flight at once
+            auto symbols = [&](uint64_t rec, uint32_t nw, uint32_t out[L::kRW]) {
+                const uint64_t p = rec >> kNwinBits;
+                const uint32_t* src = packed + (p >> 4);
+                const uint32_t sh = 2 * (uint32_t)(p & 15), need = ((uint32_t)(p & 15) + nw + K1 - 1 + 15) / 16;
+                uint32_t v[L::kRW + 1];
 #pragma unroll
-            for (int q = 0; q < R; q++) {
-                const uint32_t nw = (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
-                if (nw) {
-                    // the record's symbols from the packed reads, aligned to
-                    // a word: all of a thread's loads in flight at once
-                    const uint64_t p = rr[q] >> kNwinBits;
-                    const uint32_t* src = packed + (p >> 4);
-                    const uint32_t sh = 2 * (uint32_t)(p & 15), need = ((uint32_t)(p & 15) + nw + K1 - 1 + 15) / 16;
-                    uint32_t v[L::kRW + 1];
+                for (int i = 0; i <= L::kRW; i++) v[i] = (uint32_t)i < need ? src[i] : 0u;
 #pragma unroll
-                    for (int i = 0; i <= L::kRW; i++) v[i] = (uint32_t)i < need ? src[i] : 0u;
-                    uint4* dst = reinterpret_cast<uint4*>(sym + (R * tid + q) * L::kRW);
+                for (int i = 0; i < L::kRW; i++) out[i] = __funnelshift_l(v[i + 1], v[i], sh);
+            };
+            uint32_t tot, n_run;  // windows and records of the round
+            if constexpr (L::kAlike) {
+                // Most reads cover a place of the genome whole and without
+                // error, and give equal records there.  A record is turned
+                // to the smaller of its symbols and their reverse complement
+                // (it has the same canonical windows), the first of equal
+                // ones owns a place in a table of this round, and the others
+                // only add to its number.
+                for (int i = tid; i < L::kOwners / 4; i += 256) reinterpret_cast<uint4*>(owner)[i] = make_uint4(0, 0, 0, 0);
+                uint64_t xh[R], xl[R];
+                uint32_t nw[R];
 #pragma unroll
-                    for (int i = 0; i < L::kRW / 4; i++)
-                        dst[i] = make_uint4(__funnelshift_l(v[4 * i + 1], v[4 * i], sh), __funnelshift_l(v[4 * i + 2], v[4 * i + 1], sh),
-                                            __funnelshift_l(v[4 * i + 3], v[4 * i + 2], sh),
-                                            __funnelshift_l(v[4 * i + 4], v[4 * i + 3], sh));
-                    start[R * tid + q] = ex;
+                for (int q = 0; q < R; q++) {
+                    nw[q] = (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
+                    if (!nw[q]) continue;
+                    uint32_t w[L::kRW];
+                    symbols(rr[q], nw[q], w);
+                    const int bits = 2 * ((int)nw[q] + K1 - 1);  // of 128, at the top
+                    uint64_t h = (uint64_t)w[0] << 32 | w[1], l = (uint64_t)w[2] << 32 | w[3];
+                    if (bits <= 64) {
+                        h &= ~0ull << (64 - bits);
+                        l = 0;
+                    } else {
+                        l &= ~0ull << (128 - bits);
+                    }
+                    uint64_t rh = rev2_u64(~l), rl = rev2_u64(~h);
+                    const int up = 128 - bits;
+                    if (up >= 64) {
+                        rh = rl << (up - 64);
+                        rl = 0;
+                    } else if (up) {
+                        rh = rh << up | rl >> (64 - up);
+                        rl <<= up;
+                    }
+                    if (rh < h || (rh == h && rl < l)) {
+                        h = rh;
+                        l = rl;
+                    }
+                    xh[q] = h;
+                    xl[q] = l;
+                    const uint32_t i = R * tid + q;
+                    reinterpret_cast<uint4*>(sym)[i] = make_uint4((uint32_t)(h >> 32), (uint32_t)h, (uint32_t)(l >> 32), (uint32_t)l);
+                    start[i] = nw[q];
+                    mul[i] = 1;
                 }
-                ex += nw;
+                __syncthreads();
+                uint32_t sums = 0;
+#pragma unroll
+                for (int q = 0; q < R; q++) {
+                    if (!nw[q]) continue;
+                    const uint32_t i = R * tid + q;
+                    uint32_t o = (uint32_t)(mix_bij(xh[q] ^ mix_bij(xl[q] + nw[q])) >> 54);
+                    static_assert(L::kOwners == 1 << 10, "ten bits");
+                    while (true) {  // (at most half of the places are taken)
+                        const uint32_t first = atomicCAS(&owner[o], 0u, i + 1);
+                        if (!first) break;
+                        const uint4 y = reinterpret_cast<const uint4*>(sym)[first - 1];
+                        if (y.x == (uint32_t)(xh[q] >> 32) && y.y == (uint32_t)xh[q] && y.z == (uint32_t)(xl[q] >> 32) &&
+                            y.w == (uint32_t)xl[q] && start[first - 1] == nw[q]) {
+                            atomicAdd(&mul[first - 1], 1u);
+                            nw[q] = 0;
+                            break;
+                        }
+                        o = (o + 1) & (L::kOwners - 1);
+                    }
+                    if (nw[q]) sums += nw[q] | 1u << 16;
+                }
+                uint32_t all;
+                uint32_t ex = scan(sums, &all);
+                tot = all & 0xFFFFu;
+                n_run = all >> 16;
+#pragma unroll
+                for (int q = 0; q < R; q++)
+                    if (nw[q]) {
+                        start[ex >> 16] = (ex & 0xFFFFu) | (uint32_t)(R * tid + q) << 16;
+                        ex += nw[q] | 1u << 16;
+                    }
+            } else {
+                uint32_t ex = scan(sum, &tot);
+                n_run = nr;
+#pragma unroll
+                for (int q = 0; q < R; q++) {
+                    const uint32_t nw = (uint32_t)rr[q] & ((1u << kNwinBits) - 1u);
+                    if (nw) {
+                        uint32_t w[L::kRW];
+                        symbols(rr[q], nw, w);
+                        uint4* dst = reinterpret_cast<uint4*>(sym + (R * tid + q) * L::kRW);
+#pragma unroll
+                        for (int i = 0; i < L::kRW / 4; i++)
+                            dst[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                        start[R * tid + q] = ex;
+                    }
+                    ex += nw;
+                }
             }
             __syncthreads();
             const uint32_t per = (tot + 255) / 256 * 32;
             uint32_t j0 = warp * per;
             const uint32_t je = min(tot, j0 + per);
             if (j0 >= je) continue;
-            // the last record that starts at or before window j0
+            // the last record that starts at or before window j0 (the upper
+            // half of start is the record's place where equal ones are merged)
+            constexpr uint32_t kAt = L::kAlike ? 0xFFFFu : 0xFFFFFFFFu;
             uint32_t cur = 0;
 #pragma unroll
             for (int step = 256; step; step >>= 1)
-                if (cur + step < nr && start[cur + step] <= j0) cur += step;
+                if (cur + step < n_run && (start[cur + step] & kAt) <= j0) cur += step;
             for (; j0 < je; j0 += 32) {
                 // the record of window j0 + lane: the records after cur that
                 // start among these windows, as bits
-                const uint32_t nx = cur + 1 + lane, rel = (nx < nr ? start[nx] : 0xFFFFFFFFu) - j0;
+                const uint32_t nx = cur + 1 + lane, rel = (nx < n_run ? start[nx] & kAt : 0xFFFFFFFFu) - j0;
                 const uint32_t m = __reduce_or_sync(0xFFFFFFFFu, rel < 32u ? 1u << rel : 0u);
                 const uint32_t idx = cur + __popc(m & (0xFFFFFFFFu >> (31 - lane)));
                 cur += __popc(m);
                 if (j0 + lane < je) {
                     // the window's 2 NW words (and one more) of its record
-                    const uint32_t at = j0 + lane - start[idx], sh = 2 * (at & 15);
-                    const uint32_t* src = sym + idx * L::kRW + (at >> 4);
+                    const uint32_t st = start[idx], at = j0 + lane - (st & kAt), sh = 2 * (at & 15);
+                    const uint32_t id = L::kAlike ? st >> 16 : idx;
+                    const uint32_t* src = sym + id * L::kRW + (at >> 4);
                     Key<NW> x;
                     uint32_t hi = src[0];
 #pragma unroll
@@ -490,56 +628,13 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                     }
                     x = key_shr<NW>(x, 64 * NW - 2 * K1);
                     const Key<NW> rc = key_rc<NW>(x, K1);
-                    insert(mix_key<NW>(key_less<NW>(rc, x) ? rc : x));
+                    insert(mix_key<NW>(key_less<NW>(rc, x) ? rc : x), L::kAlike ? mul[id] : 1u);
                 }
             }
         }
         __syncthreads();
-        // entries before each word of the occupancy bits (warp 0)
-        if (warp == 0) {
-            constexpr int per = C::kWords / 32;
-            uint32_t v[per], sum = 0;
-#pragma unroll
-            for (int q = 0; q < per; q++) {
-                v[q] = __popc(occ[lane * per + q]);
-                sum += v[q];
-            }
-            uint32_t x = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= o) x += y;
-            }
-            uint32_t e = x - sum;
-#pragma unroll
-            for (int q = 0; q < per; q++) {
-                pre[lane * per + q] = (uint16_t)e;
-                e += v[q];
-            }
-            if (lane == 31) n_ent = x;
-        }
-        __syncthreads();
-        const uint32_t ne = n_ent;
-        if (over || ne > (uint32_t)L::kMost) {
-            // to the rest; its place among the rest's keys
-            if (tid == 0) {
-                soff[b] = kSuperDeferred;
-                const uint64_t q = atomicAdd(&totals[T_DEF], 1ull);
-                deferred[q] = make_ulonglong2(b, atomicAdd(&totals[T_DEFWIN], (unsigned long long)W));
-            }
-            __syncthreads();
-            continue;
-        }
-        // the occupied slots listed in order
-        if (tid < C::kWords) {
-            uint32_t m = occ[tid], at = pre[tid];
-            sidx[(uint64_t)b * C::kWords + tid] = make_uint2(m, at);
-            while (m) {
-                list[at++] = (uint16_t)(tid * 32 + __ffs(m) - 1);
-                m &= m - 1;
-            }
-        }
-        __syncthreads();
+        // a warp an eighth of the slots: the occupied ones listed in order,
+        // the occupancy bits of word q and the entries before it in lane q
         auto key_at = [&](uint32_t s) {
             Key<NW> m;
             m.w[NW - 1] = fp[s];
@@ -549,60 +644,104 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
             }
             return m;
         };
-        // kept keys: counted, a place reserved, then written with the entries
-        uint32_t no = 0;
-        for (uint32_t e0 = warp * 32; e0 < ne; e0 += 256) {
-            const uint32_t e = e0 + lane;
-            bool pl = false;
-            uint64_t lit = 0;
-            if (e < ne) {
-                const uint32_t s = list[e];
-                lit = cnt[s] & ~kReady;
-                if (!(K1 & 1)) {
+        constexpr int WW = C::kWords / 8;
+        uint32_t mine = 0, no = 0, my_occ = 0, my_pre = 0, my_palins = 0;
+#pragma unroll
+        for (int q = 0; q < WW; q++) {
+            const uint32_t s = (warp * WW + q) * 32 + lane, lit = count_at(s);
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, lit != 0), at = mine + __popc(m & lt);
+            if (lit) list[at] = (uint16_t)s;
+            if (lane == q) {
+                my_occ = m;
+                my_pre = mine;
+            }
+            mine += __popc(m);
+            // kept keys of both strands (an odd window is no palindrome)
+            if (K1 & 1) no += 2 * __popc(__ballot_sync(0xFFFFFFFFu, lit && lit >= (uint32_t)d));
+        }
+        __syncwarp();
+        if (!(K1 & 1))
+            for (uint32_t e0 = 0; e0 < mine; e0 += 32) {
+                const uint32_t e = e0 + lane;
+                bool pl = false;
+                uint64_t lit = 0;
+                if (e < mine) {
+                    const uint32_t s = list[e];
+                    lit = count_at(s);
                     const Key<NW> x = unmix_key<NW>(key_at(s));
                     pl = key_eq<NW>(key_rc<NW>(x, K1), x);
                     if (pl) lit *= 2;
                 }
+                const uint32_t sm = __ballot_sync(0xFFFFFFFFu, e < mine && lit >= (uint64_t)d), pm = __ballot_sync(0xFFFFFFFFu, pl);
+                no += 2 * __popc(sm) - __popc(sm & pm);
+                my_palins += __popc(pm);
             }
-            const uint32_t sm = __ballot_sync(0xFFFFFFFFu, e < ne && lit >= (uint64_t)d), pm = __ballot_sync(0xFFFFFFFFu, pl);
-            no += 2 * __popc(sm) - __popc(sm & pm);
-            palins += __popc(pm);
+        if (lane == 0) {
+            wsol[warp] = no;
+            went[warp] = mine;
         }
-        if (lane == 0) wsol[warp] = no;
+        fetch(b + gridDim.x);
         __syncthreads();
-        if (tid == 0) {
-            uint32_t c = 0;
-            for (int q = 0; q < 8; q++) c += wsol[q];
-            base[0] = atomicAdd(&totals[T_SPEC], (unsigned long long)ne);
-            base[1] = atomicAdd(&totals[T_SOLID], (unsigned long long)c);
-            soff[b] = base[0];
-        }
-        __syncthreads();
-        uint32_t po = 0, to = 0;
+        uint32_t po = 0, to = 0, pe = 0, ne = 0;
+#pragma unroll
         for (int q = 0; q < 8; q++) {
             po += q < warp ? wsol[q] : 0u;
             to += wsol[q];
+            pe += q < warp ? went[q] : 0u;
+            ne += went[q];
         }
+        const bool rest = over || ne > (uint32_t)L::kMost;
+        // (a warp's own slots are free once they are listed or written)
+        auto clear = [&] {
+            ulonglong2* f = reinterpret_cast<ulonglong2*>(fp + warp * L::kRegion);
+            for (int i = lane; i < L::kRegion / 2; i += 32) f[i] = make_ulonglong2(kEmpty, kEmpty);
+            constexpr int kPer = NW == 1 ? 8 : 4;  // counts in 16 bytes
+            uint4* c = reinterpret_cast<uint4*>(cnt) + warp * (L::kRegion / kPer);
+            for (int i = lane; i < L::kRegion / kPer; i += 32) c[i] = make_uint4(0, 0, 0, 0);
+        };
+        if (rest) {
+            // to the rest; its place among the rest's keys
+            if (tid == 0) {
+                soff[b] = kSuperDeferred;
+                const uint64_t q = atomicAdd(&totals[T_DEF], 1ull);
+                deferred[q] = make_ulonglong2(b, atomicAdd(&totals[T_DEFWIN], (unsigned long long)W));
+            }
+            clear();
+            __syncthreads();
+            if (tid == 0) over = next_hot();
+            continue;
+        }
+        palins += my_palins;
+        // places for the entries and the kept keys, then both written
+        if (tid == 0) {
+            base[0] = atomicAdd(&totals[T_SPEC], (unsigned long long)ne);
+            base[1] = atomicAdd(&totals[T_SOLID], (unsigned long long)to);
+            soff[b] = base[0];
+        }
+        if (lane < WW) sidx[(uint64_t)b * C::kWords + warp * WW + lane] = make_uint2(my_occ, pe + my_pre);
+        __syncthreads();
+        if (tid == 0) over = next_hot();
         // (past a buffer's end nothing is written: the host sees the totals)
         if (base[0] + ne <= spec_cap && base[1] + to <= solid_cap) {
             uint64_t so = base[1] + po;
-            for (uint32_t e0 = warp * 32; e0 < ne; e0 += 256) {
+            const uint64_t eo = base[0] + pe;
+            for (uint32_t e0 = 0; e0 < mine; e0 += 32) {
                 const uint32_t e = e0 + lane;
                 bool pl = false;
                 uint32_t lit = 0;
                 Key<NW> x{}, r{};
-                if (e < ne) {
+                if (e < mine) {
                     const uint32_t s = list[e];
                     const Key<NW> m = key_at(s);
-                    lit = cnt[s] & ~kReady;
-                    store_key<NW>(spec_k, base[0] + e, m);
-                    spec_len[base[0] + e] = lit;
+                    lit = count_at(s);
+                    store_key<NW>(spec_k, eo + e, m);
+                    spec_len[eo + e] = lit;
                     x = unmix_key<NW>(m);
                     r = key_rc<NW>(x, K1);
                     pl = key_eq<NW>(r, x);
                     if (pl) lit *= 2;
                 }
-                const bool keep = e < ne && lit >= (uint32_t)d;
+                const bool keep = e < mine && lit >= (uint32_t)d;
                 const uint32_t sm = __ballot_sync(0xFFFFFFFFu, keep), pm = __ballot_sync(0xFFFFFFFFu, pl);
                 if (keep) {
                     const uint64_t at = so + 2 * __popc(sm & lt) - __popc(sm & pm & lt);
@@ -616,7 +755,13 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                 so += 2 * __popc(sm) - __popc(sm & pm);
             }
         }
-        __syncthreads();
+        __syncwarp();
+        clear();
+        // the next records on their way to L2
+#pragma unroll
+        for (int q = 0; q < R; q++)
+            if ((uint32_t)(R * tid + q) < min((uint32_t)next_have, recs.slots))
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(packed + (next_rr[q] >> (kNwinBits + 4))));
     }
     if (lane == 0 && palins) atomicAdd(&totals[T_PALIN], (unsigned long long)palins);
 }
