@@ -66,3 +66,11 @@ def test_mercy_groups(k, n):
         reads.append("".join(r))
     a, o = synth.reads_from_strings(reads)
     _check(a, o, k, 2, with_mult=True)
+
+
+@pytest.mark.parametrize("k,n", [(21, 1), (21, 16), (21, 8191), (21, 8192), (21, 8193), (40, 4095), (40, 4097), (80, 2048), (80, 2049)])
+def test_sorts_around_one_cta(k, n):
+    # 2 n dummies, sorted by one CTA up to 16,384 words of keys
+    rng = np.random.default_rng(n)
+    a, o = synth.reads_from_strings([_dna(rng, k + 1) for _ in range(n)])
+    assert _check(a, o, k, 1)[0] == 6 * n
