@@ -626,8 +626,15 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                         x.w[NW - 1 - i] = ((uint64_t)__funnelshift_l(md, hi, sh) << 32) | __funnelshift_l(lo, md, sh);
                         hi = lo;
                     }
+                    // the window at the top of the words, whatever follows
+                    // below: shifted down it is the key; its symbols
+                    // reversed and complemented, what is above the window
+                    // masked off, the reverse complement
+                    Key<NW> rc;
+#pragma unroll
+                    for (int i = 0; i < NW; i++) rc.w[i] = rev2_u64(~x.w[NW - 1 - i]);
+                    rc = key_low<NW>(rc, 2 * K1);
                     x = key_shr<NW>(x, 64 * NW - 2 * K1);
-                    const Key<NW> rc = key_rc<NW>(x, K1);
                     insert(mix_key<NW>(key_less<NW>(rc, x) ? rc : x), L::kAlike ? mul[id] : 1u);
                 }
             }
