@@ -69,7 +69,9 @@ __device__ __forceinline__ uint64_t lb_ext(const uint64_t* __restrict__ a, uint6
 // shared memory, the four ranges are streamed past them, and a node c.g
 // clears label c of group g: what is left are targets that no edge leaves.
 // Reads every key twice and writes next to nothing; bound by the searches in
-// shared memory.  3.5e8 edges of one word: 4.4 ms, where writing the sorted
+// shared memory, a lane a key and eight CTAs an SM to hide them (four
+// searches a lane 4.0 ms, two warps a label walking on from a search in eight
+// 4.4 and more).  3.5e8 edges of one word: 3.3 ms, where writing the sorted
 // nodes and targets, one radix pass and the merge of their differences took
 // 12.6.
 template <int NW>
@@ -116,75 +118,85 @@ __global__ void zero_bounds_kernel(const uint64_t* __restrict__ ck, uint64_t E, 
 // Tile t's targets without out-edges, as reversed nodes: cnt[c * n_tiles + t]
 // of them with label c, ascending, from found[at[t]] on, label after label.
 template <int NW>
-__global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restrict__ ck, int k, uint64_t n_tiles,
+__global__ void __launch_bounds__(256, NW == 4 ? 4 : 8) zero_out_kernel(const uint64_t* __restrict__ ck, int k, uint64_t n_tiles,
                                                        const uint64_t* __restrict__ st,
                                                        const uint64_t* __restrict__ tb, uint64_t* __restrict__ found,
                                                        uint64_t* __restrict__ at, uint32_t* __restrict__ cnt,
                                                        unsigned long long* __restrict__ n_found) {
     using Z = ZeroTile<NW>;
     constexpr int I = Z::kItems;
-    // (one place of padding after kItems: a thread's entries, and so the
-    // groups its neighbours search and walk, lie about kItems apart)
-    constexpr int kPadded = Z::kCap / I * (I + 1);
-    __shared__ __align__(16) uint64_t gk[kPadded * NW];  // the groups
-    __shared__ uint32_t gm[kPadded];                     // labels left
-    auto at_pad = [](uint32_t i) { return i + i / I; };
+    __shared__ __align__(16) uint64_t gk[bisect_at<NW>(Z::kCap) * NW];  // the groups
+    __shared__ __align__(16) uint32_t gm[Z::kCap];       // a byte a label: 1 where it is left
     __shared__ uint32_t scratch[8];
     __shared__ uint64_t wsum[8], base;
+    uint8_t* left = reinterpret_cast<uint8_t*>(gm);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t t = blockIdx.x, s0 = st[t];
-    const uint32_t n = (uint32_t)(st[t + 1] - s0);  // at most kTile + 15
-    // groups, numbered in order
-    Key<NW> x[I];
-    uint32_t heads = 0;
-    const uint32_t i0 = tid * I;
-    for (int j = 0; j < I; j++) gm[at_pad(i0 + j)] = 0;
+    const uint32_t n = (uint32_t)min(st[t + 1] - s0, (uint64_t)Z::kCap);  // at most kTile + 15
+    // groups, numbered in order: a warp 32 I entries, 32 at a time
+    uint32_t ng = 0;
     {
-        Key<NW> prev = key_zero<NW>();
-        if (i0 > 0 && i0 < n) prev = load_key<NW>(ck, s0 + i0 - 1);
-#pragma unroll
-        for (int j = 0; j < I; j++)
-            if (i0 + j < n) x[j] = load_key<NW>(ck, s0 + i0 + j);
+        Key<NW> x[I];
+        uint32_t heads[I], mine = 0;
+        const uint32_t w0 = warp * 32 * I + lane;
 #pragma unroll
         for (int j = 0; j < I; j++) {
-            if (i0 + j >= n) continue;
-            if (i0 + j == 0 || !key_eq<NW>(key_shr<NW>(x[j], 4), key_shr<NW>(j ? x[j > 0 ? j - 1 : 0] : prev, 4)))
-                heads |= 1u << j;
+            gm[tid + j * 256] = 0;
+            x[j] = key_zero<NW>();
+            if (w0 + j * 32 < n) x[j] = load_key<NW>(ck, s0 + w0 + j * 32);
+        }
+        Key<NW> before = key_zero<NW>();
+        if (lane == 0 && w0 && w0 < n) before = load_key<NW>(ck, s0 + w0 - 1);
+#pragma unroll
+        for (int j = 0; j < I; j++) {
+            Key<NW> y;
+#pragma unroll
+            for (int w = 0; w < NW; w++) {
+                y.w[w] = __shfl_up_sync(0xFFFFFFFFu, x[j].w[w], 1);
+                const uint64_t last = j ? __shfl_sync(0xFFFFFFFFu, x[j > 0 ? j - 1 : 0].w[w], 31) : before.w[w];
+                if (lane == 0) y.w[w] = last;
+            }
+            const uint32_t i = w0 + j * 32;
+            heads[j] = __ballot_sync(0xFFFFFFFFu,
+                                     i < n && (i == 0 || !key_eq<NW>(key_shr<NW>(x[j], 4), key_shr<NW>(y, 4))));
+            mine += __popc(heads[j]);
+        }
+        if (lane == 0) scratch[warp] = mine;
+        __syncthreads();
+        uint32_t g = 0;
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            g += q < warp ? scratch[q] : 0u;
+            ng += scratch[q];
+        }
+#pragma unroll
+        for (int j = 0; j < I; j++) {
+            if (w0 + j * 32 < n) {
+                const uint32_t mg = g + __popc(heads[j] & (0xFFFFFFFFu >> (31 - lane))) - 1;
+                if ((heads[j] >> lane) & 1u) store_key<NW>(gk, bisect_at<NW>(mg), key_shr<NW>(x[j], 4));
+                left[4 * mg + (uint32_t)(x[j].w[0] & 3u)] = 1;
+            }
+            g += __popc(heads[j]);
         }
     }
-    uint32_t ng;
-    uint32_t g = block_excl_scan_256(__popc(heads), scratch, &ng);
-#pragma unroll
-    for (int j = 0; j < I; j++) {
-        if (i0 + j >= n) continue;
-        if ((heads >> j) & 1u) store_key<NW>(gk, at_pad(g++), key_shr<NW>(x[j], 4));
-        atomicOr(&gm[at_pad(g - 1)], 1u << (uint32_t)(x[j].w[0] & 3u));
-    }
+    const uint32_t i0 = tid * I;
     __syncthreads();
-    // the nodes with first symbol c: two warps a label, I entries a thread,
-    // the first one's group by bisection, the others' from there on
+    // the nodes with first symbol c, c = 0..3, numbered through
     {
-        const uint32_t c = (uint32_t)warp >> 1;
-        const uint64_t b0 = tb[4 * t + c], b1 = tb[4 * (t + 1) + c];
-        for (uint64_t q = b0 + (uint64_t)(tid & 63) * I; q < b1; q += 64 * I) {
-            Key<NW> y[I];
+        uint64_t from[4], end[4], total = 0;
 #pragma unroll
-            for (int j = 0; j < I; j++)
-                if (q + j < b1) y[j] = key_low<NW>(key_shr<NW>(load_key<NW>(ck, q + j), 2), 2 * (k - 1));
-            uint32_t p = 0;
-            {
-                uint32_t hi = ng;
-                while (p < hi) {
-                    const uint32_t mid = (p + hi) >> 1;
-                    if (key_less<NW>(load_key<NW>(gk, at_pad(mid)), y[0])) p = mid + 1; else hi = mid;
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < I; j++) {
-                if (q + j >= b1 || (j && key_eq<NW>(y[j], y[j > 0 ? j - 1 : 0]))) continue;
-                while (p < ng && key_less<NW>(load_key<NW>(gk, at_pad(p)), y[j])) p++;
-                if (p < ng && key_eq<NW>(load_key<NW>(gk, at_pad(p)), y[j])) atomicAnd(&gm[at_pad(p)], ~(1u << c));
-            }
+        for (int c = 0; c < 4; c++) {
+            const uint64_t b0 = tb[4 * t + c], b1 = tb[4 * (t + 1) + c];
+            from[c] = b0 - total;
+            total += b1 > b0 ? b1 - b0 : 0;
+            end[c] = total;
+        }
+        for (uint64_t q = tid; q < total; q += 256) {
+            const uint32_t c = q < end[0] ? 0u : q < end[1] ? 1u : q < end[2] ? 2u : 3u;
+            const uint64_t f = c == 0 ? from[0] : c == 1 ? from[1] : c == 2 ? from[2] : from[3];
+            const Key<NW> y = key_low<NW>(key_shr<NW>(load_key<NW>(ck, q + f), 2), 2 * (k - 1));
+            const uint32_t p = bisect_shared<NW>(gk, ng, y);
+            if (p < ng && key_eq<NW>(load_key<NW>(gk, bisect_at<NW>(p)), y)) left[4 * p + c] = 0;
         }
     }
     __syncthreads();
@@ -193,9 +205,9 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
     uint32_t m[I];
 #pragma unroll
     for (int j = 0; j < I; j++) {
-        m[j] = i0 + j < ng ? gm[at_pad(i0 + j)] : 0u;
+        m[j] = i0 + j < ng ? gm[i0 + j] : 0u;
 #pragma unroll
-        for (int c = 0; c < 4; c++) mine += (uint64_t)((m[j] >> c) & 1u) << (16 * c);
+        for (int c = 0; c < 4; c++) mine += (uint64_t)((m[j] >> (8 * c)) & 1u) << (16 * c);
     }
     uint64_t incl = mine;
 #pragma unroll
@@ -230,11 +242,11 @@ __global__ void __launch_bounds__(256) zero_out_kernel(const uint64_t* __restric
         uint64_t o = base + to[c] + ((uint32_t)(pre >> (16 * c)) & 0xFFFFu);
 #pragma unroll
         for (int j = 0; j < I; j++)
-            if ((m[j] >> c) & 1u) {
+            if ((m[j] >> (8 * c)) & 1u) {
                 Key<NW> v = key_zero<NW>();
                 v.w[0] = (uint64_t)c;
                 v = key_shl<NW>(v, 2 * (k - 1));
-                const Key<NW> gg = load_key<NW>(gk, at_pad(i0 + j));
+                const Key<NW> gg = load_key<NW>(gk, bisect_at<NW>(i0 + j));
 #pragma unroll
                 for (int w = 0; w < NW; w++) v.w[w] |= gg.w[w];
                 store_key<NW>(found, o++, v);

@@ -527,6 +527,25 @@ __device__ __forceinline__ uint64_t gallop_lb(const uint64_t* __restrict__ a, ui
     return lo;
 }
 
+// Place of element i of a sorted array in shared memory that lanes bisect:
+// one of padding after 128 bytes, or the probes of a step, powers of two
+// apart, share their banks.
+template <int NW>
+__host__ __device__ constexpr uint32_t bisect_at(uint32_t i) {
+    return i + i / (16 / NW);
+}
+
+// First index in [0, n) with a[i] >= q (a ascending, in shared memory, padded).
+template <int NW>
+__device__ __forceinline__ uint32_t bisect_shared(const uint64_t* a, uint32_t n, const Key<NW>& q) {
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (key_less<NW>(load_key<NW>(a, bisect_at<NW>(mid)), q)) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
 // ------------------------------------------------------ bitmask scans
 // First set bit at or after i in b (bits [0, n)), or n.
 __device__ __forceinline__ uint32_t next_bit(const uint32_t* b, uint32_t i, uint32_t n) {
