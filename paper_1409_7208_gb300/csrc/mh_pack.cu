@@ -62,12 +62,9 @@ __device__ __forceinline__ void load16(const uint8_t* __restrict__ a, uint64_t n
 // Fast-path pack: code word per chunk; sets *any_invalid if a byte is not a base.
 __global__ void pack_chunks_kernel(const uint8_t* __restrict__ ascii, uint64_t n_bases, bool vec,
                                    uint32_t* __restrict__ packed, uint32_t* __restrict__ any_invalid) {
-    uint64_t n_chunks = ceil_div(n_bases, 16);
+    const uint64_t n_chunks = ceil_div(n_bases, 16), stride = (uint64_t)gridDim.x * blockDim.x;
     bool bad = false;
-    for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < n_chunks;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t x[4], present;
-        load16(ascii, n_bases, c, vec, x, &present);
+    auto pack = [&](uint64_t c, const uint32_t x[4], uint32_t present) {
         uint32_t word = 0, vmask = 0;
 #pragma unroll
         for (int q = 0; q < 4; q++) {
@@ -76,6 +73,21 @@ __global__ void pack_chunks_kernel(const uint8_t* __restrict__ ascii, uint64_t n
         }
         packed[c] = word;
         bad |= (vmask & present) != present;
+    };
+    // four loads in flight a thread (one: 3 Gbp 1.71 ms, four 1.59)
+    constexpr int U = 4;
+    uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    for (; c + (U - 1) * stride < n_chunks; c += U * stride) {
+        uint32_t x[U][4], present[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) load16(ascii, n_bases, c + u * stride, vec, x[u], &present[u]);
+#pragma unroll
+        for (int u = 0; u < U; u++) pack(c + u * stride, x[u], present[u]);
+    }
+    for (; c < n_chunks; c += stride) {
+        uint32_t x[4], present;
+        load16(ascii, n_bases, c, vec, x, &present);
+        pack(c, x, present);
     }
     if (__any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(any_invalid, 1u);
 }
@@ -100,98 +112,150 @@ __global__ void iota_u32_kernel(uint32_t* __restrict__ a, uint64_t n) {
 }
 
 // --------------------------------------------------------- slow path
-// Per chunk: 16-bit validity mask and its popcount.
-__global__ void chunk_masks_kernel(const uint8_t* __restrict__ ascii, uint64_t n_bases, bool vec,
-                                   uint32_t* __restrict__ mask, uint32_t* __restrict__ cnt) {
-    uint64_t n_chunks = ceil_div(n_bases, 16);
-    for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < n_chunks;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t x[4], present;
-        load16(ascii, n_bases, c, vec, x, &present);
-        uint32_t vmask = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) vmask |= mask4(valid4(x[q])) << (4 * q);
-        vmask &= present;
-        mask[c] = vmask;
-        cnt[c] = __popc(vmask);
-    }
-}
+// Invalid bytes or empty reads: tiles of 4,096 input bases, a chunk of 16 a
+// thread, in two sweeps over the input.  The first counts a tile's valid bases
+// and fragment starts, the second (after a scan of the tiles' counts) finds
+// them again, writes the fragments and sets the valid codes side by side in
+// shared memory.  A tile reads its reads' starts once, so a fragment's read
+// comes from a rank among them.  Two sweeps of 16-byte loads and one small
+// scan, bound by memory latency; 5 M trimmed reads with Ns (450 Mbp): 0.92 ms,
+// where masks, counts and prefixes a chunk in memory and a bisection of all
+// offsets a fragment took 2.0 ms.
+constexpr uint32_t kPackTile = 4096;
 
-__global__ void read_starts_kernel(const uint64_t* __restrict__ offs, uint64_t n_reads,
-                                   uint32_t* __restrict__ rs_bits) {
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n_reads;
-         r += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t a = offs[r];
-        if (offs[r + 1] > a) atomicOr(&rs_bits[a >> 5], 1u << (a & 31));
-    }
-}
-
-// Fragment-start bits of chunk c: valid and (read start or previous base invalid).
-__device__ __forceinline__ uint32_t frag_start_bits(const uint32_t* mask, const uint32_t* rs_bits, uint64_t c) {
-    uint32_t m = mask[c];
-    uint32_t prev_valid_top = c ? (mask[c - 1] >> 15) & 1u : 0u;
-    uint32_t prev = (m << 1) | prev_valid_top;  // bit j = validity of base j-1
-    uint32_t rs = (rs_bits[(c * 16) >> 5] >> ((c * 16) & 31)) & 0xFFFFu;
-    return m & (rs | ~prev) & 0xFFFFu;
-}
-
-__global__ void frag_count_kernel(const uint32_t* __restrict__ mask, const uint32_t* __restrict__ rs_bits,
-                                  uint64_t n_chunks, uint32_t* __restrict__ fcnt) {
-    for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < n_chunks;
-         c += (uint64_t)gridDim.x * blockDim.x)
-        fcnt[c] = __popc(frag_start_bits(mask, rs_bits, c));
-}
-
-__global__ void frag_write_kernel(const uint32_t* __restrict__ mask, const uint32_t* __restrict__ rs_bits,
-                                  const uint64_t* __restrict__ dst, const uint64_t* __restrict__ fidx,
-                                  const uint64_t* __restrict__ offs, uint64_t n_reads, uint64_t n_chunks,
-                                  uint64_t* __restrict__ frag_offs, uint32_t* __restrict__ frag_read) {
-    for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < n_chunks;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t fs = frag_start_bits(mask, rs_bits, c);
-        uint32_t m = mask[c];
-        uint64_t f = fidx[c];
-        while (fs) {
-            int j = __ffs(fs) - 1;
-            fs &= fs - 1;
-            frag_offs[f] = dst[c] + __popc(m & ((1u << j) - 1));
-            // read holding base c*16+j: last r with offs[r] <= base and a non-empty read
-            uint64_t base = c * 16 + j;
-            uint64_t lo = 0, hi = n_reads;  // find first r with offs[r] > base, answer r-1
-            while (lo < hi) {
-                uint64_t mid = (lo + hi) >> 1;
-                if (offs[mid] <= base) lo = mid + 1; else hi = mid;
-            }
-            frag_read[f] = (uint32_t)(lo - 1);
-            f++;
+// first[t] = the first read with offs[r] >= t * kPackTile (n_reads if none).
+__global__ void tile_reads_kernel(const uint64_t* __restrict__ offs, uint64_t n_reads, uint64_t n_tiles,
+                                  uint64_t* __restrict__ first) {
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n_tiles;
+         t += (uint64_t)gridDim.x * blockDim.x) {
+        uint64_t lo = 0, hi = n_reads;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if (offs[mid] < t * kPackTile) lo = mid + 1; else hi = mid;
         }
+        first[t] = lo;
     }
 }
 
-__global__ void compact_pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n_bases, bool vec,
-                                    const uint32_t* __restrict__ mask, const uint64_t* __restrict__ dst,
-                                    uint32_t* __restrict__ packed) {
-    uint64_t n_chunks = ceil_div(n_bases, 16);
-    for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < n_chunks;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t x[4], present;
-        load16(ascii, n_bases, c, vec, x, &present);
-        uint32_t m = mask[c];
-        if (!m) continue;
-        uint64_t pos = dst[c];
-        uint64_t w0 = pos >> 4;
-        uint32_t acc[2] = {0u, 0u};
+// A thread's chunk of tile t: its packed codes, valid bases and fragment
+// starts (a valid base at a read's start or after an invalid one).  Also the
+// starts of the tile's non-empty reads as bits in rs (after the barriers).
+__device__ __forceinline__ void tile_chunk(const uint8_t* __restrict__ ascii, uint64_t n_bases, bool vec,
+                                           const uint64_t* __restrict__ offs, uint64_t n_reads, uint64_t r0, uint64_t t,
+                                           uint32_t* rs, uint8_t* tops, uint32_t* codes, uint32_t* valid,
+                                           uint32_t* starts) {
+    const int tid = threadIdx.x;
+    const uint64_t base = t * kPackTile;
+    if (tid < (int)kPackTile / 32) rs[tid] = 0;
+    uint32_t x[4], present;
+    load16(ascii, n_bases, t * (kPackTile / 16) + tid, vec, x, &present);
+    uint32_t word = 0, m = 0;
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-            if (m & (1u << j)) {
-                uint32_t code = (codes4(x[j >> 2]) >> (8 * (j & 3))) & 3u;
-                uint64_t wi = (pos >> 4) - w0;
-                acc[wi] |= code << (30 - 2 * (pos & 15));
-                pos++;
-            }
+    for (int q = 0; q < 4; q++) {
+        word |= pack4(codes4(x[q])) << (24 - 8 * q);
+        m |= mask4(valid4(x[q])) << (4 * q);
+    }
+    m &= present;
+    tops[tid + 1] = (uint8_t)(m >> 15);
+    if (tid == 0) tops[0] = t ? (uint8_t)(valid4(ascii[base - 1]) & 1u) : 0;
+    __syncthreads();
+    for (uint64_t r = r0 + tid; r < n_reads; r += 256) {
+        const uint64_t o = offs[r];
+        if (o - base >= kPackTile) break;
+        if (offs[r + 1] > o) atomicOr(&rs[(o - base) >> 5], 1u << ((o - base) & 31));
+    }
+    __syncthreads();
+    const uint32_t rb = (rs[tid >> 1] >> (16 * (tid & 1))) & 0xFFFFu;
+    *codes = word;
+    *valid = m;
+    *starts = m & (rb | ~(m << 1 | tops[tid])) & 0xFFFFu;
+}
+
+__global__ void __launch_bounds__(256) tile_count_kernel(const uint8_t* __restrict__ ascii, uint64_t n_bases, bool vec,
+                                                         const uint64_t* __restrict__ offs, uint64_t n_reads,
+                                                         const uint64_t* __restrict__ first,
+                                                         uint32_t* __restrict__ n_valid,
+                                                         uint32_t* __restrict__ n_starts) {
+    __shared__ uint32_t rs[kPackTile / 32], ws[8];
+    __shared__ uint8_t tops[257];
+    uint32_t codes, m, fs;
+    tile_chunk(ascii, n_bases, vec, offs, n_reads, first[blockIdx.x], blockIdx.x, rs, tops, &codes, &m, &fs);
+    // (both counts at most 4,096: one sum)
+    const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(m) << 16 | __popc(fs));
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t all = 0;
+        for (int w = 0; w < 8; w++) all += ws[w];
+        n_valid[blockIdx.x] = all >> 16;
+        n_starts[blockIdx.x] = all & 0xFFFFu;
+    }
+}
+
+__global__ void __launch_bounds__(256) tile_pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n_bases, bool vec,
+                                                        const uint64_t* __restrict__ offs, uint64_t n_reads,
+                                                        const uint64_t* __restrict__ first,
+                                                        const uint64_t* __restrict__ dst,
+                                                        const uint64_t* __restrict__ fidx,
+                                                        uint64_t* __restrict__ frag_offs,
+                                                        uint32_t* __restrict__ frag_read,
+                                                        uint32_t* __restrict__ packed) {
+    __shared__ uint32_t rs[kPackTile / 32], before[kPackTile / 32], scratch[8];
+    __shared__ uint32_t read_of[kPackTile];  // the tile's non-empty reads, then its output words
+    __shared__ uint8_t tops[257];
+    const int tid = threadIdx.x;
+    const uint64_t t = blockIdx.x, base = t * kPackTile, r0 = first[t];
+    uint32_t codes, m, fs;
+    tile_chunk(ascii, n_bases, vec, offs, n_reads, r0, t, rs, tops, &codes, &m, &fs);
+    // reads that start before each word of rs (at most 128 words)
+    uint32_t all;
+    const uint32_t reads = block_excl_scan_256(tid < (int)kPackTile / 32 ? __popc(rs[tid]) : 0u, scratch, &all);
+    if (tid < (int)kPackTile / 32) before[tid] = reads;
+    uint32_t tot;
+    const uint32_t ex = block_excl_scan_256((uint32_t)__popc(m) << 16 | __popc(fs), scratch, &tot);
+    for (uint64_t r = r0 + tid; r < n_reads; r += 256) {
+        const uint64_t o = offs[r];
+        if (o - base >= kPackTile) break;
+        const uint32_t q = (uint32_t)(o - base);
+        if (offs[r + 1] > o) read_of[before[q >> 5] + __popc(rs[q >> 5] & ((1u << (q & 31)) - 1u))] = (uint32_t)r;
+    }
+    __syncthreads();
+    const uint64_t d0 = dst[t];
+    uint64_t f = fidx[t] + (ex & 0xFFFFu);
+    const uint32_t at = ex >> 16;  // the chunk's first valid base among the tile's
+    while (fs) {
+        const int j = __ffs(fs) - 1;
+        fs &= fs - 1;
+        const uint32_t q = tid * 16 + j;
+        const uint32_t rank = before[q >> 5] + __popc(rs[q >> 5] & (0xFFFFFFFFu >> (31 - (q & 31))));
+        frag_offs[f] = d0 + at + __popc(m & ((1u << j) - 1u));
+        frag_read[f] = rank ? read_of[rank - 1] : (uint32_t)(r0 - 1);
+        f++;
+    }
+    __syncthreads();
+    // the valid codes side by side, placed as in the output's words
+    uint32_t* out = read_of;
+    for (int i = tid; i < (int)kPackTile / 16 + 2; i += 256) out[i] = 0;
+    __syncthreads();
+    const uint32_t n = tot >> 16, shift = (uint32_t)(d0 & 15);
+    if (m) {
+        uint32_t w = codes;
+        for (uint32_t inv = ~m & 0xFFFFu; inv;) {  // the last invalid code taken out first
+            const int j = 31 - __clz(inv);
+            inv ^= 1u << j;
+            const uint32_t low = 0xFFFFFFFFu >> (2 * j);
+            w = (w & ~low) | (w << 2 & low);
         }
-        if (acc[0]) atomicOr(&packed[w0], acc[0]);
-        if (acc[1]) atomicOr(&packed[w0 + 1], acc[1]);
+        const uint32_t p = shift + at, o = 2 * (p & 15);
+        atomicOr(&out[p >> 4], w >> o);
+        if (o) atomicOr(&out[(p >> 4) + 1], w << (32 - o));
+    }
+    __syncthreads();
+    // the first and the last word may be shared with the tiles beside
+    const uint32_t words = n ? (shift + n + 15) / 16 : 0;
+    for (uint32_t i = tid; i < words; i += 256) {
+        if (i == 0 || i + 1 == words) atomicOr(&packed[d0 / 16 + i], out[i]);
+        else packed[d0 / 16 + i] = out[i];
     }
 }
 
@@ -227,32 +291,33 @@ void pack_reads(mh_ctx* ctx, const uint8_t* d_ascii, uint64_t n_bases, const uin
         return;
     }
     // compaction of valid bases and fragment discovery
-    Buf<uint32_t> mask(ctx, n_chunks), cnt(ctx, n_chunks), fcnt(ctx, n_chunks);
-    Buf<uint64_t> dst(ctx, n_chunks + 1), fidx(ctx, n_chunks + 1);
-    Buf<uint32_t> rs(ctx, ceil_div(n_bases, 32) + 1);
-    rs.zero();
-    MH_LAUNCH(ctx, "chunk_masks", grid_for(ctx, n_chunks, 256), 256, 0, chunk_masks_kernel, d_ascii, n_bases, vec,
-              mask.p, cnt.p);
-    exclusive_scan_u32(ctx, cnt.p, dst.p, n_chunks);
-    if (n_reads)
-        MH_LAUNCH(ctx, "read_starts", grid_for(ctx, n_reads, 256), 256, 0, read_starts_kernel, d_offs, n_reads, rs.p);
-    MH_LAUNCH(ctx, "frag_count", grid_for(ctx, n_chunks, 256), 256, 0, frag_count_kernel, mask.p, rs.p, n_chunks,
-              fcnt.p);
-    exclusive_scan_u32(ctx, fcnt.p, fidx.p, n_chunks);
+    packed.reset();
+    const uint64_t n_tiles = ceil_div(n_bases, (uint64_t)kPackTile);
+    Buf<uint64_t> first(ctx, n_tiles), dst(ctx, n_tiles + 1), fidx(ctx, n_tiles + 1);
+    Buf<uint32_t> n_valid(ctx, n_tiles), n_starts(ctx, n_tiles);
+    if (n_tiles) {
+        MH_LAUNCH(ctx, "tile_reads", grid_for(ctx, n_tiles, 256), 256, 0, tile_reads_kernel, d_offs, n_reads, n_tiles,
+                  first.p);
+        MH_LAUNCH_B(ctx, "tile_count", n_bases, (unsigned)n_tiles, 256, 0, tile_count_kernel, d_ascii, n_bases, vec,
+                    d_offs, n_reads, first.p, n_valid.p, n_starts.p);
+    }
+    exclusive_scan_u32(ctx, n_valid.p, dst.p, n_tiles);
+    exclusive_scan_u32(ctx, n_starts.p, fidx.p, n_tiles);
     uint64_t tot[2];
-    read_u64(ctx, dst.p + n_chunks, &tot[0], 1);
-    read_u64(ctx, fidx.p + n_chunks, &tot[1], 1);
+    Buf<uint64_t> both(ctx, 2);
+    MH_CUDA(cudaMemcpyAsync(both.p, dst.p + n_tiles, sizeof(uint64_t), cudaMemcpyDeviceToDevice, ctx->stream));
+    MH_CUDA(cudaMemcpyAsync(both.p + 1, fidx.p + n_tiles, sizeof(uint64_t), cudaMemcpyDeviceToDevice, ctx->stream));
+    read_u64(ctx, both.p, tot, 2);
     const uint64_t n_packed = tot[0], n_frags = tot[1];
     Buf<uint64_t> fo(ctx, n_frags + 1);
     Buf<uint32_t> fr(ctx, n_frags);
     Buf<uint32_t> cp(ctx, ceil_div(n_packed, 16) + kPackPad);
     cp.zero();
-    MH_LAUNCH(ctx, "frag_write", grid_for(ctx, n_chunks, 256), 256, 0, frag_write_kernel, mask.p, rs.p, dst.p, fidx.p,
-              d_offs, n_reads, n_chunks, fo.p, fr.p);
-    MH_CUDA(cudaMemcpyAsync(fo.p + n_frags, dst.p + n_chunks, sizeof(uint64_t), cudaMemcpyDeviceToDevice,
+    if (n_tiles)
+        MH_LAUNCH_B(ctx, "tile_pack", n_bases + n_packed / 4 + 12 * n_frags, (unsigned)n_tiles, 256, 0, tile_pack_kernel,
+                    d_ascii, n_bases, vec, d_offs, n_reads, first.p, dst.p, fidx.p, fo.p, fr.p, cp.p);
+    MH_CUDA(cudaMemcpyAsync(fo.p + n_frags, dst.p + n_tiles, sizeof(uint64_t), cudaMemcpyDeviceToDevice,
                             ctx->stream));
-    MH_LAUNCH(ctx, "compact_pack", grid_for(ctx, n_chunks, 256), 256, 0, compact_pack_kernel, d_ascii, n_bases, vec,
-              mask.p, dst.p, cp.p);
     sync_and_check(ctx);
     out->n_frags = n_frags;
     out->n_packed = n_packed;

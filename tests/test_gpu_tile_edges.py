@@ -74,3 +74,38 @@ def test_sorts_around_one_cta(k, n):
     rng = np.random.default_rng(n)
     a, o = synth.reads_from_strings([_dna(rng, k + 1) for _ in range(n)])
     assert _check(a, o, k, 1)[0] == 6 * n
+
+
+@pytest.mark.parametrize("where", ["inside", "edges", "empty_reads", "one_base_reads", "all_invalid", "long"])
+def test_pack_around_tiles(where):
+    # the compacting path works in tiles of 4,096 input bases, chunks of 16
+    import paper_1409_7208_gb300 as mh
+
+    rng = np.random.default_rng(9)
+    if where == "inside":
+        a, o = synth.random_reads(21, 2000, 0, 90, p_invalid=0.1)
+    elif where == "edges":
+        # reads and Ns at and beside the tiles' and chunks' ends
+        g = list(_dna(rng, 5 * 4096 + 7))
+        for p in (0, 15, 16, 31, 4095, 4096, 8190, 8191, 12287, 12289, 16384, len(g) - 1):
+            g[p] = "N"
+        g = "".join(g)
+        a, o = synth.reads_from_strings([g[:4096], g[4096:8191], g[8191:8193], g[8193:12288], g[12288:]])
+    elif where == "empty_reads":
+        a, o = synth.reads_from_strings([""] * 300 + [_dna(rng, 4096), ""] + [""] * 700 + [_dna(rng, 4095), "", "A", "", _dna(rng, 33)] + [""] * 5)
+    elif where == "one_base_reads":
+        a, o = synth.reads_from_strings(["ACGTN"[i] for i in rng.integers(0, 5, 9000)])
+    elif where == "all_invalid":
+        a, o = synth.reads_from_strings(["N" * 5000, "", "nnn."])
+    else:
+        g = _dna(rng, 30_000)
+        a, o = synth.reads_from_strings([g[:17_000] + "N" + g[17_000:]])
+    bases, fo, fr = oracle.fragments(a, o)
+    r = mh.mh_pack_reads(mh.Context(device=0), a, o).tensors()
+    assert (r["n_frags"], r["n_packed"]) == (len(fr), len(bases))
+    code = np.zeros(-(-len(bases) // 16) * 16, dtype=np.uint32)
+    code[:len(bases)] = np.searchsorted(np.frombuffer(b"ACGT", np.uint8), np.frombuffer(bytes(bases), np.uint8))
+    want = (code.reshape(-1, 16) << (30 - 2 * np.arange(16, dtype=np.uint32))).sum(axis=1, dtype=np.uint32)
+    assert np.array_equal(r["packed"].cpu().numpy().view(np.uint32)[:len(want)], want)
+    assert np.array_equal(r["frag_offs"].cpu().numpy().view(np.uint64), fo)
+    assert np.array_equal(r["frag_read"].cpu().numpy().view(np.uint32), fr)
