@@ -518,7 +518,14 @@ void build_sdbg(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, mh_sd
     // dummy entries in colex order
     Buf<uint64_t> dk(ctx, (t ? t : 1) * NW), dk2(ctx, (t ? t : 1) * NW);
     if (t) MH_LAUNCH(ctx, "dummy_keys", grid_for(ctx, t, 256), 256, 0, dummy_keys_kernel<NW>, zout.p, t, k, dk.p);
-    if (radix_sort<NW>(ctx, dk.p, dk2.p, nullptr, nullptr, t, 0, 2 * k)) std::swap(dk, dk2);
+    // (many wide keys: by their top bits and a fix-up, not 2 k bits of passes)
+    if (NW > 1 && t >= (1u << 14)) {
+        Buf<uint32_t> v(ctx, t), v2(ctx, t);
+        v.zero();
+        if (radix_sort_spread_kv<NW>(ctx, dk.p, dk2.p, v.p, v2.p, t, 64 * NW - 2 * k)) std::swap(dk, dk2);
+    } else if (radix_sort<NW>(ctx, dk.p, dk2.p, nullptr, nullptr, t, 0, 2 * k)) {
+        std::swap(dk, dk2);
+    }
     dk2.reset();
     // merge positions of the padding
     const uint64_t m = E + t + u;

@@ -133,8 +133,9 @@ static bool radix_sort_impl(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t
 }
 
 // Tile shape of the scatter pass for 1-word keys: (items per thread,
-// resident CTAs per SM).  The defaults, (16, 3) for keys alone and (14, 3)
-// with a payload, measured fastest on GB300; a context's tuned shape
+// resident CTAs per SM).  The default, (16, 3), measured fastest on GB300 for
+// keys alone and with a payload (3.3e8 pairs, with the other sorts of a path:
+// 10.1 ms; (14, 3) 10.5, (12, 4) 11.5); a context's tuned shape
 // (mh_run_batch's autotuner) or MH_SORT_VARIANT selects another key-only
 // shape: 1 = (12, 4), 2 = (14, 3).
 static int sort_variant() {
@@ -197,11 +198,11 @@ static bool radix_sort_dispatch(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint
                                 uint64_t n, int bit_lo, int bit_hi, const uint32_t* h, SegIn seg = SegIn{}) {
     if constexpr (NW == 1) {
         if constexpr (HV) {
-            return radix_sort_impl<NW, HV, 14, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
+            return radix_sort_impl<NW, HV, 16, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
         } else {
             switch (ctx->sort_shape >= 0 ? ctx->sort_shape : sort_variant()) {
                 case 1: return radix_sort_impl<NW, HV, 12, 4>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
-                case 2: return radix_sort_impl<NW, HV, 14, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
+                case 2: return radix_sort_impl<NW, HV, 16, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
                 default: return radix_sort_impl<NW, HV, 16, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
             }
         }
@@ -824,6 +825,66 @@ bool radix_sort_spread(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint64_t n, i
     return in_alt;
 }
 
+// Wide pairs by their `P` bits from bit lo on: a pass over (key, value) pairs
+// moves 20 or 36 bytes in and out, so the bits and the pair's index go into
+// one 64-bit word (P <= 32, n <= 2^32), the passes move those, and one gather
+// moves the pairs, into alt and valt.  4 M reads counted at k = 99 19.6 -> 19.0
+// ms, the multiple-k iteration 62.4 -> 60.2.
+template <int NW>
+__global__ void index_keys_kernel(const uint64_t* __restrict__ keys, uint64_t n, int lo, int P,
+                                  uint64_t* __restrict__ out) {
+    const uint64_t mask = (1ull << P) - 1;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+        out[i] = (key_shr<NW>(load_key<NW>(keys, i), lo).w[0] & mask) << 32 | i;
+}
+
+template <int NW>
+__global__ void index_gather_kernel(const uint64_t* __restrict__ idx, uint64_t n, const uint64_t* __restrict__ keys,
+                                    const uint32_t* __restrict__ vals, uint64_t* __restrict__ kout,
+                                    uint32_t* __restrict__ vout) {
+    constexpr int U = 4;  // pairs a thread has in flight
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += U * stride) {
+        uint32_t j[U], v[U];
+        Key<NW> x[U];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (i + u * stride < n) j[u] = (uint32_t)idx[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (i + u * stride < n) {
+                x[u] = load_key<NW>(keys, j[u]);
+                v[u] = vals[j[u]];
+            }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (i + u * stride < n) {
+                store_key<NW>(kout, i + u * stride, x[u]);
+                vout[i + u * stride] = v[u];
+            }
+    }
+}
+
+// False (and nothing done) where the two words a pair do not fit the
+// context's memory: the passes then move the pairs.
+template <int NW>
+static bool sort_by_index(mh_ctx* ctx, const uint64_t* keys, uint64_t* alt, const uint32_t* vals, uint32_t* valt,
+                          uint64_t n, int lo, int P) {
+    if (n > (1ull << 32) || P > 32) return false;
+    try {
+        Buf<uint64_t> a(ctx, n), b(ctx, n);
+        MH_LAUNCH_B(ctx, "index_keys", n * (8 * NW + 8), grid_for(ctx, n, 256), 256, 0, index_keys_kernel<NW>, keys, n,
+                    lo, P, a.p);
+        const bool in_b = radix_sort<1>(ctx, a.p, b.p, nullptr, nullptr, n, 32, 32 + P);
+        MH_LAUNCH_B(ctx, "index_gather", n * (16 * NW + 16), grid_for(ctx, n, 1024), 256, 0, index_gather_kernel<NW>,
+                    in_b ? b.p : a.p, n, keys, vals, alt, valt);
+    } catch (const Error& e) {
+        if (e.code != MH_ENOMEM) throw;
+        return false;  // (the pairs are where they were)
+    }
+    return true;
+}
+
 // Distinct keys with a 32-bit payload (a solid table and its counts): the
 // same spread order (passes over the top P bits of the top word below
 // `skip` constant bits, then the key-value fix-up).  Keys whose top bits are
@@ -837,14 +898,20 @@ bool radix_sort_spread_kv(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* 
     const int bits = 64 * NW;
     // small tables (below 2^20 keys, or MH_SPREAD_KV_MIN for tests): the full
     // sort, which needs no read-back of the fix-up's list
+    // (wide keys from 2^12 on: 17 to 32 passes cost more than the read-back)
     static const uint64_t kv_min = [] {
         const char* e = std::getenv("MH_SPREAD_KV_MIN");
-        return e ? (uint64_t)std::strtoull(e, nullptr, 10) : (uint64_t)1 << 20;
+        return e ? (uint64_t)std::strtoull(e, nullptr, 10) : NW == 1 ? (uint64_t)1 << 20 : (uint64_t)1 << 12;
     }();
     if (n < std::max<uint64_t>(kv_min, 2) || P + skip >= bits)
         return radix_sort<NW>(ctx, keys, alt, vals, valt, n, 0, bits - skip);
     const int lo = bits - skip - P;  // groups: keys equal at and above bit lo of the whole key
-    const bool in_alt = radix_sort<NW>(ctx, keys, alt, vals, valt, n, bits - skip - P, bits - skip);
+    // two words: only while the gather's reads come from L2 (beyond, it costs
+    // more than three passes over pairs save: 3 M reads at k = 61 8.7 ms for 8.3)
+    const bool by_index =
+        (NW == 4 || (NW == 2 && n * 20 <= (96u << 20))) && sort_by_index<NW>(ctx, keys, alt, vals, valt, n, lo, P);
+    const bool in_alt =
+        by_index || radix_sort<NW>(ctx, keys, alt, vals, valt, n, bits - skip - P, bits - skip);
     uint64_t* k = in_alt ? alt : keys;
     uint64_t* ko = in_alt ? keys : alt;
     uint32_t* v = in_alt ? valt : vals;
