@@ -15,21 +15,38 @@ namespace mh {
 // byte codes: A/a 0, C/c 1, G/g 2, T/t 3 (((c >> 1) ^ (c >> 2)) & 3 on those letters)
 __device__ __forceinline__ uint32_t codes4(uint32_t x) { return ((x >> 1) ^ (x >> 2)) & 0x03030303u; }
 
-// 0xFF in each byte lane holding one of ACGTacgt
-__device__ __forceinline__ uint32_t valid4(uint32_t x) {
-    uint32_t u = x & 0xDFDFDFDFu;
-    return __vcmpeq4(u, 0x41414141u) | __vcmpeq4(u, 0x43434343u) | __vcmpeq4(u, 0x47474747u) |
-           __vcmpeq4(u, 0x54545454u);
+// The letters (upper case) of four codes: the codes as nibbles select bytes.
+__device__ __forceinline__ uint32_t letters4(uint32_t c) {
+    return __byte_perm(0x54474341u, 0, __byte_perm(c | c >> 4, 0, 0x4420));
 }
 
-// codes of 4 bytes (byte 0 = first base) -> 8 bits, first base most significant
-__device__ __forceinline__ uint32_t pack4(uint32_t c) {
-    return ((c & 3u) << 6) | (((c >> 8) & 3u) << 4) | (((c >> 16) & 3u) << 2) | ((c >> 24) & 3u);
-}
+// Zero in each byte lane holding one of ACGTacgt: a byte is a base if it is
+// the letter of the code that it would have.
+__device__ __forceinline__ uint32_t invalid4(uint32_t x) { return letters4(codes4(x)) ^ (x & 0xDFDFDFDFu); }
 
 // valid lanes (0xFF bytes) -> 4-bit mask, bit j = byte j
 __device__ __forceinline__ uint32_t mask4(uint32_t v) {
     return (v & 1u) | ((v >> 7) & 2u) | ((v >> 14) & 4u) | ((v >> 21) & 8u);
+}
+
+// 16 bytes -> the packed word of their codes (first base most significant;
+// four codes go to the top byte of a product) and the mask of the valid ones.
+// Some 50 instructions for bases alone, where byte compares took 150.
+__device__ __forceinline__ void encode16(const uint32_t x[4], uint32_t* word, uint32_t* valid) {
+    uint32_t p[4], d[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const uint32_t c = codes4(x[q]);
+        p[q] = c * 0x40100401u;  // 2^30 + 2^20 + 2^10 + 1
+        d[q] = letters4(c) ^ (x[q] & 0xDFDFDFDFu);
+    }
+    *word = __byte_perm(__byte_perm(p[3], p[2], 0x73), __byte_perm(p[1], p[0], 0x73), 0x5410);
+    *valid = 0xFFFFu;
+    if (d[0] | d[1] | d[2] | d[3]) {
+        *valid = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) *valid |= mask4(__vcmpeq4(d[q], 0u)) << (4 * q);
+    }
 }
 
 // Load the 16 bytes of chunk c as four words (zero past n_bases).
@@ -65,16 +82,13 @@ __global__ void pack_chunks_kernel(const uint8_t* __restrict__ ascii, uint64_t n
     const uint64_t n_chunks = ceil_div(n_bases, 16), stride = (uint64_t)gridDim.x * blockDim.x;
     bool bad = false;
     auto pack = [&](uint64_t c, const uint32_t x[4], uint32_t present) {
-        uint32_t word = 0, vmask = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            word |= pack4(codes4(x[q])) << (24 - 8 * q);
-            vmask |= mask4(valid4(x[q])) << (4 * q);
-        }
+        uint32_t word, vmask;
+        encode16(x, &word, &vmask);
         packed[c] = word;
         bad |= (vmask & present) != present;
     };
-    // four loads in flight a thread (one: 3 Gbp 1.71 ms, four 1.59)
+    // four loads in flight a thread (3 Gbp 0.61 ms; with byte compares and one load
+    // 1.71, four loads 1.59)
     constexpr int U = 4;
     uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     for (; c + (U - 1) * stride < n_chunks; c += U * stride) {
@@ -118,7 +132,7 @@ __global__ void iota_u32_kernel(uint32_t* __restrict__ a, uint64_t n) {
 // them again, writes the fragments and sets the valid codes side by side in
 // shared memory.  A tile reads its reads' starts once, so a fragment's read
 // comes from a rank among them.  Two sweeps of 16-byte loads and one small
-// scan, bound by memory latency; 5 M trimmed reads with Ns (450 Mbp): 0.92 ms,
+// scan, bound by memory latency; 5 M trimmed reads with Ns (450 Mbp): 0.76 ms,
 // where masks, counts and prefixes a chunk in memory and a bisection of all
 // offsets a fragment took 2.0 ms.
 constexpr uint32_t kPackTile = 4096;
@@ -149,15 +163,11 @@ __device__ __forceinline__ void tile_chunk(const uint8_t* __restrict__ ascii, ui
     if (tid < (int)kPackTile / 32) rs[tid] = 0;
     uint32_t x[4], present;
     load16(ascii, n_bases, t * (kPackTile / 16) + tid, vec, x, &present);
-    uint32_t word = 0, m = 0;
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        word |= pack4(codes4(x[q])) << (24 - 8 * q);
-        m |= mask4(valid4(x[q])) << (4 * q);
-    }
+    uint32_t word, m;
+    encode16(x, &word, &m);
     m &= present;
     tops[tid + 1] = (uint8_t)(m >> 15);
-    if (tid == 0) tops[0] = t ? (uint8_t)(valid4(ascii[base - 1]) & 1u) : 0;
+    if (tid == 0) tops[0] = t && !(invalid4(ascii[base - 1]) & 0xFFu) ? 1 : 0;
     __syncthreads();
     for (uint64_t r = r0 + tid; r < n_reads; r += 256) {
         const uint64_t o = offs[r];
