@@ -12,7 +12,7 @@
 // and an error word) lives in one statically sized device array in this file.
 //
 // That array is a module global: every GPU that loads the library holds it
-// (kScratchBytes, about 17 MiB) until the process exits, and every call on
+// (kScratchBytes, about 18 MiB) until the process exits, and every call on
 // a device shares the same copy.  Each call clears the parts that must start
 // at zero; calls that overlap on the GPU (on different streams, or from
 // several threads without ordering) race on the array and must not be made.
@@ -35,17 +35,17 @@ namespace {
 constexpr uint64_t kMaxKeyWords = 1ull << 21;                  // n * nw limit: 16 MiB of keys
 constexpr uint64_t kAltBytes = kMaxKeyWords * 8;               // ping-pong buffer
 constexpr uint64_t kMaxTiles = 1ull << 10;                     // >= ceil(limit / tile) for every nw
-constexpr uint64_t kStatusBytes = kMaxTiles * 256 * 4;         // look-back status
+constexpr uint64_t kStatusBytes = 2 * kMaxTiles * 256 * 4;     // look-back status of two passes
 constexpr int kMaxPasses = 32;                                 // 256-bit keys, 8-bit digits
 constexpr uint64_t kHistBytes = kMaxPasses * 256 * 4;
 constexpr uint64_t kBaseBytes = kMaxPasses * 256 * 8;
-constexpr uint64_t kMiscBytes = 256;                           // tile counter, error word
+constexpr uint64_t kMiscBytes = 256;                           // error word, the passes' tile counters
 constexpr uint64_t kAltOff = 0;
 constexpr uint64_t kStatusOff = kAltOff + kAltBytes;
-constexpr uint64_t kHistOff = kStatusOff + kStatusBytes;
+constexpr uint64_t kMiscOff = kStatusOff + kStatusBytes;
+constexpr uint64_t kHistOff = kMiscOff + kMiscBytes;           // (cleared together with what is before)
 constexpr uint64_t kBaseOff = kHistOff + kHistBytes;
-constexpr uint64_t kMiscOff = kBaseOff + kBaseBytes;
-constexpr uint64_t kScratchBytes = kMiscOff + kMiscBytes;
+constexpr uint64_t kScratchBytes = kBaseOff + kBaseBytes;
 static_assert(kMaxTiles * (uint64_t)sort_tile<4>() >= kMaxKeyWords / 4, "status too small for nw = 4");
 static_assert(kMaxTiles * (uint64_t)sort_tile<2>() >= kMaxKeyWords / 2, "status too small for nw = 2");
 static_assert(kMaxTiles * (uint64_t)sort_tile<1>() >= kMaxKeyWords, "status too small for nw = 1");
@@ -112,16 +112,16 @@ static int scratch_address(void** out) {
     return MH_OK;
 }
 
-template <int NW>
+template <int NW, int ITEMS>
 static int sort_noalloc(const uint64_t* in, uint64_t* out, uint64_t n, int key_bits, cudaStream_t st,
                         unsigned char* scratch) {
-    constexpr int TILE = sort_tile<NW>();
+    constexpr int TILE = sort_tile<NW, ITEMS>();
     uint64_t* alt = reinterpret_cast<uint64_t*>(scratch + kAltOff);
     uint32_t* status = reinterpret_cast<uint32_t*>(scratch + kStatusOff);
     uint32_t* hist = reinterpret_cast<uint32_t*>(scratch + kHistOff);
     uint64_t* base = reinterpret_cast<uint64_t*>(scratch + kBaseOff);
-    uint32_t* counter = reinterpret_cast<uint32_t*>(scratch + kMiscOff);
-    uint32_t* err = counter + 1;
+    uint32_t* err = reinterpret_cast<uint32_t*>(scratch + kMiscOff);
+    uint32_t* counter = err + 1;
     const int n_passes = (key_bits + 7) / 8;
     const uint64_t tiles = ceil_div(n, TILE);
 #define MH_TRY(call)                                    \
@@ -131,29 +131,31 @@ static int sort_noalloc(const uint64_t* in, uint64_t* out, uint64_t n, int key_b
             return MH_EDEVICE;                          \
         }                                               \
     } while (0)
-    // hist and the error word must start at zero; status and the tile
-    // counter are cleared before every pass
-    MH_TRY(cudaMemsetAsync(hist, 0, kHistBytes, st));
-    MH_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), st));
+    // the histogram, the error word, the passes' tile counters and the first
+    // pass's status words start at zero (two parts, so that a small sort
+    // clears little); a pass's tiles clear the next one's status words
+    MH_TRY(cudaMemsetAsync(status, 0, tiles * 256 * sizeof(uint32_t), st));
+    MH_TRY(cudaMemsetAsync(err, 0, kMiscBytes + (uint64_t)n_passes * 256 * sizeof(uint32_t), st));
     int dev = 0, sms = 1;
     MH_TRY(cudaGetDevice(&dev));
     MH_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    unsigned hist_grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(ceil_div(n, 256), (uint64_t)sms * 4));
+    // (every CTA adds its counts to all digits of all passes)
+    unsigned hist_grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(ceil_div(n, 2048), (uint64_t)sms * 2));
     radix_hist_kernel<NW><<<hist_grid, 256, sizeof(uint32_t) * n_passes * 256, st>>>(in, n, 0, n_passes, hist);
     MH_TRY(cudaGetLastError());
     radix_base_kernel<<<n_passes, 256, 0, st>>>(hist, base, 256);
     MH_TRY(cudaGetLastError());
-    constexpr size_t smem = onesweep_smem<NW, false>();
-    MH_TRY(cudaFuncSetAttribute(onesweep_kernel<NW, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    constexpr size_t smem = onesweep_smem<NW, false, ITEMS>();
+    MH_TRY(cudaFuncSetAttribute(onesweep_kernel<NW, false, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const uint64_t* src = in;
     for (int p = 0; p < n_passes; p++) {
         // the last pass writes `out`; the ones before alternate so that it does
         uint64_t* dst = ((n_passes - 1 - p) % 2 == 0) ? out : alt;
-        MH_TRY(cudaMemsetAsync(status, 0, tiles * 256 * sizeof(uint32_t), st));
-        MH_TRY(cudaMemsetAsync(counter, 0, sizeof(uint32_t), st));
-        onesweep_kernel<NW, false><<<(unsigned)tiles, kSortThreads, smem, st>>>(
-            src, dst, nullptr, nullptr, n, 8 * p, base + (uint64_t)p * 256, nullptr, status, counter, err,
-            kSpinLimit, 0, SegIn{});
+        uint32_t* now = status + (uint64_t)(p & 1) * kMaxTiles * 256;
+        uint32_t* next = status + (uint64_t)(~p & 1) * kMaxTiles * 256;
+        onesweep_kernel<NW, false, ITEMS><<<(unsigned)tiles, kSortThreads, smem, st>>>(
+            src, dst, nullptr, nullptr, n, 8 * p, base + (uint64_t)p * 256, nullptr, now, counter + p, err,
+            kSpinLimit, 0, SegIn{}, next);
         MH_TRY(cudaGetLastError());
         src = dst;
     }
@@ -189,9 +191,14 @@ extern "C" int mh_sort_keys_noalloc(const uint64_t* keys_in, uint64_t* keys_out,
     int rc = scratch_address(&scratch);
     if (rc != MH_OK) return rc;
     unsigned char* s = static_cast<unsigned char*>(scratch);
+    // Up to 2^19 words of keys in small tiles (1,024 words), so that a pass has
+    // tiles for every SM: 300,007 keys of 62 bits in 293 tiles 134 us, where
+    // the 74 tiles of the large sorts, each pass's two clears and a look-back of
+    // one tile at a time took 184.
+    const bool small = n * (uint64_t)nw <= (1u << 19);
     switch (nw) {
-        case 1: return sort_noalloc<1>(keys_in, keys_out, n, key_bits, st, s);
-        case 2: return sort_noalloc<2>(keys_in, keys_out, n, key_bits, st, s);
-        default: return sort_noalloc<4>(keys_in, keys_out, n, key_bits, st, s);
+        case 1: return (small ? sort_noalloc<1, 4> : sort_noalloc<1, SortItems<1>::v>)(keys_in, keys_out, n, key_bits, st, s);
+        case 2: return (small ? sort_noalloc<2, 2> : sort_noalloc<2, SortItems<2>::v>)(keys_in, keys_out, n, key_bits, st, s);
+        default: return (small ? sort_noalloc<4, 1> : sort_noalloc<4, SortItems<4>::v>)(keys_in, keys_out, n, key_bits, st, s);
     }
 }

@@ -13,6 +13,7 @@ constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagInc = 2u << 30;
 constexpr uint32_t kCountMask = (1u << 30) - 1;
 constexpr int kSpinLimit = 1 << 23;  // default bound of a look-back wait (polls)
+constexpr int kLookBack = 8;         // earlier tiles read at once
 
 template <int NW>
 struct SortItems;
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(kSortThreads, MINB)
                     uint32_t* __restrict__ vout, uint64_t n, int shift, const uint64_t* __restrict__ digit_base,
                     uint64_t* __restrict__ next_base, uint32_t* __restrict__ status,
                     uint32_t* __restrict__ tile_counter, uint32_t* __restrict__ err, int spin_limit,
-                    int withhold_first, SegIn seg) {
+                    int withhold_first, SegIn seg, uint32_t* __restrict__ clear = nullptr) {
     constexpr int TILE = sort_tile<NW, ITEMS>();
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* warp_hist = reinterpret_cast<uint32_t*>(smem);          // [warps][256]
@@ -139,6 +140,7 @@ __global__ void __launch_bounds__(kSortThreads, MINB)
     for (int i = tid; i < kSortWarps * 256; i += kSortThreads) warp_hist[i] = 0;
     __syncthreads();
     const uint32_t tile = misc[0];
+    if (clear) clear[(uint64_t)tile * 256 + tid] = 0;  // the next pass's status words
     const uint64_t tile_base = (uint64_t)tile * TILE;
     const uint64_t rem = n - tile_base;
     const uint32_t tile_n = rem < (uint64_t)TILE ? (uint32_t)rem : (uint32_t)TILE;
@@ -250,27 +252,37 @@ __global__ void __launch_bounds__(kSortThreads, MINB)
             if constexpr (HV) vstage[slot] = v[i];
         }
     }
-    // look back over earlier tiles for this digit
+    // look back over earlier tiles for this digit, kLookBack of them at a
+    // time: one by one, each step is a read's latency, and tiles that start
+    // together walk back over each other
     uint64_t excl = 0;
     if (tile > 0) {
         int64_t j = (int64_t)tile - 1;
-        bool ok = true;
-        while (j >= 0) {
-            const uint32_t* sp = status + (uint64_t)j * 256 + d;
-            uint32_t s = ld_relaxed_u32(sp);
-            int spins = 0;
-            while ((s & ~kCountMask) == 0) {
+        bool ok = true, done = false;
+        int spins = 0;
+        while (!done) {
+            uint32_t s[kLookBack];
+#pragma unroll
+            for (int q = 0; q < kLookBack; q++)
+                s[q] = j >= q ? ld_relaxed_u32(status + (uint64_t)(j - q) * 256 + d) : kFlagInc;
+            bool all = true;  // all before s[q] are published
+#pragma unroll
+            for (int q = 0; q < kLookBack; q++) {
+                all = all && !done && (s[q] & ~kCountMask) != 0;
+                if (all) {
+                    excl += s[q] & kCountMask;
+                    done = (s[q] & ~kCountMask) == kFlagInc;
+                    j--;
+                    spins = 0;
+                }
+            }
+            if (!done && !all) {
                 if (++spins > spin_limit) {
                     ok = false;
                     break;
                 }
                 if (spins > 64) __nanosleep(128);
-                s = ld_relaxed_u32(sp);
             }
-            if (!ok) break;
-            excl += s & kCountMask;
-            if ((s & ~kCountMask) == kFlagInc) break;
-            j--;
         }
         if (!ok) atomicOr(err, ST_SPIN_TIMEOUT);
         st_relaxed_u32(st, kFlagInc | (uint32_t)((excl + cnt) & kCountMask));
