@@ -348,9 +348,10 @@ __global__ void symbol_starts_kernel(const uint64_t* __restrict__ ck, uint64_t E
 // the same label; a group holds at most 16) and whether it ends its node from
 // the neighbours, and a warp's ballots are words of the bit-vectors.
 // Reads each key once from memory (the neighbours come from L1) and writes
-// each output once; bound by the loads in flight (four keys a thread at five
-// CTAs an SM: eight at two took 2.7 ms for 3.5e8 edges).  3.5e8 edges of one
-// word: 1.8 ms, where flags, insertion counts, their scan, bytes and their
+// each output once; bound by the loads in flight (one word: two keys a thread
+// at eight CTAs an SM; four at five 1.8 ms for 3.5e8 edges, eight at two 2.7;
+// two words: two at five, 0.34 ms for 4.1e7, at eight 0.37).  3.5e8 edges of
+// one word: 1.6 ms, where flags, insertion counts, their scan, bytes and their
 // packing (53 bytes an edge) took 6.5; build of 3 M reads at k = 47 with
 // multiplicities: 0.34 ms.
 constexpr int kEmitTile = 2048;
@@ -372,7 +373,7 @@ __global__ void emit_bounds_kernel(const uint64_t* __restrict__ pos_d, uint64_t 
 }
 
 template <int NW>
-__global__ void __launch_bounds__(256, NW == 4 ? 3 : 5) emit_kernel(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cv,
+__global__ void __launch_bounds__(256, NW == 1 ? 8 : NW == 2 ? 5 : 3) emit_kernel(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cv,
                                                    uint64_t E, const uint64_t* __restrict__ dk, uint64_t t,
                                                    const uint64_t* __restrict__ pos_d,
                                                    const uint64_t* __restrict__ pos_u, uint64_t m,
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(256, NW == 4 ? 3 : 5) emit_kernel(const uint64
                                                    uint32_t* __restrict__ valid, uint32_t* __restrict__ mult,
                                                    unsigned long long* __restrict__ n_last) {
     constexpr int kWords = kEmitTile / 32;  // 32 positions each, eight a warp
-    constexpr int U = NW == 1 ? 4 : 2;
+    constexpr int U = 2;
     __shared__ uint8_t pad[kEmitTile];      // where pmask is set: W code, bit 4 last, bit 5 dummy
     __shared__ uint32_t pmask[kWords], pre[kWords], sum_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -18,8 +18,8 @@
 //            out once
 //
 // Reads and writes every key once; bound by the shared-memory reads and the
-// waits of the serial merges.  3.5e8 edges of one word: 5.4 ms with the
-// splitters, where writing the colex keys and a tree of three two-way merges
+// waits of the serial merges (seven CTAs an SM; six 0.3 ms more, four keys a
+// thread 1.8 more).  3.5e8 edges of one word: 5.0 ms with the splitters, where writing the colex keys and a tree of three two-way merges
 // (64 bytes an edge) took 7.1; build of 3 M reads at k = 47 with
 // multiplicities: 1.24 for 1.74.
 #include "mh_internal.cuh"
@@ -167,7 +167,7 @@ __global__ void colex_bounds_kernel(ColexView<NW> v, const ColexRuns* __restrict
 }
 
 template <int NW, bool HV>
-__global__ void __launch_bounds__(256) colex_merge_kernel(ColexView<NW> v, const ColexRuns* __restrict__ runs,
+__global__ void __launch_bounds__(256, NW == 4 ? 4 : 7) colex_merge_kernel(ColexView<NW> v, const ColexRuns* __restrict__ runs,
                                                           const uint64_t* __restrict__ bnd, uint64_t* __restrict__ ck,
                                                           uint32_t* __restrict__ cv, uint32_t* __restrict__ err) {
     using C = Colex<NW>;
