@@ -34,11 +34,12 @@
 // records and 4 of outputs instead of 8 to 32 a pass.  Equal records are
 // counted once with their number (keys of one word: their records are short
 // against a read, so most recur whole), which at 3 Gbp and k = 31 takes the
-// count from 24.6 to 21.4 ms; for wider keys most runs end with their read,
+// count from 24.6 to 21.4 ms (20.3 since bins without a palindrome skip the
+// search for them); for wider keys most runs end with their read,
 // and it would cost more than it saves.  3 Gbp, k = 31, 2.38 G windows: split
-// 7.4 ms (67 thread instructions a position), count 21.4, where the
+// 7.3 ms (67 thread instructions a position), count 20.3, where the
 // extraction, two passes, the units and their compaction took 18.8 + 28 + 22.3
-// + 5.2; 3 M reads of 100-150 bp at k = 61: 5.6 ms for 15.2.
+// + 5.2; 3 M reads of 100-150 bp at k = 61: 4.5 ms for 15.2.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
     constexpr int T = kSplitTile;
     constexpr uint32_t mask = M == 16 ? 0xFFFFFFFFu : (1u << (2 * M)) - 1u;
     __shared__ uint32_t words[kSplitWords];
-    __shared__ uint32_t hash[kHashPad];                // then the runs' minima
+    __shared__ __align__(16) uint32_t hash[kHashPad];  // then the positions' minima
     __shared__ uint32_t bmin[(T + kSplitHalo) / 8];
     __shared__ uint32_t inv[T / 32], stop[T / 32];     // no window starts here; a run ends before here
     __shared__ uint16_t hpos[kSplitMaxRecs];
@@ -199,18 +200,14 @@ __global__ void __launch_bounds__(256) super_split_kernel(const uint32_t* __rest
     reinterpret_cast<uint8_t*>(stop)[tid] = (uint8_t)(hm | ~vb);
     uint32_t total;
     uint32_t at = block_excl_scan_256(__popc(hm), scratch, &total);
-#pragma unroll
-    for (int i = 0; i < 8; i++)
-        if ((hm >> i) & 1u) {
-            hpos[at] = (uint16_t)(tid * 8 + i);
-            hash[at] = mh[i];
-            at++;
-        }
+    reinterpret_cast<uint4*>(hash)[2 * tid] = make_uint4(mh[0], mh[1], mh[2], mh[3]);
+    reinterpret_cast<uint4*>(hash)[2 * tid + 1] = make_uint4(mh[4], mh[5], mh[6], mh[7]);
+    for (uint32_t left = hm; left; left &= left - 1) hpos[at++] = (uint16_t)(tid * 8 + __ffs(left) - 1);
     __syncthreads();
     // a thread per run
     for (uint32_t j = tid; j < total; j += 256) {
         const uint32_t q = hpos[j];
-        const uint32_t b = __umulhi(super_mix(hash[j]), n_bins);
+        const uint32_t b = __umulhi(super_mix(hash[q]), n_bins);
         // (a run of more windows than a record may have, in a repeat, gives
         // several)
         uint32_t left = next_bit(stop, q + 1, T) - q, at = 0;
@@ -358,7 +355,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + L::kCnt);
     uint32_t* sym = reinterpret_cast<uint32_t*>(smem + L::kSym);
     uint32_t* start = reinterpret_cast<uint32_t*>(smem + L::kStart);
-    __shared__ uint32_t over;
+    __shared__ uint32_t over, any_palin;
     __shared__ uint32_t scratch[8], wsol[8], went[8];
     __shared__ uint64_t base[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -465,7 +462,10 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     };
     auto next_hot = [&]() -> uint32_t { return (uint32_t)(next_have >> 32) > (NW == 1 ? min(hot, 0xFFFFu) : hot); };
     fetch(b0 + blockIdx.x);
-    if (tid == 0) over = next_hot();
+    if (tid == 0) {
+        over = next_hot();
+        any_palin = 0;
+    }
     for (int i = tid; i < C::kSlots / 2; i += 256)
         reinterpret_cast<ulonglong2*>(fp)[i] = make_ulonglong2(kEmpty, kEmpty);
     for (int i = tid; i < C::kSlots / (NW == 1 ? 8 : 4); i += 256)
@@ -635,6 +635,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                     for (int i = 0; i < NW; i++) rc.w[i] = rev2_u64(~x.w[NW - 1 - i]);
                     rc = key_low<NW>(rc, 2 * K1);
                     x = key_shr<NW>(x, 64 * NW - 2 * K1);
+                    if (key_eq<NW>(rc, x)) any_palin = 1;
                     insert(mix_key<NW>(key_less<NW>(rc, x) ? rc : x), L::kAlike ? mul[id] : 1u);
                 }
             }
@@ -652,6 +653,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
             return m;
         };
         constexpr int WW = C::kWords / 8;
+        const bool pal = any_palin != 0;  // (few bins hold a palindrome)
         uint32_t mine = 0, no = 0, my_occ = 0, my_pre = 0, my_palins = 0;
 #pragma unroll
         for (int q = 0; q < WW; q++) {
@@ -663,11 +665,11 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                 my_pre = mine;
             }
             mine += __popc(m);
-            // kept keys of both strands (an odd window is no palindrome)
-            if (K1 & 1) no += 2 * __popc(__ballot_sync(0xFFFFFFFFu, lit && lit >= (uint32_t)d));
+            // kept keys of both strands
+            if (!pal) no += 2 * __popc(__ballot_sync(0xFFFFFFFFu, lit && lit >= (uint32_t)d));
         }
         __syncwarp();
-        if (!(K1 & 1))
+        if (pal)
             for (uint32_t e0 = 0; e0 < mine; e0 += 32) {
                 const uint32_t e = e0 + lane;
                 bool pl = false;
@@ -715,7 +717,10 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
             }
             clear();
             __syncthreads();
-            if (tid == 0) over = next_hot();
+            if (tid == 0) {
+                over = next_hot();
+                any_palin = 0;
+            }
             continue;
         }
         palins += my_palins;
@@ -727,7 +732,10 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
         }
         if (lane < WW) sidx[(uint64_t)b * C::kWords + warp * WW + lane] = make_uint2(my_occ, pe + my_pre);
         __syncthreads();
-        if (tid == 0) over = next_hot();
+        if (tid == 0) {
+            over = next_hot();
+            any_palin = 0;
+        }
         // (past a buffer's end nothing is written: the host sees the totals)
         if (base[0] + ne <= spec_cap && base[1] + to <= solid_cap) {
             uint64_t so = base[1] + po;
@@ -745,7 +753,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                     spec_len[eo + e] = lit;
                     x = unmix_key<NW>(m);
                     r = key_rc<NW>(x, K1);
-                    pl = key_eq<NW>(r, x);
+                    pl = pal && key_eq<NW>(r, x);
                     if (pl) lit *= 2;
                 }
                 const bool keep = e < mine && lit >= (uint32_t)d;
