@@ -34,10 +34,10 @@
 // records and 4 of outputs instead of 8 to 32 a pass.  Equal records are
 // counted once with their number (keys of one word: their records are short
 // against a read, so most recur whole), which at 3 Gbp and k = 31 takes the
-// count from 24.6 to 21.4 ms (20.3 since bins without a palindrome skip the
-// search for them); for wider keys most runs end with their read,
+// count from 24.6 to 21.4 ms (18.9 since bins without a palindrome skip the
+// search for them and a lane lists 16 slots at once); for wider keys most runs end with their read,
 // and it would cost more than it saves.  3 Gbp, k = 31, 2.38 G windows: split
-// 7.3 ms (67 thread instructions a position), count 20.3, where the
+// 7.3 ms (67 thread instructions a position), count 18.9, where the
 // extraction, two passes, the units and their compaction took 18.8 + 28 + 22.3
 // + 5.2; 3 M reads of 100-150 bp at k = 61: 4.5 ms for 15.2.
 #include <algorithm>
@@ -655,18 +655,49 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
         constexpr int WW = C::kWords / 8;
         const bool pal = any_palin != 0;  // (few bins hold a palindrome)
         uint32_t mine = 0, no = 0, my_occ = 0, my_pre = 0, my_palins = 0;
+        if constexpr (NW == 1) {
+            // 16 slots a lane (two reads of eight 16-bit counts)
+            static_assert(L::kRegion == 512 && WW == 16, "16 slots a lane");
+            const uint4* c4 = reinterpret_cast<const uint4*>(cnt) + warp * 64 + lane * 2;
+            const uint4 u = c4[0], v = c4[1];
+            const uint32_t c[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+            uint32_t m = 0;
 #pragma unroll
-        for (int q = 0; q < WW; q++) {
-            const uint32_t s = (warp * WW + q) * 32 + lane, lit = count_at(s);
-            const uint32_t m = __ballot_sync(0xFFFFFFFFu, lit != 0), at = mine + __popc(m & lt);
-            if (lit) list[at] = (uint16_t)s;
-            if (lane == q) {
-                my_occ = m;
-                my_pre = mine;
+            for (int i = 0; i < 8; i++) {
+                const uint32_t r = __vminu2(c[i], 0x00010001u);
+                m |= ((r | r >> 15) & 3u) << (2 * i);
             }
-            mine += __popc(m);
-            // kept keys of both strands
-            if (!pal) no += 2 * __popc(__ballot_sync(0xFFFFFFFFu, lit && lit >= (uint32_t)d));
+            uint32_t incl = __popc(m);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t ex = incl - __popc(m);
+            mine = __shfl_sync(0xFFFFFFFFu, incl, 31);
+            uint32_t at = ex, kept = 0;
+            for (uint32_t left = m; left; left &= left - 1) {
+                const uint32_t s = warp * 512 + lane * 16 + __ffs(left) - 1;
+                list[at++] = (uint16_t)s;
+                kept += count_at(s) >= (uint32_t)d;
+            }
+            if (!pal) no = 2 * __reduce_add_sync(0xFFFFFFFFu, kept);
+            my_occ = __shfl_sync(0xFFFFFFFFu, m, 2 * lane) | __shfl_sync(0xFFFFFFFFu, m, 2 * lane + 1) << 16;
+            my_pre = __shfl_sync(0xFFFFFFFFu, ex, 2 * lane);
+        } else {
+#pragma unroll
+            for (int q = 0; q < WW; q++) {
+                const uint32_t s = (warp * WW + q) * 32 + lane, lit = count_at(s);
+                const uint32_t m = __ballot_sync(0xFFFFFFFFu, lit != 0), at = mine + __popc(m & lt);
+                if (lit) list[at] = (uint16_t)s;
+                if (lane == q) {
+                    my_occ = m;
+                    my_pre = mine;
+                }
+                mine += __popc(m);
+                // kept keys of both strands
+                if (!pal) no += 2 * __popc(__ballot_sync(0xFFFFFFFFu, lit && lit >= (uint32_t)d));
+            }
         }
         __syncwarp();
         if (pal)
