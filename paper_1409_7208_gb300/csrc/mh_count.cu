@@ -950,7 +950,7 @@ void count_kmers(mh_ctx* ctx, const mh_reads* reads, int k, int d, mh_kmers* out
     out->n_kmers = 2 * n;
     out->spectrum_mixed = kMixed;
     const int bb = count_bucket_bits(ctx, n, NW);
-    if (bb == 0 && use_unit_count(ctx) && use_super(n, k + 1)) {
+    if (bb == 0 && use_unit_count(ctx) && use_super(ctx, n, k + 1)) {
         woff.reset();
         super_count<NW>(ctx, reads, k, d, n, out);
         return;
