@@ -410,7 +410,7 @@ int mh_set_count_plan(mh_ctx* ctx, const mh_count_plan* plan);
  * memory budget, or code that must never enter the driver's allocator or
  * synchronise the device the way cudaFree does.  It calls no cudaMalloc,
  * cudaFree or other allocating routine; all scratch space is one static
- * device array of about 17 MiB that every device loading the library keeps
+ * device array of about 18 MiB that every device loading the library keeps
  * until exit.
  *   * limit: n * nw <= 2^21 words (16 MiB of keys); larger inputs return
  *     MH_EOVERFLOW and touch nothing;

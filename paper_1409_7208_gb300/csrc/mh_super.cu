@@ -853,8 +853,8 @@ static long env_long(const char* name, long dflt) {
 // passes (whole path, windows x 10^3, unit route and this one in ms: k = 31
 // 38 1.04 0.87, 376 1.28 1.05, 4,700 1.56 1.25; k = 47 62 1.34 1.02, 1,950
 // 1.63 1.23).  Windows of more symbols leave bins to the rest: k = 63 248 1.48
-// 1.58; k = 61 1,600 1.73 1.77; k = 99 2,600 2.45 2.65.  A plan set for the unit
-// route, or a variable that steers it, keeps it below 2^22.  MH_SUPER=0 turns
+// 1.58; k = 61 1,600 1.73 1.77; k = 99 2,600 2.45 2.65.  A plan that moves the
+// unit bits, or a variable that steers the unit route, keeps it below 2^22.  MH_SUPER=0 turns
 // this route off, =1 on at any size (tests).  The counters of a bin hold 32
 // bits each, so fewer than 2^32 windows.
 bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
@@ -866,7 +866,7 @@ bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
     }();
     if (v == 0 || !n || n >= (1ull << 32) || super_m(K1) == 0) return false;
     if (v == 1 || n >= (1ull << 22)) return true;
-    return K1 <= 48 && !steered && ctx->count_path < 0 && ctx->unit_bits_delta == 0;
+    return K1 <= 48 && !steered && ctx->unit_bits_delta == 0;
 }
 
 template <int NW>
