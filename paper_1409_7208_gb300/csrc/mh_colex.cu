@@ -19,9 +19,9 @@
 //
 // Reads and writes every key once; bound by the shared-memory reads and the
 // waits of the serial merges (seven CTAs an SM; six 0.3 ms more, four keys a
-// thread 1.8 more).  3.5e8 edges of one word: 5.0 ms with the splitters, where writing the colex keys and a tree of three two-way merges
-// (64 bytes an edge) took 7.1; build of 3 M reads at k = 47 with
-// multiplicities: 1.24 for 1.74.
+// thread 1.8 more).  3.5e8 edges of one word: 5.0 ms with the splitters, where
+// writing the colex keys and a tree of three two-way merges (64 bytes an edge)
+// took 7.1; build of 3 M reads at k = 47 with multiplicities: 1.24 for 1.74.
 #include "mh_internal.cuh"
 
 namespace mh {

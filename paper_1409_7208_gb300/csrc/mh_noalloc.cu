@@ -191,14 +191,14 @@ extern "C" int mh_sort_keys_noalloc(const uint64_t* keys_in, uint64_t* keys_out,
     int rc = scratch_address(&scratch);
     if (rc != MH_OK) return rc;
     unsigned char* s = static_cast<unsigned char*>(scratch);
-    // Up to 2^19 words of keys in small tiles (1,024 words), so that a pass has
-    // tiles for every SM: 300,007 keys of 62 bits in 293 tiles 134 us, where
-    // the 74 tiles of the large sorts, each pass's two clears and a look-back of
-    // one tile at a time took 184.
+    // Up to 2^19 words of keys in small tiles (2,048 words), so that a pass has
+    // tiles for every SM: 300,007 keys of 62 bits in 147 tiles 125 us (in 293
+    // of 1,024 words 134), where the 74 tiles of the large sorts, each pass's
+    // two clears and a look-back of one tile at a time took 184.
     const bool small = n * (uint64_t)nw <= (1u << 19);
     switch (nw) {
-        case 1: return (small ? sort_noalloc<1, 4> : sort_noalloc<1, SortItems<1>::v>)(keys_in, keys_out, n, key_bits, st, s);
-        case 2: return (small ? sort_noalloc<2, 2> : sort_noalloc<2, SortItems<2>::v>)(keys_in, keys_out, n, key_bits, st, s);
-        default: return (small ? sort_noalloc<4, 1> : sort_noalloc<4, SortItems<4>::v>)(keys_in, keys_out, n, key_bits, st, s);
+        case 1: return (small ? sort_noalloc<1, 8> : sort_noalloc<1, SortItems<1>::v>)(keys_in, keys_out, n, key_bits, st, s);
+        case 2: return (small ? sort_noalloc<2, 4> : sort_noalloc<2, SortItems<2>::v>)(keys_in, keys_out, n, key_bits, st, s);
+        default: return (small ? sort_noalloc<4, 2> : sort_noalloc<4, SortItems<4>::v>)(keys_in, keys_out, n, key_bits, st, s);
     }
 }
