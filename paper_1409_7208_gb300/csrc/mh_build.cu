@@ -78,7 +78,9 @@ template <int NW>
 struct ZeroTile {
     static constexpr int kItems = 8 / NW;             // entries a thread
     static constexpr int kCap = 256 * kItems;
-    static constexpr int kTile = kCap - 16;           // a group holds at most 16 entries
+    // a group holds at most 16 edges, each once a table: a solid and a mercy
+    // table that share edges are built too
+    static constexpr int kTile = kCap - 32;
 };
 
 // st[t] = the first group start at or after t * kTile (t = 0..n_tiles; E at
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(256, NW == 4 ? 4 : 8) zero_out_kernel(const ui
     uint8_t* left = reinterpret_cast<uint8_t*>(gm);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t t = blockIdx.x, s0 = st[t];
-    const uint32_t n = (uint32_t)min(st[t + 1] - s0, (uint64_t)Z::kCap);  // at most kTile + 15
+    const uint32_t n = (uint32_t)min(st[t + 1] - s0, (uint64_t)Z::kCap);  // at most kTile + 31
     // groups, numbered in order: a warp 32 I entries, 32 at a time
     uint32_t ng = 0;
     {
