@@ -993,6 +993,26 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     }
     uint64_t R = h[T_SPEC], S = h[T_SOLID], runs = R, palins = h[T_PALIN];
     const uint64_t n_main = R;
+    // the outputs' buffers grow by the rest, or shrink if much too large
+    auto fit = [&](Buf<uint64_t>& kb, Buf<uint32_t>& cb, uint64_t have, uint64_t& have_cap, const Buf<uint64_t>& rk,
+                   const Buf<uint32_t>& rcnt, uint64_t more) {
+        const uint64_t need = have + more;
+        if (need > have_cap || have_cap > need + need / 4 + 4096) {
+            Buf<uint64_t> k2(ctx, (need ? need : 1) * NW);
+            Buf<uint32_t> c2(ctx, need ? need : 1);
+            if (have) {
+                MH_CUDA(cudaMemcpyAsync(k2.p, kb.p, have * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+                MH_CUDA(cudaMemcpyAsync(c2.p, cb.p, have * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+            }
+            kb = std::move(k2);
+            cb = std::move(c2);
+            have_cap = need;
+        }
+        if (more) {
+            MH_CUDA(cudaMemcpyAsync(kb.p + have * NW, rk.p, more * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+            MH_CUDA(cudaMemcpyAsync(cb.p + have, rcnt.p, more * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+        }
+    };
     // the deferred bins, by the unit counting
     RunList rest;
     Buf<uint64_t> rest_k;
@@ -1000,6 +1020,15 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     uint64_t rest_S = 0;
     if (h[T_DEF]) {
         const uint64_t nd = h[T_DEFWIN];
+        // what the rest takes (keys twice, lengths, slots of kept pairs)
+        // beside outputs with room for all windows can pass the 24 NW + 12
+        // bytes a window that the caller's memory plan counts on: the outputs
+        // are then made to fit first (else once, with the rest; it is a copy)
+        const uint64_t pair = 8 * NW + 4;
+        if ((spec_cap + solid_cap) * pair + nd * (16 * NW + 4 + per * pair) > n * (24 * NW + 12)) {
+            fit(spec, spec_len, n_main, spec_cap, rest_k, rest_c, 0);
+            fit(solid, solid_c, h[T_SOLID], solid_cap, rest_k, rest_c, 0);
+        }
         Buf<uint64_t> keys(ctx, nd * NW), alt(ctx, nd * NW);
         Buf<unsigned long long> cursor(ctx, h[T_DEF]);
         cursor.zero();
@@ -1027,25 +1056,6 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     off.reset();
     bins.reset();
     deferred.reset();
-    // the outputs' buffers grow by the rest, or shrink if much too large
-    auto fit = [&](Buf<uint64_t>& kb, Buf<uint32_t>& cb, uint64_t have, uint64_t have_cap, const Buf<uint64_t>& rk,
-                   const Buf<uint32_t>& rcnt, uint64_t more) {
-        const uint64_t need = have + more;
-        if (need > have_cap || have_cap > need + need / 4 + 4096) {
-            Buf<uint64_t> k2(ctx, (need ? need : 1) * NW);
-            Buf<uint32_t> c2(ctx, need ? need : 1);
-            if (have) {
-                MH_CUDA(cudaMemcpyAsync(k2.p, kb.p, have * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-                MH_CUDA(cudaMemcpyAsync(c2.p, cb.p, have * 4, cudaMemcpyDeviceToDevice, ctx->stream));
-            }
-            kb = std::move(k2);
-            cb = std::move(c2);
-        }
-        if (more) {
-            MH_CUDA(cudaMemcpyAsync(kb.p + have * NW, rk.p, more * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-            MH_CUDA(cudaMemcpyAsync(cb.p + have, rcnt.p, more * 4, cudaMemcpyDeviceToDevice, ctx->stream));
-        }
-    };
     fit(spec, spec_len, n_main, spec_cap, rest.keys, rest.lens, rest.n);
     fit(solid, solid_c, h[T_SOLID], solid_cap, rest_k, rest_c, rest_S);
     rest.keys.reset();

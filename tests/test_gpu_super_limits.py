@@ -1,0 +1,44 @@
+"""Limits of counting by super-k-mers: the memory it takes where its bins do
+not fit their tables (every bin left to the unit counting by MH_SUPER_HOT=0)."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _child(code, args, env):
+    p = subprocess.run([sys.executable, "-c", "import sys; sys.path.insert(0, %r)\n" % ROOT + code] + [str(a) for a in args],
+                       env=dict(os.environ, **env), capture_output=True, text=True, timeout=900)
+    assert p.returncode == 0, p.stdout + p.stderr
+    return p.stdout.split()
+
+
+BUDGET = r"""
+import hashlib
+import synth, paper_1409_7208_gb300 as mh
+k = int(sys.argv[1])
+# little sequence: nearly every window is one of a few thousand
+a, o = synth.uniform_genome_reads(k, 2000, 60_000, 150, 0.0005)
+n = 60_000 * (150 - k)
+nw = 1 if k <= 31 else 2 if k <= 63 else 4
+# the least budget that counts in memory: 24 nw + 12 bytes a window within 90 % of it
+budget = int(n * 1.05 * (24 * nw + 12) / 0.9) + (1 << 20)
+reads = mh.mh_pack_reads(mh.Context(device=0), a, o)
+ctx = mh.Context(device=0, hbm_budget=budget, profile=True)
+s = mh.mh_count_kmers(ctx, reads, k, 2)
+g, peak, prof = s.numpy(), ctx.memory()[1], ctx.profile()
+assert peak <= budget and "bucket_hist" not in prof
+print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), "super_expand" in prof)
+"""
+
+
+@pytest.mark.parametrize("k", [31, 47, 99])
+def test_all_bins_left_over_fit_the_in_memory_budget(k):
+    old = _child(BUDGET, [k], {"MH_SUPER": "0"})
+    new = _child(BUDGET, [k], {"MH_SUPER": "1", "MH_SUPER_HOT": "0"})
+    assert new[0] == old[0] and (new[1], old[1]) == ("True", "False")
