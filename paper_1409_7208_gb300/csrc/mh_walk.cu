@@ -344,7 +344,7 @@ static bool use_links(const mh_ctx* ctx, uint64_t E, uint64_t n_walks, uint64_t 
         const uint64_t rounds = ceil_div(n_walks, (uint64_t)ctx->num_sms * 64);
         if (E > 20000 * max_len * rounds) return false;
     }
-    // 40 bytes an edge: within a budget that has room for it
+    // 40 bytes an edge, beside the index: within a budget that may have room for it
     return !ctx->budget || ctx->in_use + 40 * E + n_walks * (max_len / 4 + 64) < ctx->budget;
 }
 
@@ -358,31 +358,48 @@ void walk_contigs(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, uin
     bool linked = n_walks && use_links(ctx, E, n_walks, max_len);
     Buf<uint4> link;
     Buf<uint2> a, b, c;
-    if (linked) {
-        try {
+    Buf<uint8_t> slots;
+    Buf<uint64_t> lens, off, offS, offM;
+    uint64_t stride = 0;  // of a walk's slot, in words or bytes
+    int bits = 1;
+    auto take = [&] {
+        stride = linked ? ceil_div(max_len, 16) : max_len;
+        // bucket indexes over the top bits: about 16 entries a bucket (a
+        // thread searching for links: 4)
+        const uint64_t per = linked ? 4 : 16;
+        bits = 1;
+        while (bits < 32 && bits < 2 * (k + 1) && (2ull << bits) * per <= std::max(nS, nM)) bits++;
+        if (linked) {
             link = Buf<uint4>(ctx, E);
             a = Buf<uint2>(ctx, E);
             b = Buf<uint2>(ctx, E);
             c = Buf<uint2>(ctx, E);
-        } catch (const Error& e) {
-            // no room for them: the walks need none
-            if (e.code != MH_ENOMEM) throw;
-            link.reset();
-            a.reset();
-            b.reset();
-            linked = false;
         }
+        slots = Buf<uint8_t>(ctx, n_walks * stride * (linked ? 4 : 1));
+        lens = Buf<uint64_t>(ctx, n_walks + 1);
+        off = Buf<uint64_t>(ctx, n_walks + 1);
+        if (n_walks) {
+            offS = Buf<uint64_t>(ctx, (1ull << bits) + 1);
+            offM = Buf<uint64_t>(ctx, (1ull << bits) + 1);
+        }
+    };
+    try {
+        take();
+    } catch (const Error& e) {
+        // no room for the links and what they are made with: the walks need none
+        if (!linked || e.code != MH_ENOMEM) throw;
+        link.reset();
+        a.reset();
+        b.reset();
+        c.reset();
+        slots.reset();
+        lens.reset();
+        off.reset();
+        offS.reset();
+        linked = false;
+        take();
     }
-    const uint64_t stride = linked ? ceil_div(max_len, 16) : max_len;  // of a walk's slot, in words or bytes
-    Buf<uint8_t> slots(ctx, n_walks * stride * (linked ? 4 : 1));
-    Buf<uint64_t> lens(ctx, n_walks + 1), off(ctx, n_walks + 1);
-    // bucket indexes over the top bits: about 16 entries a bucket (a thread
-    // searching for links: 4)
-    const uint64_t per = linked ? 4 : 16;
-    int bits = 1;
-    while (bits < 32 && bits < 2 * (k + 1) && (2ull << bits) * per <= std::max(nS, nM)) bits++;
     if (n_walks) {
-        Buf<uint64_t> offS(ctx, (1ull << bits) + 1), offM(ctx, (1ull << bits) + 1);
         if (nS)
             MH_LAUNCH(ctx, "walk_index", grid_for(ctx, nS, 256), 256, 0, table_index_kernel<NW>, solid->keys, nS,
                       k + 1, bits, offS.p);
@@ -416,6 +433,8 @@ void walk_contigs(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, uin
     a.reset();
     b.reset();
     c.reset();
+    offS.reset();
+    offM.reset();
     exclusive_scan_u64(ctx, lens.p, off.p, n_walks);
     uint64_t total = 0;
     read_u64(ctx, off.p + n_walks, &total, 1);
