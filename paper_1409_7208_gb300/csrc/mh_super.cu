@@ -876,7 +876,13 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     // tests: bins of more windows than MH_SUPER_HOT, or with a key that finds
     // no place in MH_SUPER_PROBES slots, are left to the rest
     static const uint32_t hot = (uint32_t)std::max(0l, env_long("MH_SUPER_HOT", 1 << 16));
-    static const int probes = (int)std::max(1l, std::min(256l, env_long("MH_SUPER_PROBES", 128)));
+    static const int most_probes = (int)std::max(1l, std::min(256l, env_long("MH_SUPER_PROBES", 128)));
+    // tests: the first buffers for the other bins of a sampled set hold
+    // MH_SUPER_ESTIMATE percent of the estimate (no slack), and the limit on
+    // probes holds for them alone, so that the second time round bins are in
+    // place that the first left to the rest
+    static const long estimate = env_long("MH_SUPER_ESTIMATE", 0);
+    int probes = estimate ? 128 : most_probes;
     const uint64_t F = reads->n_frags, n_words = ceil_div(reads->n_packed, 16) + kPackPad;
     const uint64_t n_tiles = ceil_div(reads->n_packed, (uint64_t)kSplitTile);
     const uint32_t n_bins = (uint32_t)std::max<uint64_t>(1, n / C::kTarget);
@@ -970,8 +976,13 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         const double f = (double)n_bins / nb1;
         uint64_t a = std::min<uint64_t>(n, (uint64_t)(1.04 * f * (double)a1) + (1u << 20));
         uint64_t s = std::min<uint64_t>(n * per, (uint64_t)(1.04 * f * (double)o1) + (1u << 20));
+        if (estimate) {
+            a = std::max(a1, (uint64_t)(f * (double)a1) * estimate / 100);
+            s = std::max(o1, (uint64_t)(f * (double)o1) * estimate / 100);
+        }
         const std::vector<uint64_t> h1(h, h + T_N);
         for (int attempt = 0;; attempt++) {
+            probes = estimate && attempt ? 128 : most_probes;
             room(a, s);
             if (a1) {
                 MH_CUDA(cudaMemcpyAsync(spec.p, k1.p, a1 * NW * 8, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -985,8 +996,10 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
             read_u64(ctx, totals.p, h, T_N);
             if (h[T_SPEC] <= a && h[T_SOLID] <= s) break;
             if (attempt) fail(MH_EDEVICE, "super-k-mer outputs overflow twice");
-            a = h[T_SPEC];
-            s = h[T_SOLID];
+            // (which bins are left to the rest depends on the order of their
+            // insertions: those left out now may be in place the next time)
+            a = std::min(n, h[T_SPEC] + h[T_DEFWIN]);
+            s = std::min(n * per, h[T_SOLID] + per * h[T_DEFWIN]);
             MH_CUDA(cudaMemcpyAsync(totals.p, h1.data(), sizeof(uint64_t) * T_N, cudaMemcpyHostToDevice, ctx->stream));
             sync_and_check(ctx);
         }

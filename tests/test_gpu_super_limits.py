@@ -1,5 +1,7 @@
 """Limits of counting by super-k-mers: the memory it takes where its bins do
-not fit their tables (every bin left to the unit counting by MH_SUPER_HOT=0)."""
+not fit their tables (every bin left to the unit counting by MH_SUPER_HOT=0), and outputs whose
+sizes were estimated too small (MH_SUPER_ESTIMATE: a share of the estimate,
+and more bins left over in the first attempt than in the second)."""
 import os
 import subprocess
 import sys
@@ -42,3 +44,24 @@ def test_all_bins_left_over_fit_the_in_memory_budget(k):
     old = _child(BUDGET, [k], {"MH_SUPER": "0"})
     new = _child(BUDGET, [k], {"MH_SUPER": "1", "MH_SUPER_HOT": "0"})
     assert new[0] == old[0] and (new[1], old[1]) == ("True", "False")
+
+
+SAMPLED = r"""
+import hashlib
+import synth, paper_1409_7208_gb300 as mh
+k, n_reads = int(sys.argv[1]), int(sys.argv[2])
+a, o = synth.uniform_genome_reads(k, 3_000_000, n_reads, 150, 0.01)
+ctx = mh.Context(device=0, profile=True)
+s = mh.mh_count_kmers(ctx, mh.mh_pack_reads(ctx, a, o), k, 2)
+g = s.numpy()
+print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), s.view().n_distinct, ctx.profile()["super_count"][0])
+"""
+
+
+@pytest.mark.parametrize("k,n_reads", [(31, 300_000), (61, 400_000)])
+@pytest.mark.parametrize("probes", [6, 10, 128])
+def test_outputs_sized_too_small_are_made_again(k, n_reads, probes):
+    # above 2^25 windows: the first bins counted, the others, the others again
+    want = _child(SAMPLED, [k, n_reads], {})
+    got = _child(SAMPLED, [k, n_reads], {"MH_SUPER_ESTIMATE": "1", "MH_SUPER_PROBES": str(probes)})
+    assert got[:2] == want[:2] and (want[2], got[2]) == ("2", "3")
