@@ -933,14 +933,18 @@ static uint64_t scatter_cap(uint64_t n) {
 template <int NW>
 void count_kmers(mh_ctx* ctx, const mh_reads* reads, int k, int d, mh_kmers* out) {
     const uint64_t F = reads->n_frags;
-    Buf<uint64_t> nwin(ctx, F + 1), woff(ctx, F + 1);
-    if (F)
-        MH_LAUNCH(ctx, "frag_windows", grid_for(ctx, F, 256), 256, 0, frag_windows_kernel, reads->frag_offs, F, k,
-                  nwin.p);
-    exclusive_scan_u64(ctx, nwin.p, woff.p, F);
+    Buf<uint64_t> woff;
+    auto windows = [&] {
+        Buf<uint64_t> nwin(ctx, F + 1);
+        woff = Buf<uint64_t>(ctx, F + 1);
+        if (F)
+            MH_LAUNCH(ctx, "frag_windows", grid_for(ctx, F, 256), 256, 0, frag_windows_kernel, reads->frag_offs, F, k,
+                      nwin.p);
+        exclusive_scan_u64(ctx, nwin.p, woff.p, F);
+    };
+    windows();
     uint64_t n;
     read_u64(ctx, woff.p + F, &n, 1);
-    nwin.reset();
     // keys are sorted as mix_key images: their evenly spread top bits let
     // the sort run its passes over the top ceil(log2 n) bits only
     constexpr bool kMixed = true;
@@ -952,8 +956,8 @@ void count_kmers(mh_ctx* ctx, const mh_reads* reads, int k, int d, mh_kmers* out
     const int bb = count_bucket_bits(ctx, n, NW);
     if (bb == 0 && use_unit_count(ctx) && use_super(ctx, n, k + 1)) {
         woff.reset();
-        super_count<NW>(ctx, reads, k, d, n, out);
-        return;
+        if (super_count<NW>(ctx, reads, k, d, n, out)) return;
+        windows();
     }
     const GroupPlan gp = group_plan(ctx, n, 0, NW);
     if (bb == 0 && use_unit_count(ctx) && gp.passes >= 0) {

@@ -59,7 +59,7 @@ constexpr int kHashPad = (kSplitTile + kSplitHalo) / 8 * 9;  // one word of padd
 constexpr int kNwinBits = 12;                         // a record: start << 12 | windows (at most 2,048)
 static_assert(kSplitTile < (1 << kNwinBits), "a run fits a record");
 
-enum { T_SPEC = 0, T_SOLID = 1, T_PALIN = 2, T_DEF = 3, T_DEFWIN = 4, T_RECS = 5, T_N = 6 };
+enum { T_SPEC = 0, T_SOLID = 1, T_PALIN = 2, T_DEF = 3, T_DEFWIN = 4, T_RECS = 5, T_DONE = 6, T_LOST = 7, T_N = 8 };
 
 }  // namespace
 
@@ -329,6 +329,23 @@ struct SuperSmem {
     static_assert(kSym % 16 == 0 && kOwn % 16 == 0, "aligned");
 };
 
+// Whether w windows left to the rest of `done` counted or left are so many
+// that the set had better be counted by units: more than 2 in 5 of two words,
+// 13 in 20 of four.  What is left over is written out as keys, sorted, counted
+// and merged, which costs more a window than the units do at once, and the
+// time for its insertions is lost.  By unit counting and by bins with what they
+// leave over, two words (k = 47 and 61, 30 to 10,000 times a genome): 4.7 and
+// 4.3 ms with 22 % of the windows left over, 7.2 and 6.2 with 18 %, 3.4 and 4.2
+// with 44 %, 13.5 and 20.7 with 79 %; four words (k = 99): 8.5 and 6.3 with
+// 42 %, 3.2 and 3.4 with 46 %, 4.8 and 5.5 with 58 %, 13.3 and 19.0 with 71 %,
+// where giving up costs 0.3 to 0.8 ms.  One word (k = 31): 13.4 and 12.9 with
+// 63 %, so those never give up.
+constexpr uint32_t kLostBins = 32;
+template <int NW>
+__host__ __device__ bool super_lost(uint64_t w, uint64_t done) {
+    return NW == 2 ? 5 * w > 2 * done : 20 * w > 13 * done;
+}
+
 // A CTA per bin.  The table's first word is a mixed key's top word (the whole
 // key of one word); kEmpty marks a free slot: the mixed image of the
 // all-ones key, which is not canonical, for one word (wider keys whose top
@@ -336,11 +353,13 @@ struct SuperSmem {
 // stored beside it by the lane that claimed the slot, which then sets the
 // count's top bit; a lane that finds its top word waits for that bit
 // (bounded) and compares the rest.  A key that finds no place within
-// probe_max slots leaves the bin to the rest, as do more than kMost entries.
+// probe_max slots leaves the bin to the rest, as do more than kMost entries;
+// where that takes too much of a set of give_up windows, the CTAs stop and
+// totals[T_LOST] says so (0: they never do).
 template <int NW>
 __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     super_count_kernel(const uint32_t* __restrict__ packed, SuperRecs recs, uint32_t b0, uint32_t b1,
-                       uint64_t rec_cap, int K1, int d,
+                       uint64_t rec_cap, int K1, int d, uint64_t give_up,
                        uint32_t hot, int probe_max, uint64_t spec_cap, uint64_t* __restrict__ spec_k,
                        uint32_t* __restrict__ spec_len, uint64_t solid_cap, uint64_t* __restrict__ solid_k,
                        uint32_t* __restrict__ solid_c, uint64_t* __restrict__ soff, uint2* __restrict__ sidx,
@@ -355,7 +374,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + L::kCnt);
     uint32_t* sym = reinterpret_cast<uint32_t*>(smem + L::kSym);
     uint32_t* start = reinterpret_cast<uint32_t*>(smem + L::kStart);
-    __shared__ uint32_t over, any_palin;
+    __shared__ uint32_t over, any_palin, lost;
     __shared__ uint32_t scratch[8], wsol[8], went[8];
     __shared__ uint64_t base[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -465,6 +484,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     if (tid == 0) {
         over = next_hot();
         any_palin = 0;
+        lost = 0;
     }
     for (int i = tid; i < C::kSlots / 2; i += 256)
         reinterpret_cast<ulonglong2*>(fp)[i] = make_ulonglong2(kEmpty, kEmpty);
@@ -744,10 +764,17 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
             if (tid == 0) {
                 soff[b] = kSuperDeferred;
                 const uint64_t q = atomicAdd(&totals[T_DEF], 1ull);
-                deferred[q] = make_ulonglong2(b, atomicAdd(&totals[T_DEFWIN], (unsigned long long)W));
+                const uint64_t w = atomicAdd(&totals[T_DEFWIN], (unsigned long long)W);
+                deferred[q] = make_ulonglong2(b, w);
+                if (give_up) {
+                    const uint64_t done = atomicAdd(&totals[T_DONE], (unsigned long long)W);
+                    if (q >= kLostBins && w > give_up / 16 && super_lost<NW>(w, done)) totals[T_LOST] = 1;
+                    lost = *(volatile unsigned long long*)&totals[T_LOST] != 0;
+                }
             }
             clear();
             __syncthreads();
+            if (lost) break;
             if (tid == 0) {
                 over = next_hot();
                 any_palin = 0;
@@ -760,6 +787,7 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
             base[0] = atomicAdd(&totals[T_SPEC], (unsigned long long)ne);
             base[1] = atomicAdd(&totals[T_SOLID], (unsigned long long)to);
             soff[b] = base[0];
+            if (give_up) atomicAdd(&totals[T_DONE], (unsigned long long)W);
         }
         if (lane < WW) sidx[(uint64_t)b * C::kWords + warp * WW + lane] = make_uint2(my_occ, pe + my_pre);
         __syncthreads();
@@ -855,10 +883,15 @@ static long env_long(const char* name, long dflt) {
 // 1.63 1.23).  Windows of more symbols leave bins to the rest: k = 63 248 1.48
 // 1.58; k = 61 1,600 1.73 1.77; k = 99 2,600 2.45 2.65.  A plan that moves the
 // unit bits, or a variable that steers the unit route, keeps it below 2^22.  MH_SUPER=0 turns
-// this route off, =1 on at any size (tests).  The counters of a bin hold 32
+// this route off, =1 on at any size and whatever is left to the rest (tests).  The counters of a bin hold 32
 // bits each, so fewer than 2^32 windows.
-bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
+static long super_switch() {
     static const long v = env_long("MH_SUPER", -1);
+    return v;
+}
+
+bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
+    const long v = super_switch();
     static const bool steered = [] {
         for (const char* e : {"MH_GROUP_CAP", "MH_GROUP_UNIT_BITS", "MH_EXTRACT_SCATTER", "MH_SCATTER_CAP", "MH_SORT_CHUNK_TILES"})
             if (std::getenv(e)) return true;
@@ -870,7 +903,7 @@ bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
 }
 
 template <int NW>
-void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, mh_kmers* out) {
+bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, mh_kmers* out) {
     using C = SuperCfg<NW>;
     const int K1 = k + 1, m = super_m(K1), w = K1 - m + 1;
     // tests: bins of more windows than MH_SUPER_HOT, or with a key that finds
@@ -886,18 +919,20 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     const uint64_t F = reads->n_frags, n_words = ceil_div(reads->n_packed, 16) + kPackPad;
     const uint64_t n_tiles = ceil_div(reads->n_packed, (uint64_t)kSplitTile);
     const uint32_t n_bins = (uint32_t)std::max<uint64_t>(1, n / C::kTarget);
+    const uint64_t give_up = NW > 1 && super_switch() != 1 ? n : 0;
     Buf<uint64_t> first(ctx, n_tiles), off(ctx, (uint64_t)n_bins + 1), totals(ctx, 8);
     Buf<unsigned long long> bins(ctx, n_bins);
     MH_LAUNCH(ctx, "super_tiles", grid_for(ctx, n_tiles, 256), 256, 0, super_tiles_kernel, reads->frag_offs, F,
               n_tiles, first.p);
     // records: 2 / (w + 1) a window for random sequences (about 8 / w by
     // halves), one more a fragment and a tile; each bin has slots for half as
-    // many again as its share, and the list of those past them room for a
-    // quarter of all (again with room for what there is, if there are more)
+    // many again as its share, and the list of those past them room for all:
+    // where few minimizers take most windows it gets most records (again
+    // with room for what there is, if there are still more)
     const double run = super_half(K1) ? w / 8.0 : (w + 1) / 2.0;
     const uint64_t expect = std::min(n, (uint64_t)((double)n / run) + F + n_tiles + 1);
     const uint32_t slots = (uint32_t)((double)expect / n_bins * 1.5) + 16;
-    uint64_t cap = expect / 4 + 4096;
+    uint64_t cap = expect + 4096;
     Buf<uint64_t> rec(ctx, (uint64_t)n_bins * slots);
     unsigned long long* tot = reinterpret_cast<unsigned long long*>(totals.p);
     Buf<uint64_t> more;
@@ -916,7 +951,8 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     auto count = [&](uint32_t b0, uint32_t b1) {
         if (b0 < b1)
             MH_LAUNCH_B(ctx, "super_count", n / 4, (unsigned)std::min<uint64_t>(b1 - b0, (uint64_t)ctx->num_sms * std::max(1, per_sm)),
-                        256, smem, super_count_kernel<NW>, reads->packed, recs, b0, b1, cap, K1, d, hot,
+                        256, smem, super_count_kernel<NW>, reads->packed, recs, b0, b1, cap, K1, d,
+                        give_up, hot,
                         probes, spec_cap, spec.p, spec_len.p, solid_cap, solid.p, solid_c.p, soff.p, sidx.p,
                         deferred.p, tot);
     };
@@ -961,12 +997,14 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         room(std::max<uint64_t>(n1, 1), std::max<uint64_t>(n1 * per, 1));
         count(0, nb1);
         read_u64(ctx, totals.p, h, T_N);
+        if (h[T_LOST]) return false;
         if (h[T_RECS] <= cap && h[T_SPEC] <= spec_cap && h[T_SOLID] <= solid_cap) break;
         if (attempt >= 2) fail(MH_EDEVICE, "super-k-mer records overflow again");
         all = h[T_RECS] <= cap;
         cap = std::max(cap, h[T_RECS]);
     }
     if (sample) {
+        if (give_up && h[T_DEF] > kLostBins && super_lost<NW>(h[T_DEFWIN], h[T_DONE])) return false;
         // the other bins into buffers sized by the first ones (bins are by
         // hash: alike but for chance and the heavy ones), then the first
         // ones' entries in front of them
@@ -994,6 +1032,7 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
             }
             count(nb1, n_bins);
             read_u64(ctx, totals.p, h, T_N);
+            if (h[T_LOST]) return false;
             if (h[T_SPEC] <= a && h[T_SOLID] <= s) break;
             if (attempt) fail(MH_EDEVICE, "super-k-mer outputs overflow twice");
             // (which bins are left to the rest depends on the order of their
@@ -1096,10 +1135,11 @@ void super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     out->super_bins = n_bins;
     out->super_m = m;
     out->super_main = n_main;
+    return true;
 }
 
-template void super_count<1>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
-template void super_count<2>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
-template void super_count<4>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
+template bool super_count<1>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
+template bool super_count<2>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
+template bool super_count<4>(mh_ctx*, const mh_reads*, int, int, uint64_t, mh_kmers*);
 
 }  // namespace mh

@@ -1,7 +1,9 @@
 """Limits of counting by super-k-mers: the memory it takes where its bins do
 not fit their tables (every bin left to the unit counting by MH_SUPER_HOT=0), and outputs whose
 sizes were estimated too small (MH_SUPER_ESTIMATE: a share of the estimate,
-and more bins left over in the first attempt than in the second)."""
+and more bins left over in the first attempt than in the second).  Reads that
+cover little sequence very deeply put many windows in few bins: sets that the
+bins would mostly leave over go to the unit counting, the others do not."""
 import os
 import subprocess
 import sys
@@ -58,10 +60,40 @@ print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), s
 """
 
 
-@pytest.mark.parametrize("k,n_reads", [(31, 300_000), (61, 400_000)])
-@pytest.mark.parametrize("probes", [6, 10, 128])
+@pytest.mark.parametrize("k,n_reads,probes", [(31, 300_000, 6), (31, 300_000, 128), (61, 400_000, 10), (61, 400_000, 128)])
 def test_outputs_sized_too_small_are_made_again(k, n_reads, probes):
     # above 2^25 windows: the first bins counted, the others, the others again
     want = _child(SAMPLED, [k, n_reads], {})
     got = _child(SAMPLED, [k, n_reads], {"MH_SUPER_ESTIMATE": "1", "MH_SUPER_PROBES": str(probes)})
     assert got[:2] == want[:2] and (want[2], got[2]) == ("2", "3")
+
+
+DEEP = r"""
+import hashlib, time, torch
+import synth, paper_1409_7208_gb300 as mh
+genome, depth, k = (int(x) for x in sys.argv[1:])
+a, o = synth.uniform_genome_reads(3, genome, genome * depth // 150, 150, 0.01)
+ctx = mh.Context(device=0, profile=True)
+reads = mh.mh_pack_reads(ctx, a, o)
+s = mh.mh_count_kmers(ctx, reads, k, 2)
+g, units = s.numpy(), "extract_canonical" in ctx.profile() or "extract_scatter" in ctx.profile()
+ctx.set_profile(False)
+times = []
+for _ in range(6):
+    s.free()
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    s = mh.mh_count_kmers(ctx, reads, k, 2)
+    torch.cuda.synchronize()
+    times.append(time.perf_counter() - t0)
+print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), g["n_distinct"], units, min(times))
+"""
+
+
+@pytest.mark.parametrize("genome,depth,k,units", [(30_000, 1000, 31, False), (100_000, 1000, 61, True), (300_000, 300, 47, False),
+                                                  (30_000, 1000, 99, True), (3000, 5000, 61, True), (300_000, 30, 61, False)])
+def test_deep_coverage_is_no_slower_than_the_unit_route(genome, depth, k, units):
+    # a quarter more for what is done before the bins are given up
+    new, old = (_child(DEEP, [genome, depth, k], e) for e in ({}, {"MH_SUPER": "0"}))
+    assert new[:2] == old[:2] and (new[2], old[2]) == (str(units), "True")
+    assert float(new[3]) <= 1.25 * float(old[3]), (new, old)
