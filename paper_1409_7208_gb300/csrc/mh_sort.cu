@@ -892,7 +892,11 @@ static bool sort_by_index(mh_ctx* ctx, const uint64_t* keys, uint64_t* alt, cons
 // Distinct keys with a 32-bit payload (a solid table and its counts): the
 // same spread order (passes over the top P bits of the top word below
 // `skip` constant bits, then the key-value fix-up).  Keys whose top bits are
-// crowded (more than 256 groups past the thread sorts) are sorted fully.
+// crowded (more groups past the fix-up's sorts than `most`) are sorted fully:
+// a group's own sort is ten launches and more, some 35 us, and a full sort 8 to
+// 30 passes whose time grows with n.  Whole path of a sequence of 3 kbp read
+// 1,000 times, k = 61, 333,534 pairs: 2.9 ms, 3.6 by up to 256 groups; of 30 kbp,
+// k = 31, 3.4 M pairs, 105 groups: 2.7 for 7.8.
 // Returns true when the result is in alt / valt.
 template <int NW>
 bool radix_sort_spread_kv(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* vals, uint32_t* valt, uint64_t n,
@@ -921,13 +925,16 @@ bool radix_sort_spread_kv(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* 
     uint32_t* v = in_alt ? valt : vals;
     uint32_t* vo = in_alt ? vals : valt;
     constexpr uint64_t kMaxSegments = 256;
+    // (MH_SPREAD_KV_MIN: tests sort the groups of small tables too)
+    static const bool all_groups = std::getenv("MH_SPREAD_KV_MIN") != nullptr;
+    const uint64_t most = all_groups ? kMaxSegments : std::min(kMaxSegments, std::max<uint64_t>(2, n >> 17));
     Buf<uint64_t> list(ctx, kMaxSegments), cnt(ctx, 2);
     cnt.zero();
     MH_LAUNCH_B(ctx, "spread_fixup_kv", n * (8 * NW + 4), (unsigned)ceil_div(n, F::kTile), 256, 0,
                 spread_fix_kv_kernel<NW>, k, v, n, lo, list.p, kMaxSegments, (unsigned long long*)cnt.p);
     uint64_t n_big = 0;
     read_u64(ctx, cnt.p, &n_big, 1);
-    if (n_big > kMaxSegments) return in_alt != radix_sort<NW>(ctx, k, ko, v, vo, n, 0, bits - skip);
+    if (n_big > most) return in_alt != radix_sort<NW>(ctx, k, ko, v, vo, n, 0, bits - skip);
     if (!n_big) return in_alt;
     Buf<ulonglong2> rest(ctx, n_big);
     MH_LAUNCH(ctx, "spread_bounds", (unsigned)n_big, 256, 0, spread_bounds_kernel<NW>, k, n, lo, list.p, n_big,
