@@ -365,9 +365,10 @@ mh_ctx* mh_server_context(mh_server* s, int slot);
  * worker contexts and the server. */
 int mh_server_destroy(mh_server* s);
 
-/* The scatter-pass tile shape the context uses for 1-word keys: 0 = 16 keys
- * a thread at 3 CTAs per SM (the default), 1 = 12 at 4, 2 = 14 at 3; -1
- * before any autotuning (the default applies). */
+/* The scatter-pass tile shape the context uses for 1-word keys without a
+ * payload: 0 = 16 keys a thread at 3 CTAs per SM (the default; small sorts
+ * take smaller tiles), 1 = 12 at 4, 2 = 14 at 3; -1 before any autotuning (the
+ * default applies). */
 int mh_sort_shape(const mh_ctx* ctx);
 
 /* How the context counts (Sec. 2, third paragraph: the sort and count of

@@ -196,17 +196,19 @@ static void tiny_sort(mh_ctx* ctx, uint64_t* keys, uint64_t n) {
 template <int NW, bool HV>
 static bool radix_sort_dispatch(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* vals, uint32_t* valt,
                                 uint64_t n, int bit_lo, int bit_hi, const uint32_t* h, SegIn seg = SegIn{}) {
+    // the shape of large sorts of one-word keys alone; others have one each
+    const int shape = NW > 1 || HV ? 0 : ctx->sort_shape >= 0 ? ctx->sort_shape : sort_variant();
     // up to 2^19 words of keys: tiles of 1,024 words, so that a pass has some
     // for every SM (14 passes of a path of 10,000 reads 0.156 -> 0.132 ms)
-    if (!seg.cnt && n * (uint64_t)NW <= (1u << 19) && ctx->sort_shape < 0 && sort_variant() == 0)
+    if (!seg.cnt && n * (uint64_t)NW <= (1u << 19) && shape == 0)
         return radix_sort_impl<NW, HV, 4 / NW, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
     if constexpr (NW == 1) {
         if constexpr (HV) {
             return radix_sort_impl<NW, HV, 16, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
         } else {
-            switch (ctx->sort_shape >= 0 ? ctx->sort_shape : sort_variant()) {
+            switch (shape) {
                 case 1: return radix_sort_impl<NW, HV, 12, 4>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
-                case 2: return radix_sort_impl<NW, HV, 16, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
+                case 2: return radix_sort_impl<NW, HV, 14, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
                 default: return radix_sort_impl<NW, HV, 16, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
             }
         }

@@ -1,5 +1,8 @@
-"""Which routes the radix sorts take, seen by their launches: a table of keys
-crowded in their top bits is sorted by passes, not group by group."""
+"""Which tiles and routes the radix sorts take, seen by their launches: with
+MH_SORT_CHUNK_TILES=1 a scatter pass is a launch a tile.  The tile shapes of
+one-word keys differ (16, 12 and 14 keys a thread), and small sorts keep their
+own; a table of keys crowded in their top bits is sorted
+by passes, not group by group."""
 import os
 import subprocess
 import sys
@@ -9,6 +12,42 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SHAPES = r"""
+import sys
+sys.path.insert(0, %r)
+import synth, paper_1409_7208_gb300 as mh
+k = int(sys.argv[1])
+a, o = synth.uniform_genome_reads(9, int(sys.argv[2]), int(sys.argv[3]), 150, 0.01)
+ctx = mh.Context(device=0, profile=True)
+reads = mh.mh_pack_reads(ctx, a, o)
+for shape in (-1, 0, 1, 2):
+    mh.mh_set_count_plan(ctx, path=0, sort_shape=shape, unit_bits_delta=0, spread_bits_delta=0, bucket_bits=-1)
+    ctx.profile_reset()
+    mh.mh_count_kmers(ctx, reads, k, 2)
+    print(ctx.profile()["radix_onesweep"][0])
+""" % ROOT
+
+
+def _launches(code, args, env):
+    p = subprocess.run([sys.executable, "-c", code] + [str(x) for x in args], env=dict(os.environ, **env),
+                       capture_output=True, text=True, timeout=600)
+    assert p.returncode == 0, p.stdout + p.stderr
+    return [int(x) for x in p.stdout.split()]
+
+
+def test_shapes_of_large_one_word_sorts_differ():
+    # 2 million windows by the unit counting
+    default, s0, s1, s2 = _launches(SHAPES, [31, 100_000, 17_000], {"MH_SUPER": "0", "MH_SORT_CHUNK_TILES": "1"})
+    assert default == s0 < s2 < s1
+
+
+@pytest.mark.parametrize("k", [31, 47, 99])
+def test_the_default_shape_keeps_the_tiles_of_small_sorts(k):
+    # 60 thousand windows and the pairs kept of them
+    default, s0 = _launches(SHAPES, [k, 4000, 60_000 // (150 - k)], {"MH_SUPER": "0", "MH_SORT_CHUNK_TILES": "1"})[:2]
+    assert default == s0
+
 
 CROWDED = r"""
 import sys
