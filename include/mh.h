@@ -374,19 +374,23 @@ int mh_sort_shape(const mh_ctx* ctx);
 /* How the context counts (Sec. 2, third paragraph: the sort and count of
  * every (k+1)-mer).  Every plan gives the same results; only the route and
  * its speed change.  -1 / 0 fields mean the library's default.
- *   path              0: unit counting (8-bit passes over the top bits of
- *                     the mixed keys, then each unit of about 160 / 96 / 56
- *                     keys (1 / 2 / 4 key words) sorted and counted by one
- *                     warp); 1: the spread sort (passes over the top
+ *   path              0: the default route: super-k-mers (from k = 20 on, sets
+ *                     of 2^22 windows and more, up to k = 47 smaller ones
+ *                     too) or unit counting (8-bit passes over the top bits
+ *                     of the mixed keys, then each unit of about 160 / 96 /
+ *                     56 keys (1 / 2 / 4 key words) sorted and counted by
+ *                     one warp); 1: the spread sort (passes over the top
  *                     ceil(log2 n) bits, a fix-up of keys sharing them, a run
  *                     pass)
  *   sort_shape        the scatter tile shape (see mh_sort_shape)
- *   unit_bits_delta   added to the unit bits of path 0 (-2..2)
+ *   unit_bits_delta   added to the unit bits of path 0 (-2..2), wherever it
+ *                     counts by units
  *   spread_bits_delta added to the bits path 1 sorts by passes (-8, 0, 8)
  *   bucket_bits       out-of-core buckets: 2^bucket_bits (0..6), -1 = the
  *                     memory plan's choice
  * MH_BATCH_AUTOTUNE tries a set of plans on the largest set of a batch (per
- * key width, k and size class of that set) and keeps the fastest.
+ * key width, k and size class of that set) and keeps the fastest, the default
+ * one unless another is faster by 5 %.
  * Errors: MH_EINVAL (NULL, a field out of range). */
 typedef struct {
     int path;

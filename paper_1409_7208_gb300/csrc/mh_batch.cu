@@ -22,7 +22,7 @@
 #include <thread>
 #include <vector>
 
-#include "mh_internal.cuh"
+#include "mh_super.cuh"
 
 namespace mh {
 void profile_merge(mh_ctx* dst, mh_ctx* src);
@@ -79,13 +79,18 @@ void apply_plan(mh_ctx* w, const Plan& p) {
     w->bucket_bits = p[4];
 }
 
-// The plans tried for a set: for 1-word keys the unit counting with each
-// tile shape and unit bits one either side, and the spread route with its
-// bits one digit either side; for wider keys the spread bits; and, when the
-// memory plan splits the set into buckets, one bucket bit more.
-std::vector<Plan> candidate_plans(int nw, int auto_buckets) {
+// The plans tried for a set, the default one first.  A set counted by
+// super-k-mers: that, and the spread route with its bits one digit either side
+// (shapes and unit bits change nothing for it).  Others, 1-word keys: the unit
+// counting with each tile shape and unit bits one either side, and the spread
+// route; wider keys: unit bits and spread bits.  And, when the memory plan
+// splits the set into buckets, one bucket bit more.
+std::vector<Plan> candidate_plans(int nw, int auto_buckets, bool super) {
     std::vector<Plan> c;
-    if (nw == 1) {
+    if (super) {
+        c.push_back({0, 0, 0, 0, -1});
+        for (int sb : {0, 8, -8}) c.push_back({1, 0, 0, sb, -1});
+    } else if (nw == 1) {
         for (int shape = 0; shape < kSortShapes; shape++) c.push_back({0, shape, 0, 0, -1});
         c.push_back({0, 0, -1, 0, -1});
         c.push_back({0, 0, 1, 0, -1});
@@ -105,7 +110,10 @@ std::vector<Plan> candidate_plans(int nw, int auto_buckets) {
 }
 
 // Count `s` on worker w once untimed, then once per candidate plan, and
-// return the fastest plan (empty if a count failed).
+// return the fastest plan (empty if a count failed): the default one unless
+// another takes less than kTuneGain of its time, since counts of one plan differ
+// by a few percent and the plan holds for smaller sets too.
+constexpr float kTuneGain = 0.95f;
 Plan tune_plan(mh_ctx* w, const mh_read_set& s, int k, int d) {
     mh_reads* reads = nullptr;
     if (mh_pack_reads(w, s.ascii, s.n_bases, s.offs, s.n_reads, s.on_device, &reads) != MH_OK) return {};
@@ -117,7 +125,9 @@ Plan tune_plan(mh_ctx* w, const mh_read_set& s, int k, int d) {
         const int nw = words_for(k);
         const uint64_t kk = (uint64_t)k * s.n_reads;
         w->bucket_bits = -1;
-        std::vector<Plan> cands = candidate_plans(nw, count_bucket_bits(w, s.n_bases > kk ? s.n_bases - kk : 0, nw));
+        const uint64_t windows = s.n_bases > kk ? s.n_bases - kk : 0;
+        const int buckets = count_bucket_bits(w, windows, nw);
+        std::vector<Plan> cands = candidate_plans(nw, buckets, buckets == 0 && use_super(windows, k + 1));
         for (size_t i = 0; i <= cands.size(); i++) {
             apply_plan(w, i == 0 ? cands[0] : cands[i - 1]);  // the first count warms up
             mh_kmers* solid = nullptr;
@@ -134,7 +144,7 @@ Plan tune_plan(mh_ctx* w, const mh_read_set& s, int k, int d) {
             }
             if (i > 0 && (best.empty() || ms < best_ms)) {
                 best = cands[i - 1];
-                best_ms = ms;
+                best_ms = i == 1 ? kTuneGain * ms : ms;
             }
         }
     }

@@ -19,9 +19,10 @@
 //   units     each unit sorted and run-length counted on chip by one warp,
 //             the solid filter applied, both strands out (mh_group.cu)
 //   sort      the solid table by the key-value spread sort, ascending
-// From 2^22 windows on (k >= 20), the default plan counts by super-k-mers
-// instead (mh_super.cu); the unit counting takes the smaller sets and the
-// out-of-core buckets.
+// From k = 20 on, sets of 2^22 windows and more, and with k up to 47 smaller
+// ones too, are counted by super-k-mers instead (mh_super.cu); the unit counting
+// takes the others, the out-of-core buckets, sets of very deep coverage and what
+// the super-k-mers' bins leave over.
 // The spread route (a plan's alternative): passes over the top ceil(log2 n)
 // bits, a fix-up of keys sharing them, a run pass (runs_kernel: run heads
 // in a shared-memory bitmask, run lengths from the next head, the solid
@@ -954,7 +955,7 @@ void count_kmers(mh_ctx* ctx, const mh_reads* reads, int k, int d, mh_kmers* out
     out->n_kmers = 2 * n;
     out->spectrum_mixed = kMixed;
     const int bb = count_bucket_bits(ctx, n, NW);
-    if (bb == 0 && use_unit_count(ctx) && use_super(ctx, n, k + 1)) {
+    if (bb == 0 && use_unit_count(ctx) && use_super(n, k + 1)) {
         woff.reset();
         if (super_count<NW>(ctx, reads, k, d, n, out)) return;
         windows();

@@ -881,16 +881,17 @@ static long env_long(const char* name, long dflt) {
 // passes (whole path, windows x 10^3, unit route and this one in ms: k = 31
 // 38 1.04 0.87, 376 1.28 1.05, 4,700 1.56 1.25; k = 47 62 1.34 1.02, 1,950
 // 1.63 1.23).  Windows of more symbols leave bins to the rest: k = 63 248 1.48
-// 1.58; k = 61 1,600 1.73 1.77; k = 99 2,600 2.45 2.65.  A plan that moves the
-// unit bits, or a variable that steers the unit route, keeps it below 2^22.  MH_SUPER=0 turns
-// this route off, =1 on at any size and whatever is left to the rest (tests).  The counters of a bin hold 32
-// bits each, so fewer than 2^32 windows.
+// 1.58; k = 61 1,600 1.73 1.77; k = 99 2,600 2.45 2.65.  A plan's unit bits do not
+// choose: they are those of the sets, buckets and rests that units count.  A
+// variable that steers the unit counting (tests) does.  MH_SUPER=0 turns this
+// route off, =1 on at any size and whatever is left to the rest (tests).  The
+// counters of a bin hold 32 bits each, so fewer than 2^32 windows.
 static long super_switch() {
     static const long v = env_long("MH_SUPER", -1);
     return v;
 }
 
-bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
+bool use_super(uint64_t n, int K1) {
     const long v = super_switch();
     static const bool steered = [] {
         for (const char* e : {"MH_GROUP_CAP", "MH_GROUP_UNIT_BITS", "MH_EXTRACT_SCATTER", "MH_SCATTER_CAP", "MH_SORT_CHUNK_TILES"})
@@ -898,8 +899,7 @@ bool use_super(const mh_ctx* ctx, uint64_t n, int K1) {
         return false;
     }();
     if (v == 0 || !n || n >= (1ull << 32) || super_m(K1) == 0) return false;
-    if (v == 1 || n >= (1ull << 22)) return true;
-    return K1 <= 48 && !steered && ctx->unit_bits_delta == 0;
+    return v == 1 || (!steered && (n >= (1ull << 22) || K1 <= 48));
 }
 
 template <int NW>

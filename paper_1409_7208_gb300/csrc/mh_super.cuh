@@ -131,7 +131,7 @@ __device__ __forceinline__ uint32_t super_find(const SuperIndex& S, const uint64
 }
 
 // Whether n windows of K1 symbols are counted by super-k-mers.
-bool use_super(const mh_ctx* ctx, uint64_t n, int K1);
+bool use_super(uint64_t n, int K1);
 
 // False (and nothing done): too many windows would be left to the rest, the
 // set is one for the unit counting.
