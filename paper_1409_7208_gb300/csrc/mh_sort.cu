@@ -193,6 +193,16 @@ static void tiny_sort(mh_ctx* ctx, uint64_t* keys, uint64_t n) {
     MH_LAUNCH(ctx, "tiny_sort", 1, 1024, smem, tiny_sort_kernel<NW>, keys, (uint32_t)n, slots);
 }
 
+// Words of keys of a sort in small tiles: 2^19, or MH_SORT_SMALL when set (tests
+// run the large tiles on small inputs with 0).
+static uint64_t small_words() {
+    static const uint64_t v = [] {
+        const char* e = std::getenv("MH_SORT_SMALL");
+        return e ? (uint64_t)std::strtoull(e, nullptr, 10) : (uint64_t)1 << 19;
+    }();
+    return v;
+}
+
 template <int NW, bool HV>
 static bool radix_sort_dispatch(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* vals, uint32_t* valt,
                                 uint64_t n, int bit_lo, int bit_hi, const uint32_t* h, SegIn seg = SegIn{}) {
@@ -200,7 +210,7 @@ static bool radix_sort_dispatch(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint
     const int shape = NW > 1 || HV ? 0 : ctx->sort_shape >= 0 ? ctx->sort_shape : sort_variant();
     // up to 2^19 words of keys: tiles of 1,024 words, so that a pass has some
     // for every SM (14 passes of a path of 10,000 reads 0.156 -> 0.132 ms)
-    if (!seg.cnt && n * (uint64_t)NW <= (1u << 19) && shape == 0)
+    if (!seg.cnt && n * (uint64_t)NW <= small_words() && shape == 0)
         return radix_sort_impl<NW, HV, 4 / NW, 3>(ctx, keys, alt, vals, valt, n, bit_lo, bit_hi, h, seg);
     if constexpr (NW == 1) {
         if constexpr (HV) {

@@ -2,7 +2,10 @@
 MH_SORT_CHUNK_TILES=1 a scatter pass is a launch a tile.  The tile shapes of
 one-word keys differ (16, 12 and 14 keys a thread), and small sorts keep their
 own; a table of keys crowded in their top bits is sorted
-by passes, not group by group."""
+by passes, not group by group.  And the tiles of large sorts on inputs small
+enough for the oracle (MH_SORT_SMALL=0, MH_TINY_SORT=0), in chains of one and
+three tiles: every key width, keys alone and pairs (with MH_SPREAD_KV_MIN=0 and
+without)."""
 import os
 import subprocess
 import sys
@@ -77,3 +80,19 @@ def test_crowded_small_wide_tables_take_few_launches(k, genome):
     assert got[:2] == full[:2] and 1 << 12 < int(got[1]) < 1 << 20
     # beside the full sort: the passes by the top bits, and two groups' sorts
     assert int(got[2]) <= 2.5 * int(full[2]) + 8, (got, full)
+
+
+@pytest.mark.parametrize("chunk", ["1", "3"])
+@pytest.mark.parametrize("kv_min", ["0", str(1 << 30)])
+def test_large_tiles_on_small_inputs_match_oracle(chunk, kv_min):
+    from test_gpu_chunks import CHILD
+
+    env = dict(os.environ, MH_SORT_SMALL="0", MH_TINY_SORT="0", MH_SORT_CHUNK_TILES=chunk, MH_SPREAD_KV_MIN=kv_min)
+    p = subprocess.run([sys.executable, "-c", CHILD], env=env, capture_output=True, text=True, timeout=900)
+    assert p.returncode == 0 and "ok" in p.stdout, p.stdout + p.stderr
+
+
+def test_small_and_large_tiles_differ():
+    def run(env):
+        return _launches(SHAPES, [47, 4000, 600], dict(env, MH_SUPER="0", MH_SORT_CHUNK_TILES="1"))[0]
+    assert run({"MH_SORT_SMALL": "0"}) < run({})
