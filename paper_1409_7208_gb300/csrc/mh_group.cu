@@ -697,7 +697,7 @@ static uint32_t group_cap() {
 template <int NW>
 void group_count(mh_ctx* ctx, Buf<uint64_t>& sorted, Buf<uint64_t>& other, uint64_t n, int k, int d, int skip,
                  const GroupPlan& plan, Buf<uint64_t>& out_keys, Buf<uint32_t>& out_cnt, uint64_t* n_out,
-                 uint64_t* n_runs, uint64_t* n_palin_runs, RunList* list) {
+                 uint64_t* n_runs, uint64_t* n_palin_runs, RunList* list, bool ascending) {
     using C = UnitCfg<NW>;
     const int K1 = k + 1;
     const int ub = plan.unit_bits;
@@ -791,8 +791,12 @@ void group_count(mh_ctx* ctx, Buf<uint64_t>& sorted, Buf<uint64_t>& other, uint6
     list->n = R;
     list->keys = Buf<uint64_t>(ctx, (R ? R : 1) * NW);
     list->lens = Buf<uint32_t>(ctx, R ? R : 1);
-    Buf<uint64_t> keys(ctx, (S ? S : 1) * NW), alt(ctx, (S ? S : 1) * NW);
-    Buf<uint32_t> cnt(ctx, S ? S : 1), calt(ctx, S ? S : 1);
+    Buf<uint64_t> keys(ctx, (S ? S : 1) * NW), alt;
+    Buf<uint32_t> cnt(ctx, S ? S : 1), calt;
+    if (ascending) {
+        alt = Buf<uint64_t>(ctx, (S ? S : 1) * NW);
+        calt = Buf<uint32_t>(ctx, S ? S : 1);
+    }
     if (n)
         MH_LAUNCH_B(ctx, "unit_compact", (R + S) * (16 * NW + 8), grid_for(ctx, n_units * 32, 256, 8), 256, 0,
                     unit_compact_kernel<NW>, other.p, spec_len.p, sk.p, sc.p, ustart.p, ucount.p, scount.p, uoff.p,
@@ -808,7 +812,8 @@ void group_count(mh_ctx* ctx, Buf<uint64_t>& sorted, Buf<uint64_t>& other, uint6
     sorted.reset();
     other.reset();
     // the solid table: S distinct keys with their counts, sorted
-    const bool in_alt = radix_sort_spread_kv<NW>(ctx, keys.p, alt.p, cnt.p, calt.p, S, 64 * NW - 2 * K1);
+    const bool in_alt =
+        ascending && radix_sort_spread_kv<NW>(ctx, keys.p, alt.p, cnt.p, calt.p, S, 64 * NW - 2 * K1);
     if (in_alt) {
         out_keys = std::move(alt);
         out_cnt = std::move(calt);
@@ -821,7 +826,7 @@ void group_count(mh_ctx* ctx, Buf<uint64_t>& sorted, Buf<uint64_t>& other, uint6
 #define MH_GROUP_COUNT(NW)                                                                                          \
     template void group_count<NW>(mh_ctx*, Buf<uint64_t>&, Buf<uint64_t>&, uint64_t, int, int, int,               \
                                   const GroupPlan&, Buf<uint64_t>&, Buf<uint32_t>&, uint64_t*, uint64_t*, uint64_t*, \
-                                  RunList*);
+                                  RunList*, bool);
 MH_GROUP_COUNT(1)
 MH_GROUP_COUNT(2)
 MH_GROUP_COUNT(4)

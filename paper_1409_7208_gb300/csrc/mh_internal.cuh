@@ -738,13 +738,14 @@ GroupPlan group_plan(mh_ctx* ctx, uint64_t n, int skip, int nw);
 // mh_group.cu): `sorted` holds n keys sorted by the top skip + 8 *
 // plan.passes bits of their top word, `other` n free keys.  Each unit is
 // sorted on chip and run-length counted: out_keys / out_cnt get the kept
-// (k+1)-mers of both strands (count >= d, ascending), list the spectrum
+// (k+1)-mers of both strands (count >= d; ascending, or in no order for a
+// caller that sorts them with others), list the spectrum
 // (every run's mixed key and length, ascending).  Both input buffers are
 // consumed (freed).
 template <int NW>
 void group_count(mh_ctx* ctx, Buf<uint64_t>& sorted, Buf<uint64_t>& other, uint64_t n, int k, int d, int skip,
                  const GroupPlan& plan, Buf<uint64_t>& out_keys, Buf<uint32_t>& out_cnt, uint64_t* n_out,
-                 uint64_t* n_runs, uint64_t* n_palin_runs, RunList* list);
+                 uint64_t* n_runs, uint64_t* n_palin_runs, RunList* list, bool ascending = true);
 
 
 struct SuperIndex;

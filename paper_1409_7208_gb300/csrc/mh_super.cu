@@ -59,7 +59,7 @@ constexpr int kHashPad = (kSplitTile + kSplitHalo) / 8 * 9;  // one word of padd
 constexpr int kNwinBits = 12;                         // a record: start << 12 | windows (at most 2,048)
 static_assert(kSplitTile < (1 << kNwinBits), "a run fits a record");
 
-enum { T_SPEC = 0, T_SOLID = 1, T_PALIN = 2, T_DEF = 3, T_DEFWIN = 4, T_RECS = 5, T_DONE = 6, T_LOST = 7, T_N = 8 };
+enum { T_SPEC = 0, T_SOLID = 1, T_PALIN = 2, T_DEF = 3, T_DEFWIN = 4, T_RECS = 5, T_DONE = 6, T_FULL = 7, T_LOST = 8, T_N = 9 };
 
 }  // namespace
 
@@ -329,22 +329,19 @@ struct SuperSmem {
     static_assert(kSym % 16 == 0 && kOwn % 16 == 0, "aligned");
 };
 
-// Whether w windows left to the rest of `done` counted or left are so many
-// that the set had better be counted by units: more than 2 in 5 of two words,
-// 13 in 20 of four.  What is left over is written out as keys, sorted, counted
-// and merged, which costs more a window than the units do at once, and the
-// time for its insertions is lost.  By unit counting and by bins with what they
-// leave over, two words (k = 47 and 61, 30 to 10,000 times a genome): 4.7 and
-// 4.3 ms with 22 % of the windows left over, 7.2 and 6.2 with 18 %, 3.4 and 4.2
-// with 44 %, 13.5 and 20.7 with 79 %; four words (k = 99): 8.5 and 6.3 with
-// 42 %, 3.2 and 3.4 with 46 %, 4.8 and 5.5 with 58 %, 13.3 and 19.0 with 71 %,
-// where giving up costs 0.3 to 0.8 ms.  One word (k = 31): 13.4 and 12.9 with
-// 63 %, so those never give up.
+// Whether w windows of bins that filled their tables, of `done` counted or left
+// over, are so many that the set had better be counted by units: more than 3 in
+// 5, of keys of two words.  The insertions into those bins are lost, and their
+// windows are written out as keys, sorted and counted all the same (a bin of
+// more windows than it may have is left over before that).  By unit counting
+// and by bins with what they leave over, k = 61: 5.4 and 7.2 ms with 63 % of the
+// windows in full tables (300 kbp 300 times; 6.0 given up), 13.4 and 16.3 with
+// 79 % (100 kbp 1,000 times; 14.1), 3.5 and 4.0 with 44 %, 5.8 and 5.6 with 54 %,
+// 4.7 and 4.1 with 22 %.  Of four words 4.8 and 5.3 ms with 58 %, 9.8 and 10.3
+// with 71 %, 10.2 and 10.1 with 67 %: as much as giving up costs.  Keys of one
+// word are faster by bins at any depth.
 constexpr uint32_t kLostBins = 32;
-template <int NW>
-__host__ __device__ bool super_lost(uint64_t w, uint64_t done) {
-    return NW == 2 ? 5 * w > 2 * done : 20 * w > 13 * done;
-}
+__host__ __device__ inline bool super_lost(uint64_t w, uint64_t done) { return 5 * w > 3 * done; }
 
 // A CTA per bin.  The table's first word is a mixed key's top word (the whole
 // key of one word); kEmpty marks a free slot: the mixed image of the
@@ -768,7 +765,8 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
                 deferred[q] = make_ulonglong2(b, w);
                 if (give_up) {
                     const uint64_t done = atomicAdd(&totals[T_DONE], (unsigned long long)W);
-                    if (q >= kLostBins && w > give_up / 16 && super_lost<NW>(w, done)) totals[T_LOST] = 1;
+                    const uint64_t full = atomicAdd(&totals[T_FULL], W > hot ? 0ull : (unsigned long long)W);
+                    if (q >= kLostBins && full > give_up / 16 && super_lost(full, done)) totals[T_LOST] = 1;
                     lost = *(volatile unsigned long long*)&totals[T_LOST] != 0;
                 }
             }
@@ -919,8 +917,8 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     const uint64_t F = reads->n_frags, n_words = ceil_div(reads->n_packed, 16) + kPackPad;
     const uint64_t n_tiles = ceil_div(reads->n_packed, (uint64_t)kSplitTile);
     const uint32_t n_bins = (uint32_t)std::max<uint64_t>(1, n / C::kTarget);
-    const uint64_t give_up = NW > 1 && super_switch() != 1 ? n : 0;
-    Buf<uint64_t> first(ctx, n_tiles), off(ctx, (uint64_t)n_bins + 1), totals(ctx, 8);
+    const uint64_t give_up = NW == 2 && super_switch() != 1 ? n : 0;
+    Buf<uint64_t> first(ctx, n_tiles), off(ctx, (uint64_t)n_bins + 1), totals(ctx, T_N);
     Buf<unsigned long long> bins(ctx, n_bins);
     MH_LAUNCH(ctx, "super_tiles", grid_for(ctx, n_tiles, 256), 256, 0, super_tiles_kernel, reads->frag_offs, F,
               n_tiles, first.p);
@@ -937,7 +935,7 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     unsigned long long* tot = reinterpret_cast<unsigned long long*>(totals.p);
     Buf<uint64_t> more;
     SuperRecs recs{rec.p, nullptr, off.p, bins.p, slots};
-    uint64_t h[8] = {0};
+    uint64_t h[T_N] = {0};
     Buf<uint64_t> spec, solid, soff(ctx, n_bins);
     Buf<uint32_t> spec_len, solid_c;
     Buf<uint2> sidx(ctx, (uint64_t)n_bins * C::kWords);
@@ -1004,7 +1002,7 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         cap = std::max(cap, h[T_RECS]);
     }
     if (sample) {
-        if (give_up && h[T_DEF] > kLostBins && super_lost<NW>(h[T_DEFWIN], h[T_DONE])) return false;
+        if (give_up && h[T_DEF] > kLostBins && super_lost(h[T_FULL], h[T_DONE])) return false;
         // the other bins into buffers sized by the first ones (bins are by
         // hash: alike but for chance and the heavy ones), then the first
         // ones' entries in front of them
@@ -1096,7 +1094,7 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
                                       : false;
         uint64_t r2 = 0, p2 = 0;
         group_count<NW>(ctx, in_alt ? alt : keys, in_alt ? keys : alt, nd, k, d, 0, gp, rest_k, rest_c, &rest_S, &r2, &p2,
-                        &rest);
+                        &rest, false);
         runs += r2;
         palins += p2;
         R += rest.n;
