@@ -579,18 +579,22 @@ __device__ __forceinline__ bool same_above(const Key<NW>& a, const Key<NW>& b, i
 // are sorted by one thread each, pairs moving together; larger groups inside
 // the window by one warp (successive minima: each round writes every copy
 // of the smallest key above the previous one with its payloads); groups that
-// run past the window or hold more than 64 distinct keys go to a list, each
+// run past the window or hold more than 64 keys go to a list, each
 // listed group then to a segment sort of its own (few, for spread keys).
+// Where more than `most` are listed the table is sorted by other means, so
+// CTAs that see that leave the rest as it is.  (With warps that went 64 rounds
+// into longer groups before listing them, and without an end to it, 1.77 ms for
+// 7.5 M pairs of a satellite at k = 61, now 0.11; 0.27 for 0.33 M pairs of 3 kbp, now 0.03.)
 template <int NW>
 __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                             uint64_t n, int lo, uint64_t* __restrict__ big,
-                                                            uint64_t big_cap, unsigned long long* __restrict__ n_big) {
+                                                            uint64_t big_cap, unsigned long long* __restrict__ n_big, uint64_t most) {
     using F = Fix<NW>;
     __shared__ uint64_t K[F::kWin * NW];
     __shared__ uint32_t V[F::kWin];
     __shared__ uint32_t head[F::kWords], desc[F::kWords];
     __shared__ uint32_t queue[2 * F::kQueue];  // (start, end) of the groups for warps
-    __shared__ uint32_t n_queue;
+    __shared__ uint32_t n_queue, enough;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t s = blockIdx.x * (uint64_t)F::kTile;
     const uint32_t W = (uint32_t)(n - s < (uint64_t)F::kWin ? n - s : (uint64_t)F::kWin);
@@ -608,8 +612,12 @@ __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict
     };
     for (uint32_t i = tid; i < W * NW; i += 256) K[i] = keys[s * NW + i];
     for (uint32_t i = tid; i < W; i += 256) V[i] = vals[s + i];
-    if (tid == 0) n_queue = 0;
+    if (tid == 0) {
+        n_queue = 0;
+        enough = *(volatile unsigned long long*)n_big > most;
+    }
     __syncthreads();
+    if (enough) return;
     for (uint32_t wd = warp; wd < (uint32_t)F::kWords; wd += 8) {
         const uint32_t i = wd * 32 + lane;
         bool h = false, d = false;
@@ -644,7 +652,8 @@ __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict
             if (h == ~0u || h >= len) continue;
             if (any_bit(desc, h + 1, jd)) continue;
             const uint32_t g1 = next_bit(head, jd + 1, W);
-            if (g1 == W && !window_ends_array) {
+            // (the keys are distinct: a warp's rounds cannot finish a longer group)
+            if ((g1 == W && !window_ends_array) || g1 - h > (uint32_t)kFixWarpRounds) {
                 to_big(h);
                 continue;
             }
@@ -674,14 +683,13 @@ __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict
     }
     __syncthreads();
     // larger groups: a warp each, from K and V to keys and vals
-    const uint32_t nq = n_queue;
+    const uint32_t nq = *(volatile unsigned long long*)n_big > most ? 0 : n_queue;
     for (uint32_t q = warp; q < nq; q += 8) {
         const uint32_t g0 = queue[2 * q], g1 = queue[2 * q + 1];
         uint32_t pos = g0;
         Key<NW> prev = key_zero<NW>();
         bool first = true;
-        int rounds = 0;
-        while (pos < g1 && rounds < kFixWarpRounds) {
+        while (pos < g1) {
             Key<NW> mn = key_ones<NW>();
             bool have = false;
             for (uint32_t i = g0 + lane; i < g1; i += 32) {
@@ -713,16 +721,6 @@ __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict
             }
             prev = mn;
             first = false;
-            rounds++;
-        }
-        __syncwarp();
-        if (pos < g1) {
-            // too many distinct keys: rewrite the group as it was and defer it
-            for (uint32_t i = g0 + lane; i < g1; i += 32) {
-                store_key<NW>(keys, s + i, kget(i));
-                vals[s + i] = V[i];
-            }
-            if (lane == 0) to_big(g0);
         }
     }
 }
@@ -907,8 +905,8 @@ static bool sort_by_index(mh_ctx* ctx, const uint64_t* keys, uint64_t* alt, cons
 // crowded (more groups past the fix-up's sorts than `most`) are sorted fully:
 // a group's own sort is ten launches and more, some 35 us, and a full sort 8 to
 // 30 passes whose time grows with n.  Whole path of a sequence of 3 kbp read
-// 1,000 times, k = 61, 333,534 pairs: 2.9 ms, 3.6 by up to 256 groups; of 30 kbp,
-// k = 31, 3.4 M pairs, 105 groups: 2.7 for 7.8.
+// 1,000 times, k = 61, 333,534 pairs: 2.6 ms, 3.6 by up to 256 groups; of 30 kbp,
+// k = 31, 3.4 M pairs, 105 groups: 2.2 for 7.8.
 // Returns true when the result is in alt / valt.
 template <int NW>
 bool radix_sort_spread_kv(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* vals, uint32_t* valt, uint64_t n,
@@ -943,7 +941,7 @@ bool radix_sort_spread_kv(mh_ctx* ctx, uint64_t* keys, uint64_t* alt, uint32_t* 
     Buf<uint64_t> list(ctx, kMaxSegments), cnt(ctx, 2);
     cnt.zero();
     MH_LAUNCH_B(ctx, "spread_fixup_kv", n * (8 * NW + 4), (unsigned)ceil_div(n, F::kTile), 256, 0,
-                spread_fix_kv_kernel<NW>, k, v, n, lo, list.p, kMaxSegments, (unsigned long long*)cnt.p);
+                spread_fix_kv_kernel<NW>, k, v, n, lo, list.p, kMaxSegments, (unsigned long long*)cnt.p, most);
     uint64_t n_big = 0;
     read_u64(ctx, cnt.p, &n_big, 1);
     if (n_big > most) return in_alt != radix_sort<NW>(ctx, k, ko, v, vo, n, 0, bits - skip);
