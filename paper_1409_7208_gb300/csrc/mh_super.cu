@@ -838,32 +838,48 @@ __global__ void __launch_bounds__(256, NW == 1 ? 4 : NW == 2 ? 4 : 3)
     if (lane == 0 && palins) atomicAdd(&totals[T_PALIN], (unsigned long long)palins);
 }
 
+// groups[q] = groups of 32 records of the q-th deferred bin.
+__global__ void super_groups_kernel(SuperRecs recs, const ulonglong2* __restrict__ deferred, uint64_t n_def,
+                                    uint32_t* __restrict__ groups) {
+    for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < n_def; q += (uint64_t)gridDim.x * blockDim.x)
+        groups[q] = ((uint32_t)recs.bins[deferred[q].x] + 31) / 32;
+}
+
 // The mixed canonical keys of the deferred bins, bin q's from its place on,
 // in no fixed order (a warp reserves its windows' places on the bin's cursor).
+// A warp a group of 32 records, wherever its bin: groups [first[q], first[q + 1])
+// are bin q's.  Bins differ in size without bound; of a satellite of 171
+// symbols, read 30 times, k = 61, with as many CTAs for every bin 7.6 ms, by groups
+// 0.29.
 template <int NW>
 __global__ void __launch_bounds__(256) super_expand_kernel(const uint32_t* __restrict__ packed,
                                                            SuperRecs recs,
                                                            const ulonglong2* __restrict__ deferred, uint64_t n_def,
-                                                           int K1, unsigned long long* __restrict__ cursor,
+                                                           const uint64_t* __restrict__ first, int K1,
+                                                           unsigned long long* __restrict__ cursor,
                                                            uint64_t* __restrict__ out) {
     const int lane = threadIdx.x & 31;
-    const uint32_t wy = blockIdx.y * 8 + (threadIdx.x >> 5), ny = gridDim.y * 8;
-    for (uint64_t q = blockIdx.x; q < n_def; q += gridDim.x) {
-        const uint64_t b = deferred[q].x, o0 = recs.off[b];
-        const uint32_t n_rec = (uint32_t)recs.bins[b];
-        for (uint64_t rb = (uint64_t)wy * 32; rb < n_rec; rb += (uint64_t)ny * 32) {
-            const uint64_t r = rb + lane < n_rec ? recs.at(b, o0, (uint32_t)rb + lane) : 0ull;
-            const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)r & ((1u << kNwinBits) - 1u));
-            uint64_t at = 0;
-            if (lane == 0) at = deferred[q].y + atomicAdd(&cursor[q], (unsigned long long)tot);
-            at = __shfl_sync(0xFFFFFFFFu, at, 0);
-            for_windows(r, [&](bool valid, uint32_t j, uint64_t p) {
-                if (!valid) return;
-                const Key<NW> x = load_window<NW>(packed, p, K1);
-                const Key<NW> rc = key_rc<NW>(x, K1);
-                store_key<NW>(out, at + j, mix_key<NW>(key_less<NW>(rc, x) ? rc : x));
-            });
+    const uint64_t warps = (uint64_t)gridDim.x * 8, n_groups = first[n_def];
+    for (uint64_t g = blockIdx.x * 8ull + (threadIdx.x >> 5); g < n_groups; g += warps) {
+        // the last bin that starts at or before group g (empty ones start with the next)
+        uint64_t lo = 0, hi = n_def;
+        while (hi - lo > 1) {
+            const uint64_t mid = (lo + hi) / 2;
+            if (first[mid] <= g) lo = mid; else hi = mid;
         }
+        const uint64_t q = lo, b = deferred[q].x;
+        const uint32_t n_rec = (uint32_t)recs.bins[b], i = (uint32_t)(g - first[q]) * 32 + lane;
+        const uint64_t r = i < n_rec ? recs.at(b, recs.off[b], i) : 0ull;
+        const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)r & ((1u << kNwinBits) - 1u));
+        uint64_t at = 0;
+        if (lane == 0) at = deferred[q].y + atomicAdd(&cursor[q], (unsigned long long)tot);
+        at = __shfl_sync(0xFFFFFFFFu, at, 0);
+        for_windows(r, [&](bool valid, uint32_t j, uint64_t p) {
+            if (!valid) return;
+            const Key<NW> x = load_window<NW>(packed, p, K1);
+            const Key<NW> rc = key_rc<NW>(x, K1);
+            store_key<NW>(out, at + j, mix_key<NW>(key_less<NW>(rc, x) ? rc : x));
+        });
     }
 }
 
@@ -1082,10 +1098,13 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         Buf<uint64_t> keys(ctx, nd * NW), alt(ctx, nd * NW);
         Buf<unsigned long long> cursor(ctx, h[T_DEF]);
         cursor.zero();
-        const unsigned gx = (unsigned)std::min<uint64_t>(h[T_DEF], 4096);
-        const unsigned gy = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(64, (uint64_t)ctx->num_sms * 8 / gx));
-        MH_LAUNCH(ctx, "super_expand", dim3(gx, gy), 256, 0, super_expand_kernel<NW>, reads->packed, recs,
-                  deferred.p, h[T_DEF], K1, cursor.p, keys.p);
+        Buf<uint32_t> groups(ctx, h[T_DEF]);
+        Buf<uint64_t> first_group(ctx, h[T_DEF] + 1);
+        MH_LAUNCH(ctx, "super_groups", grid_for(ctx, h[T_DEF], 256), 256, 0, super_groups_kernel, recs, deferred.p,
+                  h[T_DEF], groups.p);
+        exclusive_scan_u32(ctx, groups.p, first_group.p, h[T_DEF]);
+        MH_LAUNCH(ctx, "super_expand", grid_for(ctx, nd, 2048), 256, 0, super_expand_kernel<NW>, reads->packed, recs,
+                  deferred.p, h[T_DEF], first_group.p, K1, cursor.p, keys.p);
         rec.reset();
         more.reset();
         const GroupPlan gp = group_plan(ctx, nd, 0, NW);

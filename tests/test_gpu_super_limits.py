@@ -115,3 +115,37 @@ print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), c
 def test_pairs_of_left_over_bins_are_sorted_once(k):
     new, old = _child(SORTS, [k], {"MH_SUPER": "1", "MH_SUPER_HOT": "0"}), _child(SORTS, [k], {"MH_SUPER": "0"})
     assert new[0] == old[0] and (new[1], old[1]) == ("1", "1")
+
+
+SATELLITE = r"""
+import hashlib, time, torch
+import numpy as np
+import synth, paper_1409_7208_gb300 as mh
+k = int(sys.argv[1])
+# copies of one unit, a tenth of their bases changed: bins of very different sizes
+rng = np.random.default_rng(2)
+g = np.tile(rng.integers(0, 4, 171), 6000)
+g = np.where(rng.random(len(g)) < 0.1, rng.integers(0, 4, len(g)), g)
+at = rng.integers(0, len(g) - 150, 200_000)
+b = g[at[:, None] + np.arange(150)]
+b = np.where(rng.random(b.shape) < 0.01, rng.integers(0, 4, b.shape), b)
+a = np.frombuffer(b"ACGT", np.uint8)[b].reshape(-1).copy()
+ctx = mh.Context(device=0)
+reads = mh.mh_pack_reads(ctx, a, np.arange(200_001, dtype=np.uint64) * 150)
+times = []
+for _ in range(6):
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    s = mh.mh_count_kmers(ctx, reads, k, 2)
+    torch.cuda.synchronize()
+    times.append(time.perf_counter() - t0)
+g = s.numpy()
+print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), g["n_distinct"], min(times))
+"""
+
+
+@pytest.mark.parametrize("k", [31, 47, 61, 99])
+def test_bins_of_very_different_sizes(k):
+    new, old = _child(SATELLITE, [k], {}), _child(SATELLITE, [k], {"MH_SUPER": "0"})
+    assert new[:2] == old[:2]
+    assert float(new[2]) <= 1.25 * float(old[2]), (new, old)
