@@ -32,6 +32,7 @@
 // instead of one for each.  (A node with one out-edge needs no random value,
 // so jumps skip none that counts.)
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "mh_internal.cuh"
@@ -234,6 +235,28 @@ __global__ void __launch_bounds__(256) walk_links_kernel(const uint64_t* __restr
     }
 }
 
+// *n_ends += edges without out-edges among kEndSamples evenly spaced ones.
+constexpr uint32_t kEndSamples = 4096;
+template <int NW>
+__global__ void __launch_bounds__(64) walk_ends_kernel(const uint64_t* __restrict__ S, uint64_t nS,
+                                                       const uint64_t* __restrict__ offS,
+                                                       const uint64_t* __restrict__ M, uint64_t nM,
+                                                       const uint64_t* __restrict__ offM, int bits, int k,
+                                                       unsigned long long* __restrict__ n_ends) {
+    const uint32_t t = blockIdx.x * 64 + threadIdx.x;
+    const uint64_t i = (nS + nM) / kEndSamples * t;
+    const Key<NW> v = key_low<NW>(i < nS ? load_key<NW>(S, i) : load_key<NW>(M, i - nS), 2 * k);
+    const Key<NW> q = key_shl<NW>(v, 2);
+    auto leaves = [&](const uint64_t* __restrict__ A, uint64_t nA, const uint64_t* __restrict__ off) {
+        if (!nA) return false;
+        const uint64_t p = bucket_lb<NW>(A, off, q, k + 1, bits);
+        return p < nA && key_eq<NW>(key_shr<NW>(load_key<NW>(A, p), 2), v);
+    };
+    const bool end = !leaves(S, nS, offS) && !leaves(M, nM, offM);
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, end);
+    if (m && (threadIdx.x & 31) == 0) atomicAdd(n_ends, (unsigned long long)__popc(m));
+}
+
 // Jumps of twice the steps from jumps of `steps` steps.
 __global__ void __launch_bounds__(256) walk_double_kernel(const uint2* __restrict__ in, uint64_t n, int steps,
                                                           uint2* __restrict__ out) {
@@ -333,17 +356,29 @@ __global__ void contig_compact_kernel(const uint8_t* __restrict__ slots, uint32_
 // us a million edges (1.3 ms for 25 M edges) and the walks by them 0.5 ms.
 // They even out near E = 49,000 max_len; the line is drawn at 20,000, since
 // doubling over arrays far beyond L2 costs more an edge.
-// MH_WALK_LINKS=0 / 1 decides it for tests.
-static bool use_links(const mh_ctx* ctx, uint64_t E, uint64_t n_walks, uint64_t max_len) {
+// Walks end at dead ends, so max_len is only as many steps as they could make:
+// from 2^22 edges on the dead ends among some edges are counted before links are
+// made (10 us), and the longest of n_walks walks is taken as ln(n_walks) times
+// the mean distance of one (2,000 walks over 17.9 M edges, 1 % of them dead ends:
+// 0.8 ms by search, 1.2 by links; 18.4 M edges of reads that overlap nowhere 0.26
+// and 1.44).  MH_WALK_LINKS=0 / 1 decides it for tests.
+static int links_switch() {
     static const int v = [] {
         const char* e = std::getenv("MH_WALK_LINKS");
         return e ? std::atoi(e) : -1;
     }();
+    return v;
+}
+
+static bool links_pay(const mh_ctx* ctx, uint64_t E, uint64_t n_walks, double steps) {
+    const uint64_t rounds = ceil_div(n_walks, (uint64_t)ctx->num_sms * 64);
+    return (double)E <= 20000.0 * steps * (double)rounds;
+}
+
+static bool use_links(const mh_ctx* ctx, uint64_t E, uint64_t n_walks, uint64_t max_len) {
+    const int v = links_switch();
     if (v == 0 || E >= kNoJump) return false;
-    if (v != 1) {
-        const uint64_t rounds = ceil_div(n_walks, (uint64_t)ctx->num_sms * 64);
-        if (E > 20000 * max_len * rounds) return false;
-    }
+    if (v != 1 && !links_pay(ctx, E, n_walks, (double)max_len)) return false;
     // 40 bytes an edge, beside the index: within a budget that may have room for it
     return !ctx->budget || ctx->in_use + 40 * E + n_walks * (max_len / 4 + 64) < ctx->budget;
 }
@@ -399,13 +434,46 @@ void walk_contigs(mh_ctx* ctx, const mh_kmers* solid, const mh_kmers* mercy, uin
         linked = false;
         take();
     }
-    if (n_walks) {
+    auto index = [&] {
         if (nS)
             MH_LAUNCH(ctx, "walk_index", grid_for(ctx, nS, 256), 256, 0, table_index_kernel<NW>, solid->keys, nS,
                       k + 1, bits, offS.p);
         if (nM)
             MH_LAUNCH(ctx, "walk_index", grid_for(ctx, nM, 256), 256, 0, table_index_kernel<NW>, mk, nM, k + 1, bits,
                       offM.p);
+    };
+    if (n_walks) {
+        index();
+        if (linked && links_switch() != 1 && E >= (1ull << 22)) {
+            Buf<unsigned long long> ends(ctx, 1);
+            ends.zero();
+            MH_LAUNCH(ctx, "walk_ends", kEndSamples / 64, 64, 0, walk_ends_kernel<NW>, solid->keys, nS, offS.p, mk, nM,
+                      offM.p, bits, k, ends.p);
+            uint64_t n_ends = 0;
+            read_u64(ctx, reinterpret_cast<const uint64_t*>(ends.p), &n_ends, 1);
+            const double far = n_ends ? std::log((double)n_walks + 1.0) * kEndSamples / (double)n_ends : max_len;
+            if (!links_pay(ctx, E, n_walks, std::min((double)max_len, far))) {
+                link.reset();
+                a.reset();
+                b.reset();
+                c.reset();
+                slots.reset();
+                linked = false;
+                stride = max_len;
+                try {
+                    slots = Buf<uint8_t>(ctx, n_walks * stride);
+                } catch (const Error& e) {
+                    // (perhaps with the coarser index)
+                    if (e.code != MH_ENOMEM) throw;
+                    lens.reset();
+                    off.reset();
+                    offS.reset();
+                    offM.reset();
+                    take();
+                    index();
+                }
+            }
+        }
         if (linked) {
             if (nS)
                 MH_LAUNCH(ctx, "walk_links", grid_for(ctx, nS, 256), 256, 0, walk_links_kernel<NW>, solid->keys, nS,
