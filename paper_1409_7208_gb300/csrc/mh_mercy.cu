@@ -21,10 +21,9 @@
 //   walk     a few lanes per hit: step forward to the next solid window q; if
 //            q > p+1 and q has no indegree, the windows p+1..q-1 are emitted
 //            (canonical keys).  Solidity: a search of the counting spectrum
-//            (distinct canonical keys, ascending as mix_key images, so their
-//            top bits are evenly spread, with their run lengths) through a
-//            bucket index on the top bits of the top word; handles without a
-//            mixed spectrum: a hash set of the canonical solid keys.
+//            (distinct canonical keys as mix_key images, with their run
+//            lengths), in its super-k-mer bins or, where it is ascending,
+//            through a bucket index on the top bits of the top word.
 //   finish   sort + dedup of the candidates, counts looked up in the
 //            counting spectrum, both strands, sorted.
 #include "mh_super.cuh"
@@ -302,10 +301,6 @@ __device__ __forceinline__ uint32_t ends_find(const Slot<NW>* __restrict__ table
     return 0;
 }
 
-// Canonical solid keys into the solidity set.  1-word keys use 8-byte slots
-// holding the key itself, empty = all ones (never canonical: the reverse
-// complement of T...T is A...A, which is smaller); wider keys use Slot
-// (32-bit tag + key).
 // Bucket index over the ascending mixed spectrum keys: off[b] = first index
 // whose top `bits` bits (of the top word) are >= b, for b = 0..2^bits
 // (thread per key; each bucket boundary is written by exactly one thread).
@@ -336,49 +331,6 @@ __device__ __forceinline__ uint32_t spec_find(const uint64_t* __restrict__ spec,
         if (!key_less<NW>(v, m)) return key_eq<NW>(v, m) ? len[i] : 0u;
     }
     return 0u;
-}
-
-template <int NW>
-__global__ void __launch_bounds__(256) solid_insert_kernel(const uint64_t* __restrict__ S, uint64_t n, int K1,
-                                                           Slot<NW>* __restrict__ table, uint64_t cap_mask,
-                                                           uint32_t* __restrict__ err) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        Key<NW> x = load_key<NW>(S, i);
-        if (key_less<NW>(key_rc<NW>(x, K1), x)) continue;
-        uint64_t h = key_hash<NW>(x);
-        uint32_t tag = slot_tag(h);
-        uint64_t s = h & cap_mask;
-        bool placed = false;
-        for (uint64_t probe = 0; probe <= cap_mask; probe++) {
-            if (atomicCAS(&table[s].tag, 0u, tag) == 0u) {
-#pragma unroll
-                for (int w = 0; w < NW; w++) table[s].k[w] = x.w[w];
-                placed = true;
-                break;
-            }
-            s = (s + 1) & cap_mask;
-        }
-        if (!placed) atomicOr(err, ST_TABLE_FULL);
-    }
-}
-
-template <int NW>
-__device__ __forceinline__ bool table_has(const Slot<NW>* __restrict__ table, uint64_t cap_mask, const Key<NW>& x) {
-    uint64_t h = key_hash<NW>(x);
-    uint32_t tag = slot_tag(h);
-    uint64_t s = h & cap_mask;
-    for (uint64_t probe = 0; probe <= cap_mask; probe++) {
-        uint32_t t = table[s].tag;
-        if (t == 0u) return false;
-        if (t == tag) {
-            bool eq = true;
-#pragma unroll
-            for (int w = 0; w < NW; w++) eq &= table[s].k[w] == x.w[w];
-            if (eq) return true;
-        }
-        s = (s + 1) & cap_mask;
-    }
-    return false;
 }
 
 // Probe every window; record windows without outdegree as (position, end).
@@ -491,16 +443,14 @@ __global__ void __launch_bounds__(256) mercy_probe_kernel(const uint32_t* __rest
 // dependent reads, and an error makes K1 windows in a row unsolid.  3 Gbp at
 // k = 31 3.9 ms with a lane a hit; 2.79, 2.55, 2.49 and 2.63 with 4, 8, 16 and
 // 32; one job's 450 k reads 0.48, and 0.17, 0.12, 0.09 and 0.08.
-// SOL 1 and 2: candidates out as mix_key images, solidity from the counting
-// spectrum (run length, doubled for a palindrome, >= d) through its bucket
-// index (1) or its super-k-mer bins (2); SOL 0 (unmixed handles): from the
-// hash set `solid`.
+// Candidates go out as mix_key images; solidity from the counting spectrum
+// (run length, doubled for a palindrome, >= d) in its super-k-mer bins (BINS)
+// or through its bucket index.
 constexpr int kWalkLanes = 16;
-template <int NW, int SOL, int G>
+template <int NW, bool BINS, int G>
 __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restrict__ packed,
                                                          const ulonglong2* __restrict__ hits, uint64_t n_hits, int k,
                                                          const Slot<NW>* __restrict__ ends, uint64_t ends_mask,
-                                                         const Slot<NW>* __restrict__ solid, uint64_t solid_mask,
                                                          const uint64_t* __restrict__ spec,
                                                          const uint32_t* __restrict__ spec_len,
                                                          const uint64_t* __restrict__ spec_off, int spec_bits,
@@ -522,12 +472,9 @@ __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restr
                 x = load_window<NW>(packed, mine, K1);
                 const Key<NW> r = key_rc<NW>(x, K1);
                 const Key<NW> c = key_less<NW>(r, x) ? r : x;
-                if constexpr (SOL != 0) {
-                    const uint32_t len = SOL == 2 ? super_find<NW>(super, spec, spec_len, x, r, mix_key<NW>(c), K1)
-                                                  : spec_find<NW>(spec, spec_len, spec_off, spec_bits, mix_key<NW>(c));
-                    present = (uint64_t)len * (key_eq<NW>(r, x) ? 2 : 1) >= (uint64_t)d;
-                } else
-                    present = table_has<NW>(solid, solid_mask, c);
+                const uint32_t len = BINS ? super_find<NW>(super, spec, spec_len, x, r, mix_key<NW>(c), K1)
+                                          : spec_find<NW>(spec, spec_len, spec_off, spec_bits, mix_key<NW>(c));
+                present = (uint64_t)len * (key_eq<NW>(r, x) ? 2 : 1) >= (uint64_t)d;
             }
             const uint32_t m = __ballot_sync(group, present);
             if (m) {
@@ -547,8 +494,7 @@ __global__ void __launch_bounds__(256) mercy_walk_kernel(const uint32_t* __restr
             Key<NW> z = load_window<NW>(packed, j, K1);
             Key<NW> rz = key_rc<NW>(z, K1);
             Key<NW> c = key_less<NW>(rz, z) ? rz : z;
-            if constexpr (SOL != 0) c = mix_key<NW>(c);
-            store_key<NW>(out, idx, c);
+            store_key<NW>(out, idx, mix_key<NW>(c));
         }
     }
 }
@@ -590,12 +536,9 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
         MH_LAUNCH(ctx, "mercy_ends_insert", (unsigned)ceil_div(S, (uint64_t)kEndsTile), 256, 0, ends_insert_kernel<NW>,
                   solid->keys, S, k + 1, flags.p, table.p, cap - 1, filter.p, fbits / 32 - 1, ctx->d_status);
     flags.reset();
-    // solidity: the counting handle's ascending mixed spectrum with a bucket
-    // index (4 to 8 keys a bucket); without one, a hash set of the canonical
-    // solid keys, load <= 1/2 (<= 0.61 if all palindromes)
-    const bool mixed = solid->spectrum_mixed;
-    Buf<Slot<NW>> sset;
-    uint64_t scap = 1;
+    // solidity: the counting handle's spectrum in its bins, or ascending with
+    // a bucket index (4 to 8 keys a bucket)
+    if (!solid->spectrum_mixed) fail(MH_EINVAL, "mercy: the spectrum's keys are not mixed");
     Buf<uint64_t> spec_off;
     int spec_bits = 1;
     const bool super = solid->super_idx != nullptr;
@@ -603,20 +546,13 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     if (super) {
         sx = SuperIndex{solid->super_off, solid->super_idx, solid->super_bins, solid->super_m, solid->super_main,
                         solid->n_spectrum};
-    } else if (mixed) {
+    } else {
         while (spec_bits < 40 && (2ull << spec_bits) * 4 <= solid->n_spectrum) spec_bits++;
         spec_off = Buf<uint64_t>(ctx, (1ull << spec_bits) + 1);
         spec_off.zero();
         if (solid->n_spectrum)
             MH_LAUNCH(ctx, "mercy_spectrum_index", grid_for(ctx, solid->n_spectrum, 256), 256, 0,
                       canon_index_kernel<NW>, solid->spectrum, solid->n_spectrum, spec_bits, spec_off.p);
-    } else {
-        scap = next_pow2(std::max<uint64_t>(S + S / 2, 64));
-        sset = Buf<Slot<NW>>(ctx, scap);
-        sset.zero();
-        if (S)
-            MH_LAUNCH(ctx, "mercy_solid_insert", grid_for(ctx, S, 256), 256, 0, solid_insert_kernel<NW>, solid->keys,
-                      S, k + 1, sset.p, scap - 1, ctx->d_status);
     }
     // windows without outdegree
     uint64_t hit_cap = std::max<uint64_t>(1u << 20, reads->n_packed / 256);
@@ -641,9 +577,7 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
     // candidates in the spectrum's order (mix_key images), so that their
     // sorted spectrum lookups ascend
     uint64_t out_cap = std::max<uint64_t>(1u << 20, 16 * n_hits);
-    const auto walk = super   ? mercy_walk_kernel<NW, 2, kWalkLanes>
-                      : mixed ? mercy_walk_kernel<NW, 1, kWalkLanes>
-                              : mercy_walk_kernel<NW, 0, kWalkLanes>;
+    const auto walk = super ? mercy_walk_kernel<NW, true, kWalkLanes> : mercy_walk_kernel<NW, false, kWalkLanes>;
     Buf<uint64_t> cand;
     uint64_t n_cand = 0;
     for (int attempt = 0; attempt < 2; attempt++) {
@@ -651,7 +585,7 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
         MH_CUDA(cudaMemsetAsync(stats.p + 1, 0, sizeof(uint64_t), ctx->stream));
         if (n_hits)
             MH_LAUNCH(ctx, "mercy_walk", grid_for(ctx, n_hits * kWalkLanes, 256, 8), 256, 0, walk, reads->packed,
-                      hits.p, n_hits, k, table.p, cap - 1, sset.p, scap - 1, solid->spectrum, solid->spectrum_len,
+                      hits.p, n_hits, k, table.p, cap - 1, solid->spectrum, solid->spectrum_len,
                       spec_off.p, spec_bits, sx, solid->d,
                       cand.p, out_cap, (unsigned long long*)(stats.p + 1));
         read_u64(ctx, stats.p + 1, &n_cand, 1);
@@ -659,18 +593,16 @@ void mercy_kmers(mh_ctx* ctx, const mh_reads* reads, const mh_kmers* solid, mh_k
         out_cap = n_cand;
     }
     hits.reset();
-    sset.reset();
     spec_off.reset();
     table.reset();
     Buf<uint64_t> alt(ctx, (n_cand ? n_cand : 1) * NW);
-    bool in_alt = mixed ? radix_sort_spread<NW>(ctx, cand.p, alt.p, n_cand)
-                        : radix_sort<NW>(ctx, cand.p, alt.p, nullptr, nullptr, n_cand, 0, 2 * (k + 1));
+    const bool in_alt = radix_sort_spread<NW>(ctx, cand.p, alt.p, n_cand);
     Buf<uint64_t>& sorted = in_alt ? alt : cand;
     Buf<uint64_t> mk;
     Buf<uint32_t> mc;
     uint64_t M = 0, runs = 0, palins = 0;
     expand_runs<NW>(ctx, sorted.p, n_cand, k, 1, mk, mc, &M, &runs, &palins, solid->spectrum, solid->spectrum_len,
-                    solid->n_spectrum, mixed, solid->spectrum_mixed, nullptr, super ? &sx : nullptr);
+                    solid->n_spectrum, true, true, nullptr, super ? &sx : nullptr);
     sync_and_check(ctx);
     out->k = k;
     out->nw = NW;
