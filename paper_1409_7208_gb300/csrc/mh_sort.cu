@@ -584,11 +584,13 @@ __device__ __forceinline__ bool same_above(const Key<NW>& a, const Key<NW>& b, i
 // Where more than `most` are listed the table is sorted by other means, so
 // CTAs that see that leave the rest as it is.  (With warps that went 64 rounds
 // into longer groups before listing them, and without an end to it, 1.77 ms for
-// 7.5 M pairs of a satellite at k = 61, now 0.11; 0.27 for 0.33 M pairs of 3 kbp, now 0.03.)
+// 7.5 M pairs of a satellite at k = 61, now 0.11; 0.27 for 0.33 M pairs of 3 kbp,
+// now 0.03.)
 template <int NW>
 __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                             uint64_t n, int lo, uint64_t* __restrict__ big,
-                                                            uint64_t big_cap, unsigned long long* __restrict__ n_big, uint64_t most) {
+                                                            uint64_t big_cap, unsigned long long* __restrict__ n_big,
+                                                            uint64_t most) {
     using F = Fix<NW>;
     __shared__ uint64_t K[F::kWin * NW];
     __shared__ uint32_t V[F::kWin];

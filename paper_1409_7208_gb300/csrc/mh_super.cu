@@ -27,7 +27,8 @@
 //            bins' order does not matter.
 //   rest     bins with more windows than one CTA should take, or whose keys
 //            do not fit the table, are expanded to keys and counted by the
-//            unit counting (mh_group.cu); their spectrum goes last
+//            unit counting (mh_group.cu); their spectrum goes last.  Where too
+//            much would go that way the whole set does (super_lost)
 //
 // What bounds it: the waits between a bin's barriers and instruction issue (a
 // hash insertion a window), not memory: a window moves about 2 bytes of

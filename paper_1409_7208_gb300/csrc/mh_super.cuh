@@ -9,7 +9,9 @@ namespace mh {
 // Minimizer length of windows of K1 symbols (0: too short for it).  The
 // kernel takes window minima from blocks of 8 positions, so a window has at
 // least 8 minimizer positions; within that, longer minimizers spread the
-// windows over more bins and shorter ones give longer super-k-mers.
+// windows over more bins and shorter ones give longer super-k-mers.  (Windows
+// of 16 to 20 symbols would have room for minimizers of 9 to 13; those were not
+// measured, and such sets are counted by units.)
 __host__ __device__ inline int super_m(int K1) { return K1 >= 32 ? 16 : K1 >= 26 ? 14 : K1 >= 21 ? 12 : 0; }
 
 // Windows of many words: a bin by one minimizer would get whole runs of about
