@@ -685,7 +685,9 @@ __global__ void __launch_bounds__(256) spread_fix_kv_kernel(uint64_t* __restrict
     }
     __syncthreads();
     // larger groups: a warp each, from K and V to keys and vals
-    const uint32_t nq = *(volatile unsigned long long*)n_big > most ? 0 : n_queue;
+    // (one lane's reading for the warp: others add to n_big meanwhile)
+    const bool listed = __shfl_sync(0xFFFFFFFFu, lane == 0 ? *(volatile unsigned long long*)n_big > most : 0, 0);
+    const uint32_t nq = listed ? 0 : n_queue;
     for (uint32_t q = warp; q < nq; q += 8) {
         const uint32_t g0 = queue[2 * q], g1 = queue[2 * q + 1];
         uint32_t pos = g0;
