@@ -853,9 +853,15 @@ template void expand_runs<4>(mh_ctx*, const uint64_t*, uint64_t, int, int, Buf<u
                              uint64_t*, uint64_t*, const uint64_t*, const uint32_t*, uint64_t, bool, bool,
                              RunList*, const SuperIndex*);
 
+// Memory a count may plan with: the HBM budget, or without one 85% of the
+// device's memory, less what the context holds.
+uint64_t count_memory(const mh_ctx* ctx) {
+    const uint64_t budget = ctx->budget ? ctx->budget : ctx->device_bytes / 20 * 17;
+    return budget > ctx->in_use ? budget - ctx->in_use : 0;
+}
+
 // Buckets of the mixed canonical keys to count one at a time (0 = all at
-// once).  Memory still free: the HBM budget, or without one 85% of the
-// device's memory, less what the context holds.  All at once if the count's
+// once).  All at once if the count's
 // working set (keys, sort buffer, run slots: about 24 nw + 12 bytes a
 // window) fits in 90% of it; otherwise enough buckets (up to 64) that one
 // bucket's working set and the byte a window of bucket numbers take at most
@@ -870,8 +876,7 @@ int count_bucket_bits(mh_ctx* ctx, uint64_t n, int nw) {
     if (ctx->bucket_bits >= 0) return ctx->bucket_bits;
     if (!n) return 0;
     const double per = 24.0 * nw + 12.0;
-    const uint64_t budget = ctx->budget ? ctx->budget : ctx->device_bytes / 20 * 17;
-    const double avail = budget > ctx->in_use ? (double)(budget - ctx->in_use) : 0.0;
+    const double avail = (double)count_memory(ctx);
     // in memory if the whole count fits in 90% of what is free; bucketed, the
     // buckets' outputs accumulate beside the next bucket's working set, and
     // one byte a window (its bucket) stays for the whole count

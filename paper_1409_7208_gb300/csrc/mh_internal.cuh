@@ -723,6 +723,9 @@ struct RunList {
 // 0 (all in memory) or bits of 2^bits buckets (mh_count.cu).
 int count_bucket_bits(mh_ctx* ctx, uint64_t n, int nw);
 
+// Memory a count may plan with (mh_count.cu).
+uint64_t count_memory(const mh_ctx* ctx);
+
 // How the unit counting splits n keys of nw words whose top `skip` bits
 // are equal: units of the next unit_bits bits of the top word (about
 // 160 / 96 / 56 keys each for 1 / 2 / 4 words), sorted into place by

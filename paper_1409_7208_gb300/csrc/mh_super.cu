@@ -935,10 +935,6 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     const uint64_t n_tiles = ceil_div(reads->n_packed, (uint64_t)kSplitTile);
     const uint32_t n_bins = (uint32_t)std::max<uint64_t>(1, n / C::kTarget);
     const uint64_t give_up = NW == 2 && super_switch() != 1 ? n : 0;
-    Buf<uint64_t> first(ctx, n_tiles), off(ctx, (uint64_t)n_bins + 1), totals(ctx, T_N);
-    Buf<unsigned long long> bins(ctx, n_bins);
-    MH_LAUNCH(ctx, "super_tiles", grid_for(ctx, n_tiles, 256), 256, 0, super_tiles_kernel, reads->frag_offs, F,
-              n_tiles, first.p);
     // records: 2 / (w + 1) a window for random sequences (about 8 / w by
     // halves), one more a fragment and a tile; each bin has slots for half as
     // many again as its share, and the list of those past them room for all:
@@ -948,6 +944,21 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     const uint64_t expect = std::min(n, (uint64_t)((double)n / run) + F + n_tiles + 1);
     const uint32_t slots = (uint32_t)((double)expect / n_bins * 1.5) + 16;
     uint64_t cap = expect + 4096;
+    const uint64_t per = d >= 2 ? 1 : 2;  // kept keys of both strands a window, at most
+    // large sets: a sixteenth of the bins first, to size the outputs by
+    const bool sample = n >= (1ull << 25) && n_bins >= 4096;
+    // short fragments make a record of every window or two, and those beside
+    // outputs with room for all windows need more than the units: a set that
+    // does not fit with them is theirs
+    const uint64_t out_bytes = (sample ? n / 8 : n) * (1 + per) * (8 * NW + 4);
+    const uint64_t bin_bytes = 8 * n_tiles + (uint64_t)n_bins * (8 * slots + 8 * C::kWords + 64);
+    const uint64_t avail = count_memory(ctx);
+    auto fits = [&] { return bin_bytes + std::max(24 * cap, 8 * cap + out_bytes) + (1u << 20) <= avail; };
+    if (!fits()) return false;
+    Buf<uint64_t> first(ctx, n_tiles), off(ctx, (uint64_t)n_bins + 1), totals(ctx, T_N);
+    Buf<unsigned long long> bins(ctx, n_bins);
+    MH_LAUNCH(ctx, "super_tiles", grid_for(ctx, n_tiles, 256), 256, 0, super_tiles_kernel, reads->frag_offs, F,
+              n_tiles, first.p);
     Buf<uint64_t> rec(ctx, (uint64_t)n_bins * slots);
     unsigned long long* tot = reinterpret_cast<unsigned long long*>(totals.p);
     Buf<uint64_t> more;
@@ -958,7 +969,6 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
     Buf<uint2> sidx(ctx, (uint64_t)n_bins * C::kWords);
     Buf<ulonglong2> deferred(ctx, n_bins);
     uint64_t spec_cap = 0, solid_cap = 0;
-    const uint64_t per = d >= 2 ? 1 : 2;  // kept keys of both strands a window, at most
     constexpr size_t smem = SuperSmem<NW>::kBytes;
     MH_CUDA(cudaFuncSetAttribute(super_count_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
@@ -979,8 +989,6 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         solid = Buf<uint64_t>(ctx, s * NW);
         solid_c = Buf<uint32_t>(ctx, s);
     };
-    // large sets: a sixteenth of the bins first, to size the outputs by
-    const bool sample = n >= (1ull << 25) && n_bins >= 4096;
     const uint32_t nb1 = sample ? n_bins / 16 : n_bins;
     bool all = false;
     for (int attempt = 0;; attempt++) {
@@ -1017,6 +1025,11 @@ bool super_count(mh_ctx* ctx, const mh_reads* reads, int k, int d, uint64_t n, m
         if (attempt >= 2) fail(MH_EDEVICE, "super-k-mer records overflow again");
         all = h[T_RECS] <= cap;
         cap = std::max(cap, h[T_RECS]);
+        spec.reset();
+        spec_len.reset();
+        solid.reset();
+        solid_c.reset();
+        if (!fits()) return false;
     }
     if (sample) {
         if (give_up && h[T_DEF] > kLostBins && super_lost(h[T_FULL], h[T_DONE])) return false;

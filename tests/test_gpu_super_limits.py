@@ -25,16 +25,17 @@ def _child(code, args, env):
 BUDGET = r"""
 import hashlib
 import synth, paper_1409_7208_gb300 as mh
-k = int(sys.argv[1])
+k, reads, length, d = (int(x) for x in sys.argv[1:])
 # little sequence: nearly every window is one of a few thousand
-a, o = synth.uniform_genome_reads(k, 2000, 60_000, 150, 0.0005)
-n = 60_000 * (150 - k)
+a, o = synth.uniform_genome_reads(k, 2000, reads, length, 0.0005)
+n = reads * (length - k)
 nw = 1 if k <= 31 else 2 if k <= 63 else 4
-# the least budget that counts in memory: 24 nw + 12 bytes a window within 90 % of it
-budget = int(n * 1.05 * (24 * nw + 12) / 0.9) + (1 << 20)
-reads = mh.mh_pack_reads(mh.Context(device=0), a, o)
+# the least budget that counts in memory: 24 nw + 12 bytes a window within 90 %
+# of what the offsets of the fragments' windows leave of it
+budget = int(n * 1.05 * (24 * nw + 12) / 0.9) + 8 * (reads + 1) + (1 << 20)
+packed = mh.mh_pack_reads(mh.Context(device=0), a, o)
 ctx = mh.Context(device=0, hbm_budget=budget, profile=True)
-s = mh.mh_count_kmers(ctx, reads, k, 2)
+s = mh.mh_count_kmers(ctx, packed, k, d)
 g, peak, prof = s.numpy(), ctx.memory()[1], ctx.profile()
 assert peak <= budget and "bucket_hist" not in prof
 print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), "super_expand" in prof)
@@ -43,9 +44,15 @@ print(hashlib.sha256(g["keys"].tobytes() + g["counts"].tobytes()).hexdigest(), "
 
 @pytest.mark.parametrize("k", [31, 47, 99])
 def test_all_bins_left_over_fit_the_in_memory_budget(k):
-    old = _child(BUDGET, [k], {"MH_SUPER": "0"})
-    new = _child(BUDGET, [k], {"MH_SUPER": "1", "MH_SUPER_HOT": "0"})
+    old = _child(BUDGET, [k, 60_000, 150, 2], {"MH_SUPER": "0"})
+    new = _child(BUDGET, [k, 60_000, 150, 2], {"MH_SUPER": "1", "MH_SUPER_HOT": "0"})
     assert new[0] == old[0] and (new[1], old[1]) == ("True", "False")
+
+
+@pytest.mark.parametrize("k,windows,d", [(31, 2, 1), (31, 1, 2), (31, 2, 2), (47, 2, 2), (99, 2, 2)])
+def test_a_record_a_window_or_two_fits_the_in_memory_budget(k, windows, d):
+    args = [k, 6_000_000 // windows, k + windows, d]
+    assert _child(BUDGET, args, {"MH_SUPER": "1"})[0] == _child(BUDGET, args, {"MH_SUPER": "0"})[0]
 
 
 SAMPLED = r"""
